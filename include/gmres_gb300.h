@@ -138,7 +138,9 @@ typedef enum {
 } gmres_ortho;
 
 typedef enum {
-  GMRES_DOT_FP64 = 0,  /* the basis multi-dot in FP64 FMAs */
+  GMRES_DOT_FP64 = 0,  /* the basis multi-dot to FP64 accuracy (in the fused step as exact
+                          integer sums of fixed-point operands, 57 bits below the largest
+                          entry of each block's rows; in FP64 FMAs elsewhere) */
   GMRES_DOT_DF32 = 1   /* the multi-dot V^T [w, v_j] of the one-reduction MGS step in
                           double-FP32 on the FP32 pipe: each FP64 operand split into two
                           floats (47 significant bits), products exact by FMA (Dekker's

@@ -12,12 +12,13 @@
 //      the update reads it there), u_j next to it.  Step 0's diagonal part runs before the
 //      programmatic-launch wait, overlapping the coarse-solve kernel that produces its s'.
 //   2. Multi-dot g = V^T w and the new row of L (u_j . u_c), streamed from HBM against the
-//      shared-memory slices (FP64: four warps per column; FP32: row chunks over column
-//      groups; double-FP32 on request).
+//      shared-memory slices, by row chunks over column groups (FP64: fixed point on the
+//      integer pipe, fixed.cuh; double-FP32 on request).
 //   3. Grid barrier 1; every block adds the G partial sums in the same order (identical
 //      totals in every block) and solves (I + L) h = g itself.
 //   4. Update of its rows, u_{j+1} = w - V (sigma o h), in the reverse order of step 2 (the
-//      columns read last are the likeliest to be in L2); partial sums of ||u_{j+1}||^2 and
+//      columns read last are the likeliest to be in L2; FP64 in fixed point); partial sums of
+//      ||u_{j+1}||^2 and
 //      of u_{j+1} over the block's pieces of aggregates (U^T u_{j+1}).
 //   5. Grid barrier 2; block 0 adds the norm partials and applies the rotations and the
 //      stopping tests; the other blocks form c = U^T u_{j+1} from the piece sums and share
@@ -36,6 +37,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "fixed.cuh"
 #include "internal.h"
 #include "kernels.cuh"
 
@@ -49,14 +51,13 @@ constexpr int kArnUnit = kPartUnit;              // rows per unit of the row par
 constexpr size_t kArnSmem = 220 * 1024;          // dynamic shared memory
 // reductions: lane-wise totals [2][kMaxK][33] (FP64) or warp sums [2][16][kMaxK] (FP32)
 constexpr size_t kArnScratch = 2 * kMaxK * 33 * sizeof(double);
-constexpr size_t kArnStaging = 2 * 2 * 16 * 32 * sizeof(double);  // FP64 multi-dot staging
+constexpr size_t kArnEbBytes = 32 * kMaxK * sizeof(int);  // FP64: column exponents
 constexpr long long kArnSpins = 1LL << 21;       // polls of the barrier word: about a second
 constexpr int kArnNormCol = 2 * kMaxK;           // column of ctl.part holding the norm partials
 constexpr int kArnAwRows64 = 6;  // rows per thread of an A W gather batch: FP64 (CSR rows)
 constexpr int kArnAwRows32 = 7;  // FP32 (row-indexed planes)
-// 16-byte basis loads in flight per lane in the multi-dot: FP32 (bound by HBM) asks for
-// more bytes in flight than FP64 (bound by its FMA pipe)
-template <typename TV> constexpr int arn_loads() { return sizeof(TV) == 8 ? 6 : 12; }
+constexpr int kArnFxGroup = 3;   // columns per pass of the fixed-point multi-dot
+constexpr int kArnEbTiles = 32;  // super-tiles with exponents of their own (the last is shared)
 
 template <typename TV, typename TACC>
 struct ArnArgs {
@@ -263,9 +264,7 @@ __device__ __forceinline__ double arn_ldcg_d(const double* p) { return __ldcg(p)
 __device__ __forceinline__ double arn_ldcg_d(const float* p) { return (double)__ldcg(p); }
 
 // ---- double-FP32 arithmetic for the FP64 multi-dot (GMRES_DOT_DF32) ---------------------
-// GB300 issues FP64 FMAs at 2 lanes per clock and multiprocessor, FP32 FMAs at 128: the
-// FP64 multi-dot is bound by its FMA pipe, not by HBM.  In the double-FP32 form each FP64
-// operand is split into two floats, x ~ hi + lo, with integer operations only (hi = x with
+// In the double-FP32 form of the multi-dot each FP64 operand is split into two floats, x ~ hi + lo, with integer operations only (hi = x with
 // its significand cut to 24 bits, lo = the remaining 29 bits rounded to 24: 47 significant
 // bits in all); a product takes the exact product of the high parts by an FMA (Dekker's
 // two-product), the two cross terms in FP32 (lo * lo, below 2^-46 of the product, is
@@ -347,6 +346,86 @@ __device__ __forceinline__ void arn_reduce_cols_df(const double* src, int nrows,
     if (c < ncols && q == 0) dst[c] = (double)hs + (double)hc;
   }
   __syncthreads();
+}
+
+// Multi-dot of an FP64 basis in fixed point (fixed.cuh): NSET dots per column, with w (Wf)
+// and u_j (Uf), both already converted (h, l limbs of two rows per int4).  Row order: warp w
+// takes the chunks w, w + 16, ... of 64 rows of the super-tile and, per pass, a group of G
+// columns at the same rows (one 16-byte load per column and lane); each value's register is
+// reloaded for the next chunk as soon as it is converted.  ebt[c] is the largest exponent of column c in
+// these rows.  At the end of a group the lanes' integer totals meet by warp reductions and
+// lane 0 stores them in slot[set][warp][c] (every slot is written once per super-tile).
+// Bound by the loads and the integer pipes together: per element 6 IMAD.WIDE and about 12
+// simple integer operations, where 2 FP64 multiply-adds hold their pipe for 64 issue slots each
+// (q1-n1024, GMRES(50), a step of the whole kernel: 228 us with FP64 multiply-adds in dots and
+// update, 162 us in fixed point; 4.2M rows, GMRES(40): 690 to 470 us; 3 columns a pass and 6
+// loads in flight in the update spill nothing, 4 and 8 were 2 to 3 % slower).
+template <int NSET, int G>
+__device__ __forceinline__ void arn_dots_fx(int4* slot, const double* V, long long ldv, int k,
+                                            long long s0, int nch, const int4* Wf,
+                                            const int4* Uf, const int* ebt, int warp, int lane) {
+  const int nqw = warp < nch ? (nch - 1 - warp) / kArnWarps + 1 : 0;  // chunks of this warp
+  if (nqw == 0) {
+    for (int q = lane; q < NSET * k; q += 32)
+      slot[(size_t)((q / k) * kArnWarps + warp) * kMaxK + q % k] = make_int4(0, 0, 0, 0);
+    return;
+  }
+  const double* const base = V + s0 + (size_t)warp * 64 + (size_t)lane * 2;
+  const double* pn = base;  // the next unit (a group's columns at one chunk) to load
+  int ln = 0, gn = 0;       // its chunk and first column
+  double b[G][2];
+#pragma unroll
+  for (int u = 0; u < G; ++u)
+    if (u < k) arn_ldg<double, double, 2>(pn + (size_t)u * ldv, b[u]);
+  for (int g0 = 0; g0 < k; g0 += G) {
+    const int gc = k - g0;
+    long long hh[NSET][G], cr[NSET][G];
+    int ll[NSET][G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+#pragma unroll
+      for (int s = 0; s < NSET; ++s) hh[s][u] = cr[s][u] = ll[s][u] = 0;
+    }
+    const int4* pw = Wf + (size_t)warp * 32 + lane;
+    const int4* pu = Uf + (size_t)warp * 32 + lane;
+#pragma unroll 1
+    for (int qi = 0; qi < nqw; ++qi) {
+      pn += kArnWarps * 64;
+      if (++ln == nqw) {  // on to the next group's first chunk
+        ln = 0;
+        gn += G;
+        pn = base + (size_t)gn * ldv;
+      }
+      const int4 w = *pw;
+      int4 uu = make_int4(0, 0, 0, 0);
+      if (NSET == 2) uu = *pu;
+      pw += kArnWarps * 32;
+      pu += kArnWarps * 32;
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        // (an absent column's stale values and exponent meet its accumulators only)
+        const int e = ebt[g0 + u] + 7;
+        const Fx v0 = fx_conv(b[u][0], e), v1 = fx_conv(b[u][1], e);
+        if (gn + u < k) arn_ldg<double, double, 2>(pn + (size_t)u * ldv, b[u]);
+        fx_fma(hh[0][u], cr[0][u], ll[0][u], v0, w.x, w.y);
+        fx_fma(hh[0][u], cr[0][u], ll[0][u], v1, w.z, w.w);
+        if (NSET == 2) {
+          fx_fma(hh[NSET - 1][u], cr[NSET - 1][u], ll[NSET - 1][u], v0, uu.x, uu.y);
+          fx_fma(hh[NSET - 1][u], cr[NSET - 1][u], ll[NSET - 1][u], v1, uu.z, uu.w);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+      if (u < gc)
+#pragma unroll
+        for (int s = 0; s < NSET; ++s) {
+          const FxSum t = fx_warp_sum(hh[s][u], cr[s][u], ll[s][u]);
+          if (lane == 0)
+            slot[(size_t)(s * kArnWarps + warp) * kMaxK + g0 + u] =
+                make_int4((int)t.s, (int)(t.s >> 32), (int)t.f, 0);
+        }
+  }
 }
 
 // Multi-dot of an FP64 basis in double-FP32 (row order): warp w takes the chunks w, w + 16,
@@ -536,105 +615,6 @@ __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long lo
   }
 }
 
-// Multi-dot of an FP64 basis: the 16 warps form 4 groups; group cg takes the columns
-// cg, cg + 4, ... one after the other, and its 4 warps stream each column together, warp ws
-// taking the chunks ws, ws + 4, ... (D chunks in flight per warp, the stream running on
-// across column boundaries).  Four warps on one column keep long contiguous runs of the
-// column in flight, which DRAM serves about twice as fast as one warp per column.  When a
-// column ends, the group's 4 lane-wise partial sums meet in shared memory (double-buffered
-// staging, one named barrier of the group) and warp ws = 0 adds them, in warp order, into
-// the lane-wise totals sbuf[set][c][lane]: one FP64 add per lane, warp and column.
-template <typename TV, typename TACC>
-__device__ __forceinline__ void arn_dots_group4(double* sbuf, double* stg, const TV* V,
-                                                long long ldv, int k, long long s0, int nch,
-                                                const TACC* Ws, const TACC* Us, int warp,
-                                                int lane) {
-  constexpr int VN = ArnVec<TV>::n;
-  constexpr int D = arn_loads<TV>();
-  const int cg = warp >> 2, ws = warp & 3;
-  const int ncg = cg < k ? (k - cg + 3) / 4 : 0;  // columns of this group
-  const int cpw = (nch - ws + 3) / 4;              // chunks of this warp per column
-  const int T = ncg * cpw;
-  if (ncg == 0) return;  // the same in the group's four warps
-  if (T == 0) {  // no chunk of this warp (nch < 4): zeros at the group's column ends
-    for (int i = 0; i < ncg; ++i) {
-      double* sb = stg + (size_t)(i & 1) * 2 * kArnWarps * 32;
-      sb[(0 * kArnWarps + warp) * 32 + lane] = 0.0;
-      sb[(1 * kArnWarps + warp) * 32 + lane] = 0.0;
-      asm volatile("bar.sync %0, 128;" ::"r"(1 + cg) : "memory");
-    }
-    return;
-  }
-  // load side: a pointer that steps 4 chunks down the column, then on to the group's next
-  // column (no division per load)
-  const size_t step = (size_t)4 * 32 * VN;
-  const long long jump = 4 * ldv - (long long)cpw * (long long)step;
-  const TV* pl = V + (size_t)cg * ldv + s0 + (size_t)ws * 32 * VN + lane * VN;
-  int lq = 0;
-  auto next_load = [&](TACC (&o)[VN]) {
-    arn_ldg<TV, TACC, VN>(pl, o);
-    pl += step;
-    if (++lq == cpw) {
-      lq = 0;
-      pl += jump;
-    }
-  };
-  TACC buf[D][VN];
-#pragma unroll
-  for (int d = 0; d < D; ++d)
-    if (d < T) next_load(buf[d]);
-  TACC a1[VN], a2[VN];  // one chain per vector element (FP64 latency hidden by ILP)
-#pragma unroll
-  for (int e = 0; e < VN; ++e) {
-    a1[e] = 0;
-    a2[e] = 0;
-  }
-  int i = 0, qi = 0;  // column of the group and chunk of the warp being consumed
-  const TACC* pw = Ws + (size_t)ws * 32 * VN + lane * VN;
-  const TACC* pu = Us + (size_t)ws * 32 * VN + lane * VN;
-  for (int t0 = 0; t0 < T; t0 += D) {
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const int t = t0 + d;
-      if (t < T) {
-        TACC wv[VN], uv[VN];
-        ld_acc<VN>(pw + (size_t)qi * step, wv);
-        ld_acc<VN>(pu + (size_t)qi * step, uv);
-#pragma unroll
-        for (int e = 0; e < VN; ++e) {
-          a1[e] += buf[d][e] * wv[e];
-          a2[e] += buf[d][e] * uv[e];
-        }
-        if (t + D < T) next_load(buf[d]);
-        if (++qi == cpw) {  // column cg + 4 i is done in this warp
-          double* sb = stg + (size_t)(i & 1) * 2 * kArnWarps * 32;
-          double s1 = 0.0, s2 = 0.0;
-#pragma unroll
-          for (int e = 0; e < VN; ++e) {
-            s1 += (double)a1[e];
-            s2 += (double)a2[e];
-            a1[e] = 0;
-            a2[e] = 0;
-          }
-          sb[(0 * kArnWarps + warp) * 32 + lane] = s1;
-          sb[(1 * kArnWarps + warp) * 32 + lane] = s2;
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + cg) : "memory");
-          if (ws == 0) {
-            const int c = cg + 4 * i;
-#pragma unroll
-            for (int set = 0; set < 2; ++set) {
-              const double* g = sb + (size_t)(set * kArnWarps + 4 * cg) * 32 + lane;
-              sbuf[((size_t)set * kMaxK + c) * 33 + lane] += ((g[0] + g[32]) + (g[64] + g[96]));
-            }
-          }
-          qi = 0;
-          ++i;
-        }
-      }
-    }
-  }
-}
-
 // Diagonal part of step j's SpMV for the rows [s0, s1) of a super-tile: (A v_j) into Ws and
 // u_j into Us (shared memory, from row s0; zeros past N)
 template <int ND, typename TV, typename TACC>
@@ -663,7 +643,7 @@ __device__ __forceinline__ void arn_diag(const ArnArgs<TV, TACC>& a, int j, long
 template <typename TV, typename TACC, int ND, bool DF>
 __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TACC sig, bool waited,
                                        bool first_diag_done, TACC* Ws, TACC* Us, TACC* Ss,
-                                       double* sbuf, double* stg) {
+                                       double* sbuf, int* sEb, int* semax, double* sred) {
   constexpr int VN = ArnVec<TV>::n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = threadIdx.x;
@@ -673,7 +653,8 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
   const long long N = a.N;
   const int k = j + 1;
   const bool multi = R1 - R0 > a.RS;  // w goes through global memory to the update
-  for (long long s0 = R0; s0 < R1; s0 += a.RS) {
+  int tile = 0;
+  for (long long s0 = R0; s0 < R1; s0 += a.RS, ++tile) {
     const long long s1 = s0 + a.RS < R1 ? s0 + a.RS : R1;
     // ---- 1. SpMV of the super-tile's rows: w and u_j into shared memory (the first
     // super-tile's may have been formed during the previous step's coarse solve) ---------
@@ -692,7 +673,9 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
       }
       if (a.defl && s0 == R0)
         for (int q = t; q < a.r; q += kArnThreads) Ss[q] = sig * __ldcg(a.sdefl + q);
+      if (t < 2) semax[t] = 0;
       __syncthreads();
+      int mw = 0, mu = 0;  // high words of the largest |w|, |u_j| of the super-tile
       constexpr int AWR = kArnAwRows64;
       for (long long i0 = s0 + t; i0 < s1; i0 += (long long)AWR * kArnThreads) {
         int e0[AWR], e1[AWR];
@@ -720,11 +703,19 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
               TACC aw = a.defl ? av[b] * Ss[ac[b]] : (TACC)0;
               for (int e = e0[b] + 1; e < e1[b]; ++e) aw += __ldg(a.auval + e) * Ss[__ldg(a.aucol + e)];
               wv = fma(sig, Ws[row - s0], aw);
+              a.w[row] = wv;  // the update reads w there
             }
             Ws[row - s0] = wv;
-            if ((multi || DF) && row < N) a.w[row] = wv;
+            mw = max(mw, fx_mag(wv));
+            mu = max(mu, fx_mag(Us[row - s0]));
           }
         }
+      }
+      mw = __reduce_max_sync(0xffffffffu, mw);
+      mu = __reduce_max_sync(0xffffffffu, mu);
+      if (lane == 0) {
+        atomicMax(&semax[0], mw);
+        atomicMax(&semax[1], mu);
       }
     } else {
       // FP32: a row's first two A W entries from the row-indexed planes (one level of loads,
@@ -763,7 +754,7 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
             }
             const TACC wv = row < N ? sig * (Ws[row - s0] + aw) : (TACC)0;
             Ws[row - s0] = wv;
-            if ((multi || DF) && row < N) a.w[row] = wv;
+            if (multi && row < N) a.w[row] = wv;
           }
         }
       };
@@ -783,24 +774,56 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
     }
     __syncthreads();
     const int nch = (int)((s1 - s0) / (32 * VN));
-    if constexpr (DF) {
-      // w and u_j split in place (float2 hi, lo in the 8 bytes of each double); the
-      // update reads w from global memory
-      for (long long q = t; q < s1 - s0; q += kArnThreads) {
-        float h1, l1, h2, l2;
-        arn_df_split((double)Ws[q], h1, l1);
-        arn_df_split((double)Us[q], h2, l2);
-        reinterpret_cast<float2*>(Ws)[q] = make_float2(h1, l1);
-        reinterpret_cast<float2*>(Us)[q] = make_float2(h2, l2);
+    if constexpr (sizeof(TV) == 8) {
+      // w and u_j to fixed point in place (relative to their largest exponents in the
+      // super-tile), then the dots with every column; the columns' exponents are kept per
+      // super-tile (the last slot is shared by all later ones, as their maximum)
+      const int ew = semax[0] >> 20, eu = semax[1] >> 20;
+      int* ebt = sEb + (tile < kArnEbTiles ? tile : kArnEbTiles - 1) * kMaxK;
+      if (t == 0) ebt[j] = tile < kArnEbTiles ? eu : max(ebt[j], eu);
+      if constexpr (DF) {
+        // w and u_j split in place (float2 hi, lo in the 8 bytes of each double)
+        for (int q = t; q < (int)(s1 - s0); q += kArnThreads) {
+          float h1, l1, h2, l2;
+          arn_df_split((double)Ws[q], h1, l1);
+          arn_df_split((double)Us[q], h2, l2);
+          reinterpret_cast<float2*>(Ws)[q] = make_float2(h1, l1);
+          reinterpret_cast<float2*>(Us)[q] = make_float2(h2, l2);
+        }
+        __syncthreads();
+        arn_dots_df(reinterpret_cast<float*>(sbuf), reinterpret_cast<const double*>(a.V), a.ldv,
+                    k, s0, nch, reinterpret_cast<const float2*>(Ws),
+                    reinterpret_cast<const float2*>(Us), warp, lane);
+        __syncthreads();
+        continue;
+      }
+      for (int q = t; q < (int)(s1 - s0); q += kArnThreads) {
+        const Fx fw = fx_conv((double)Ws[q], ew + 8);
+        const Fx fu = fx_conv((double)Us[q], eu + 8);
+        reinterpret_cast<int2*>(Ws)[q] = make_int2(fw.h, fw.l);
+        reinterpret_cast<int2*>(Us)[q] = make_int2(fu.h, fu.l);
       }
       __syncthreads();
-      arn_dots_df(reinterpret_cast<float*>(sbuf), reinterpret_cast<const double*>(a.V), a.ldv,
-                  k, s0, nch, reinterpret_cast<const float2*>(Ws),
-                  reinterpret_cast<const float2*>(Us), warp, lane);
-    } else if constexpr (sizeof(TV) == 8) {
-      // FP64 (its FMA pipe is the bound and its adds are dear): lane-wise partial sums
-      // per column, four warps per column
-      arn_dots_group4<TV, TACC>(sbuf, stg, a.V, a.ldv, k, s0, nch, Ws, Us, warp, lane);
+      int4* slot = reinterpret_cast<int4*>(sbuf);
+      arn_dots_fx<2, kArnFxGroup>(slot, reinterpret_cast<const double*>(a.V), a.ldv, k, s0, nch,
+                                  reinterpret_cast<const int4*>(Ws),
+                                  reinterpret_cast<const int4*>(Us), ebt, warp, lane);
+      __syncthreads();
+      // the block's column sums: the 16 warps' integer totals, then FP64 once per super-tile
+      for (int q = t; q < 2 * k; q += kArnThreads) {
+        const int set = q / k, c = q % k;
+        long long sum = 0;
+        unsigned long long f = 0;
+#pragma unroll 4
+        for (int w = 0; w < kArnWarps; ++w) {
+          const int4 v = slot[(size_t)(set * kArnWarps + w) * kMaxK + c];
+          sum += ((long long)v.y << 32) | (unsigned)v.x;
+          f += (unsigned)v.z;
+        }
+        sum += (long long)(f >> 32);
+        const double d = fx_value(sum, (unsigned)f, ebt[c], (set ? eu : ew) + 1);
+        sred[q] = tile == 0 ? d : sred[q] + d;
+      }
     } else {
         arn_dots_rows<TV, TACC, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, Ws, Us, warp, lane);
     }
@@ -808,9 +831,77 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
   }
 }
 
-// u_{j+1} = w - V (sigma o h) over the block's rows (also into ush, indexed from the block's
-// first row, when given); returns the warp's part of ||u_{j+1}||^2 (in every lane)
-template <typename TV, typename TACC, int ND, bool DF>
+// The same update of an FP64 basis in fixed point (fixed.cuh), super-tile by super-tile from the
+// last: the coefficients, each times its column's unit, become integers K_c relative to the
+// largest of them, a row's sum of M_c K_c (at most kMaxK terms) stays in integer
+// accumulators, and FP64 enters once per row, u = w - scale * sum.  Bound by the basis loads;
+// FP64 multiply-adds would cost 64 issue slots per entry, this form about 16.
+__device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, double* vout,
+                                                const double* w, int RS, long long R0,
+                                                long long R1, int k, const double* scoef,
+                                                const int* sEb, int4* sK, double* sscale,
+                                                double* ush) {
+  constexpr int U = 6;  // basis loads in flight per lane
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double nrm = 0.0;
+  const int tiles = (int)((R1 - R0 + RS - 1) / RS);
+  for (int tile = tiles - 1; tile >= 0; --tile) {
+    const long long s0 = R0 + (long long)tile * RS;
+    const long long s1 = s0 + RS < R1 ? s0 + RS : R1;
+    const int* ebt = sEb + (tile < kArnEbTiles ? tile : kArnEbTiles - 1) * kMaxK;
+    __syncthreads();
+    if (warp == 0) {
+      int m = 0;
+      bool bad = false;
+      for (int c = lane; c < k; c += 32) {
+        const int e = fx_mag(scoef[c]) >> 20;
+        bad |= e == 2047 || ebt[c] == 2047;
+        m = max(m, e + ebt[c]);
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      bad = __any_sync(0xffffffffu, bad);
+      for (int c = lane; c < k; c += 32) {
+        const int3 f = fx_coef(scoef[c], m, ebt[c]);
+        sK[c] = make_int4(f.x, f.y, f.z, ebt[c] + 3);
+      }
+      if (lane == 0)
+        *sscale = bad ? __longlong_as_double(0x7ff8000000000000ll) : -ldexp(1.0, m - 2098);
+    }
+    __syncthreads();
+    const double nscale = *sscale;
+    const int nch = (int)((s1 - s0) >> 6);
+    for (int q = nch - 1 - warp; q >= 0; q -= kArnWarps) {
+      const long long r = s0 + (long long)q * 64 + lane * 2;
+      const double2 wv = __ldcg(reinterpret_cast<const double2*>(w + r));
+      FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
+      for (int b = 0; b < k; b += U) {
+        double v[U][2];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (b + u < k) arn_ldg<double, double, 2>(V + (size_t)(b + u) * ldv + r, v[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (b + u < k) {
+            const int4 kc = sK[b + u];
+            fx_axpy(a0, fx_conv_near(v[u][0], kc.w), kc);
+            fx_axpy(a1, fx_conv_near(v[u][1], kc.w), kc);
+          }
+      }
+      // rows past N: w and the basis are zero there
+      double un[2];
+      un[0] = fx_axpy_sub(a0, wv.x, nscale);
+      un[1] = fx_axpy_sub(a1, wv.y, nscale);
+      *reinterpret_cast<double2*>(vout + r) = make_double2(un[0], un[1]);
+      if (ush) *reinterpret_cast<double2*>(ush + (r - R0)) = make_double2(un[0], un[1]);
+      nrm = fma(un[0], un[0], fma(un[1], un[1], nrm));
+    }
+  }
+  return warp_sum(nrm);
+}
+
+// u_{j+1} = w - V (sigma o h) over the block's rows of an FP32 basis (also into ush, indexed from
+// the block's first row, when given); returns the warp's part of ||u_{j+1}||^2 (in every lane)
+template <typename TV, typename TACC>
 __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, const TACC* Ws,
                                           const TACC* scoef, TACC* ush) {
   constexpr int VN = ArnVec<TV>::n;
@@ -820,13 +911,12 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
   const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
   const long long N = a.N;
   TV* __restrict__ vout = const_cast<TV*>(a.V) + (size_t)k * a.ldv;
-  double nrm = 0.0;       // FP64 basis
-  float ns = 0.f, nc = 0.f;  // FP32 basis: a double-FP32 pair (FP64 adds are dear)
+  float ns = 0.f, nc = 0.f;  // a double-FP32 pair (FP64 adds are dear)
   {
-    constexpr int U = sizeof(TV) == 4 ? 8 : (ND == 9 && !DF ? 13 : 10);  // basis loads in flight per lane
+    constexpr int U = 8;  // basis loads in flight per lane
     const int chunk = 32 * VN;
     const long long nch = (R1 - R0) / chunk;
-    const bool wsm = !DF && R1 - R0 <= a.RS;  // the block's w is still in shared memory
+    const bool wsm = R1 - R0 <= a.RS;  // the block's w is still in shared memory
     for (long long q = nch - 1 - warp; q >= 0; q -= kArnWarps) {
       const long long r = R0 + q * chunk + (long long)lane * VN;
       TACC wv[VN], p[VN];
@@ -859,21 +949,17 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
       TACC s = 0;
 #pragma unroll
       for (int e = 0; e < VN; ++e) s += un[e] * un[e];
-      if constexpr (sizeof(TACC) == 8) nrm += s;
-      else arn_df_add(ns, nc, s, 0.f);
+      arn_df_add(ns, nc, s, 0.f);
     }
   }
-  if constexpr (sizeof(TACC) == 8) {
-    return warp_sum(nrm);
-  } else {  // the warp's total in double-FP32, rounded once
+  // the warp's total in double-FP32, rounded once
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float a2 = __shfl_xor_sync(0xffffffffu, ns, o);
-      const float b2 = __shfl_xor_sync(0xffffffffu, nc, o);
-      arn_df_add(ns, nc, a2, b2);
-    }
-    return (double)ns + (double)nc;
+  for (int o = 16; o > 0; o >>= 1) {
+    const float a2 = __shfl_xor_sync(0xffffffffu, ns, o);
+    const float b2 = __shfl_xor_sync(0xffffffffu, nc, o);
+    arn_df_add(ns, nc, a2, b2);
   }
+  return (double)ns + (double)nc;
 }
 
 // Sums of u_{j+1} over this block's aggregate pieces (c of the next step's coarse solve, by
@@ -969,8 +1055,6 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     k_arnoldi(const __grid_constant__ ArnArgs<TV, TACC> a) {
   static_assert(std::is_same<TV, TACC>::value, "w and u_j slices share the basis element type");
   static_assert(!DF || sizeof(TV) == 8, "the double-FP32 multi-dot takes an FP64 basis");
-  constexpr int VN = ArnVec<TV>::n;
-  constexpr int B = sizeof(TACC) == 8 ? 2 : 4;  // SpMV rows per thread and batch
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double tot[2 * kMaxK + 1];
   __shared__ double sred[2 * kMaxK];
@@ -978,6 +1062,8 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   __shared__ TACC scoef[kMaxK];
   __shared__ double snrm[kArnWarps];
   __shared__ double ssig[kMaxK + 1];
+  __shared__ int semax[2];
+  __shared__ double sscale;
   // the control block is read from the grid-constant parameter (no register copy)
   Ctl& ctl = const_cast<Ctl&>(a.ctl);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -994,7 +1080,7 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   double* scratch = reinterpret_cast<double*>(
       smem + ((2 * (size_t)a.RS + (size_t)a.r) * sizeof(TACC) + 127) / 128 * 128);
   double* sL = scratch + kArnScratch / sizeof(double);
-  double* stg = sL + (size_t)kMaxK * kMaxK;
+  int* sEb = reinterpret_cast<int*>(sL + (size_t)kMaxK * kMaxK);  // FP64: [tile][column]
   double* sbuf = scratch;
   double* sc = reinterpret_cast<double*>(smem);  // c of the coarse solve (w, u_j are dead)
 
@@ -1091,8 +1177,11 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // partial sums of the multi-dot in shared memory, so that they persist across
     // super-tiles (FP64: lane-wise per column; FP32: per warp and column; double-FP32:
     // pairs per warp and column)
-    for (int q = t; q < 2 * kMaxK * 33; q += kArnThreads) sbuf[q] = 0.0;
-    arn_front<TV, TACC, ND, DF>(a, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, stg);
+    if constexpr (sizeof(TV) == 4 || DF)
+      for (int q = t; q < 2 * kMaxK * 33; q += kArnThreads) sbuf[q] = 0.0;
+    if (sizeof(TV) == 8 && t == 0)
+      sEb[(kArnEbTiles - 1) * kMaxK + j] = 0;  // a running maximum
+    arn_front<TV, TACC, ND, DF>(a, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sEb, semax, sred);
     waited = true;
     // per-block column sums (fixed order)
     if constexpr (DF) {  // the 16 warps' pairs of each column in warp order, then FP64 once
@@ -1106,18 +1195,7 @@ __global__ void __launch_bounds__(kArnThreads, 1)
         }
         sred[q] = (double)s + (double)cc;
       }
-    } else if constexpr (sizeof(TV) == 8) {  // the 32 lane-wise totals of each column, pairwise
-      for (int q0 = 0; q0 < 2 * k; q0 += kArnThreads / 2) {
-        const int q = q0 + (t >> 1), half = t & 1;
-        double v = 0.0;
-        if (q < 2 * k) {
-          const int set = q / k, c = q % k;
-          v = tree16(sbuf + ((size_t)set * kMaxK + c) * 33 + half * 16);
-        }
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        if (q < 2 * k && half == 0) sred[q] = v;
-      }
-    } else {  // the 16 warps' pairs of each column in warp order, kept as a pair
+    } else if constexpr (sizeof(TV) == 4) {  // the 16 warps' pairs in warp order, kept as a pair
       for (int q = t; q < 2 * k; q += kArnThreads) {
         const int set = q / k, c = q % k;
         const float2* ws = reinterpret_cast<const float2*>(sbuf);
@@ -1185,7 +1263,12 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // a shared-memory copy of u_{j+1} for the piece sums when the block's rows fit one
     // super-tile (u_j's slice is dead by now)
     TACC* ush = (a.defl && k < a.jmax && R1 - R0 <= a.RS) ? Us : nullptr;
-    double nrm = arn_update<TV, TACC, ND, DF>(a, k, Ws, scoef, ush);
+    double nrm;
+    if constexpr (sizeof(TV) == 8)
+      nrm = arn_update_fx(a.V, a.ldv, vout, a.w, a.RS, R0, R1, k, scoef, sEb,
+                          reinterpret_cast<int4*>(sbuf), &sscale, ush);
+    else
+      nrm = arn_update<TV, TACC>(a, k, Ws, scoef, ush);
     // ---- 5. norm partial; partial sums of u_{j+1} over this block's aggregate pieces ----
     {
       // the warp sums (formed by the update), then warp 0 adds the 16 of them (a block-wide
@@ -1332,7 +1415,7 @@ struct Arn {
   // rows of a super-tile: w and u_j slices, s' and the reduction scratch in kArnSmem
   static long long super_rows(int r) {
     const size_t fixed = ((size_t)r * sizeof(TACC) + 127) / 128 * 128 + kArnScratch +
-                         sizeof(double) * kMaxK * kMaxK + kArnStaging + 256;
+                         sizeof(double) * kMaxK * kMaxK + kArnEbBytes + 256;
     if (fixed >= kArnSmem) return 0;
     return (long long)((kArnSmem - fixed) / (2 * sizeof(TACC))) / kArnUnit * kArnUnit;
   }
