@@ -20,6 +20,7 @@
 // All floating-point reductions are formed in a fixed order (deterministic).
 #include <utility>
 
+#include "fixed.cuh"
 #include "internal.h"
 #include "kernels.cuh"
 
@@ -857,6 +858,39 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// The same from a basis in fixed point (fixed.cuh): integer sums, two rows per thread.  Bound by
+// the basis loads (FP64 multiply-adds: 111 us per cycle at 1M rows and 50 columns).
+template <bool DEFL>
+__global__ void __launch_bounds__(kThreads)
+    k_xupdate_fx(int N, const long long* __restrict__ V, long long ldv, double* __restrict__ x,
+                 double* __restrict__ t, Ctl ctl) {
+  if (ctl.flags[F_STOP]) return;
+  __shared__ int4 sK[kMaxK];
+  __shared__ double sscale;
+  const int k = ctl.flags[F_K];
+  if (threadIdx.x < 32) {
+    const double s = fx_coefs(k, ctl.coef, ctl.vexp, sK);
+    if (threadIdx.x == 0) sscale = s;
+  }
+  __syncthreads();
+  const double scale = sscale;
+  // (the columns are padded to whole 256-row tiles)
+  for (long long r = 2 * (blockIdx.x * (long long)blockDim.x + threadIdx.x); r < N;
+       r += 2ll * gridDim.x * blockDim.x) {
+    FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
+#pragma unroll 8
+    for (int c = 0; c < k; ++c) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(V + (size_t)c * ldv + r));
+      const int4 kc = sK[c];
+      fx_axpy(a0, fx_limbs(v.x, v.y), kc);
+      fx_axpy(a1, fx_limbs(v.z, v.w), kc);
+    }
+    double* out = DEFL ? t : x;
+    out[r] = fx_axpy_add(a0, DEFL ? 0.0 : x[r], scale);
+    if (r + 1 < N) out[r + 1] = fx_axpy_add(a1, DEFL ? 0.0 : x[r + 1], scale);
+  }
+}
+
 __global__ void __launch_bounds__(kThreads)
     k_xapply(int N, double* __restrict__ x, const double* __restrict__ t,
              const int* __restrict__ agg, Ctl ctl) {
@@ -1088,6 +1122,23 @@ struct Kern {
     }
   }
 
+  // t = V_k (sigma o y), or x += it
+  template <bool DEFL>
+  static void xupdate(const CycleArgs& a, double* x, cudaStream_t st) {
+    const int N = a.op.n;
+    const Grids& g = grids(a.sms);
+    if constexpr (sizeof(TV) == sizeof(double)) {
+      if (a.fixv) {
+        k_xupdate_fx<DEFL><<<grid_for((N + 2 * kThreads - 1) / (2 * kThreads), 1, 8 * a.sms),
+                             kThreads, 0, st>>>(N, static_cast<const long long*>(a.V), a.ldv, x,
+                                                a.t, a.ctl);
+        return;
+      }
+    }
+    k_xupdate<TV, DEFL><<<grid_for((N + kThreads - 1) / kThreads, 1, DEFL ? g.xupd_d : g.xupd_n),
+                          kThreads, 0, st>>>(N, static_cast<const TV*>(a.V), a.ldv, x, a.t, a.ctl);
+  }
+
   static cudaError_t phase(const CycleArgs& a, int ph, int j, bool defl, double* x,
                            const double* b, cudaStream_t st, int* launches) {
     const int N = a.op.n;
@@ -1228,14 +1279,12 @@ struct Kern {
           k_xapply_dense<<<grid_for(tiles, 1, g.xapply), kThreads, 0, st>>>(N, x, a.t, d, a.ctl);
           nl = 4;
         } else if (defl) {
-          k_xupdate<TV, true><<<grid_for(tiles, 1, g.xupd_d), kThreads, 0, st>>>(N, V, a.ldv, x,
-                                                                                a.t, a.ctl);
+          xupdate<true>(a, x, st);
           coarse(a, (const double*)a.t, nullptr, F_STOP, 0, st);
           k_xapply<<<grid_for(tiles, 1, g.xapply), kThreads, 0, st>>>(N, x, a.t, d.agg, a.ctl);
           nl = 5;
         } else {
-          k_xupdate<TV, false><<<grid_for(tiles, 1, g.xupd_n), kThreads, 0, st>>>(N, V, a.ldv,
-                                                                                 x, a.t, a.ctl);
+          xupdate<false>(a, x, st);
           nl = 2;
         }
         break;
@@ -1269,7 +1318,7 @@ struct Kern {
         k_ritz<<<1, 32, 0, st>>>(a.ctl);
         nl = 1;
         break;
-      case PH_ARNOLDI: {  // the steps of a cycle in one persistent kernel (fused.cu; j = steps)
+      case PH_ARNOLDI: {  // the steps of a cycle in one persistent kernel (fused.cuh; j = steps)
         const cudaError_t e = launch_arnoldi(a, j, defl, st);
         if (e != cudaSuccess) return e;
         nl = 1;

@@ -69,6 +69,7 @@ struct Ctl {
   double* sigma;  // ldh+1: basis scales, v_c = sigma_c * V[:, c]
   double* h;      // ldh+1: projection coefficients of the current column
   double* coef;   // ldh+1: coefficients of the pending basis update
+  int* vexp;      // ldh+1: largest biased exponent of each basis column (fixed-point basis)
   double* part;   // [max_grid][ldp] per-block partial sums
   double* part2;  // [kMaxGroups][ldp] per-group partial sums
   double* scal;   // S_NSCAL scalars

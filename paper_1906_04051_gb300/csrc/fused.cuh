@@ -1,8 +1,10 @@
-// fused.cu -- the Arnoldi steps of a restart cycle of deflated GMRES(m) in one persistent
-// kernel: per step the SpMV w = A M^-1 v_j (Eq. 10 with Eqs. 16-17), the paper's modified
-// Gram-Schmidt projections (Eq. 13) in their one-reduction form, ||w||, the plane rotations
-// with the stopping tests (Eqs. 12, 14) and the coarse solve of the next step's
-// preconditioner (Eq. 17: s' = U (|mu| T^-1 - I) U^T v_{j+1}).
+// fused.cuh -- the Arnoldi steps of a restart cycle of deflated GMRES(m) in one persistent
+// kernel: per step the SpMV w = A M^-1 v_j (Eq. 10 with Eqs. 16-17), the orthogonalisation
+// (Eq. 13), ||w||, the plane rotations with the stopping tests (Eqs. 12, 14) and the coarse
+// solve of the next step's preconditioner (Eq. 17: s' = U (|mu| T^-1 - I) U^T v_{j+1}).  The
+// orthogonalisation is the paper's modified Gram-Schmidt projections in their one-reduction
+// form or CGS2; the operator is in diagonal storage or CSR; the basis is FP64, FP32 or (CGS2)
+// BF16.  Each precision is instantiated in a file of its own (fused_*.cu).
 //
 // One block of 16 warps per multiprocessor, launched cooperatively (every block resident).
 // Block b owns a contiguous range of rows (a multiple of 128) for the whole cycle, taken in
@@ -26,6 +28,9 @@
 //   6. A split barrier: each block arrives once its share of step 5 is published, forms the
 //      diagonal part of the next step's SpMV (it needs only u_{j+1}), then waits for all
 //      arrivals and reads the same stopping decision and sigma_{j+1}.
+// CGS2 forms only g = V^T w in step 2, takes h = g in step 3 and inserts between 3 and 4 the
+// first update w -= V h with the second multi-dot h' = V^T w (a pass over each super-tile's
+// rows, w' in shared memory in between), one more grid barrier, and coefficients h + h'.
 // Every reduction is formed in a fixed order: runs are bitwise reproducible.  The per-phase
 // register budgets (loads in flight) are set so that the kernel needs no local memory:
 // with 220 KB of shared memory per block, spilled registers would live in L2.
@@ -33,6 +38,8 @@
 // The basis is streamed with plain vectorised loads rather than bulk asynchronous copies:
 // measured on GB300, a multiprocessor fed by bulk copies reached about 10 bytes per clock,
 // against the 22 that the HBM copy bandwidth asks of each of the 152.
+#pragma once
+
 #include <algorithm>
 #include <type_traits>
 #include <utility>
@@ -51,13 +58,22 @@ constexpr int kArnUnit = kPartUnit;              // rows per unit of the row par
 constexpr size_t kArnSmem = 220 * 1024;          // dynamic shared memory
 // reductions: lane-wise totals [2][kMaxK][33] (FP64) or warp sums [2][16][kMaxK] (FP32)
 constexpr size_t kArnScratch = 2 * kMaxK * 33 * sizeof(double);
-constexpr size_t kArnEbBytes = 32 * kMaxK * sizeof(int);  // FP64: column exponents
 constexpr long long kArnSpins = 1LL << 21;       // polls of the barrier word: about a second
 constexpr int kArnNormCol = 2 * kMaxK;           // column of ctl.part holding the norm partials
+constexpr int kArnMaxCol = kArnNormCol + 1;      // and the blocks' largest |u_{j+1}| (high words)
 constexpr int kArnAwRows64 = 6;  // rows per thread of an A W gather batch: FP64 (CSR rows)
 constexpr int kArnAwRows32 = 7;  // FP32 (row-indexed planes)
-constexpr int kArnFxGroup = 3;   // columns per pass of the fixed-point multi-dot
-constexpr int kArnEbTiles = 32;  // super-tiles with exponents of their own (the last is shared)
+// columns per pass of the fixed-point multi-dot with two dots and with one, passes in flight
+// (q1-n1024, create + 300 steps: 58.7 ms; 4 and 6 columns, one pass: 60.6; 2 columns, 3 passes:
+// 60.9; reads alone run at 4.7, 5.6 and 5.8 TB/s with 4, 6 and 8 16-byte loads per lane)
+constexpr int kArnFxGroup = 3;
+constexpr int kArnFxGroup1 = 4;
+constexpr int kArnFxDepth = 2;
+
+// orthogonalisation of an instantiation, and its operator (ND): 9 diagonals unrolled, a run-time
+// number of diagonals, CSR
+enum { kArnLowsync = 0, kArnLowsyncDf = 1, kArnCgs2 = 2 };
+constexpr int kArnCsr = -1;
 
 template <typename TV, typename TACC>
 struct ArnArgs {
@@ -74,6 +90,10 @@ struct ArnArgs {
   TACC* w;        // working vector
   DiaOffsets dia;
   const TACC* dval;
+  const int* rowptr;  // CSR (no diagonal storage)
+  const int* col;
+  const TACC* val;
+  int vec;            // CSR: long rows, 4 lanes each
   const int* aurp;
   const int* aucol;
   const TACC* auval;
@@ -95,8 +115,9 @@ struct ArnArgs {
   unsigned* gbar;  // [0] arrivals, [1] generation
 };
 
-// rows VN elements at a time (16-byte loads of the basis type)
-template <typename TV> struct ArnVec { static constexpr int n = Vec<TV>::n; };
+// rows VN elements at a time (16-byte loads of the basis type, 8-byte for BF16: a warp's chunk is
+// then at most kArnUnit rows)
+template <typename TV> struct ArnVec { static constexpr int n = sizeof(TV) == 8 ? 2 : 4; };
 
 // Grid barrier (cooperative launch: every block resident).  Thread 0 arrives on bar[0];
 // the last arrival resets it and advances the generation bar[1]; the others poll the
@@ -211,14 +232,15 @@ __device__ __forceinline__ void arn_ldg(const TV* p, TACC (&o)[VN]) {
                  : "l"(p));
     o[0] = x; o[1] = y; o[2] = z; o[3] = w;
   } else {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 f = __bfloat1622float2(h[e]);
-      o[2 * e] = f.x;
-      o[2 * e + 1] = f.y;
-    }
+    unsigned x, y;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.b32 {%0, %1}, [%2];"
+                 : "=r"(x), "=r"(y)
+                 : "l"(p));
+    // a BF16 value is the upper half of its FP32 form
+    o[0] = __uint_as_float(x << 16);
+    o[1] = __uint_as_float(x & 0xffff0000u);
+    o[2] = __uint_as_float(y << 16);
+    o[3] = __uint_as_float(y & 0xffff0000u);
   }
 }
 
@@ -242,11 +264,11 @@ __device__ __forceinline__ void arn_stv(TV* p, const TACC (&v)[VN]) {
   } else if constexpr (std::is_same<TV, float>::value) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   } else {
-    uint4 o;
+    uint2 o;
     __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) h[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-    *reinterpret_cast<uint4*>(p) = o;
+    for (int e = 0; e < 2; ++e) h[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+    *reinterpret_cast<uint2*>(p) = o;
   }
 }
 
@@ -262,6 +284,9 @@ __device__ __forceinline__ void arn_timeout(Ctl& ctl) {
 // a basis entry written earlier in this launch, read through L2 as FP64
 __device__ __forceinline__ double arn_ldcg_d(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ double arn_ldcg_d(const float* p) { return (double)__ldcg(p); }
+__device__ __forceinline__ double arn_ldcg_d(const __nv_bfloat16* p) {
+  return (double)__bfloat162float(__ldcg(p));
+}
 
 // ---- double-FP32 arithmetic for the FP64 multi-dot (GMRES_DOT_DF32) ---------------------
 // In the double-FP32 form of the multi-dot each FP64 operand is split into two floats, x ~ hi + lo, with integer operations only (hi = x with
@@ -348,83 +373,126 @@ __device__ __forceinline__ void arn_reduce_cols_df(const double* src, int nrows,
   __syncthreads();
 }
 
+// How the 16 warps share nch 64-row chunks: from 16 chunks on a warp takes the chunks warp, warp +
+// 16, ... with all columns; with fewer, S = 16 / nch warps share a chunk's columns (integer sums:
+// the result does not depend on the split).
+struct ArnSplit {
+  int S, q0, p, rows;  // warps per chunk, the warp's first chunk, its share, chunks taken at once
+  bool live;
+};
+__device__ __forceinline__ ArnSplit arn_split(int nch) {
+  const int warp = threadIdx.x >> 5;
+  if (nch >= kArnWarps) return ArnSplit{1, warp, 0, kArnWarps, true};
+  const int S = kArnWarps / nch;
+  return ArnSplit{S, warp % nch, warp / nch, nch, warp / nch < S};
+}
+
+// Two rows of a basis column held as fixed-point integers, past L1 (a column is converted in
+// place within the launch, after its FP64 form was read through L1)
+__device__ __forceinline__ void arn_ldfx(const long long* p, uint4& o) {
+  asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w)
+               : "l"(p));
+}
+
 // Multi-dot of an FP64 basis in fixed point (fixed.cuh): NSET dots per column, with w (Wf)
-// and u_j (Uf), both already converted (h, l limbs of two rows per int4).  Row order: warp w
-// takes the chunks w, w + 16, ... of 64 rows of the super-tile and, per pass, a group of G
-// columns at the same rows (one 16-byte load per column and lane); each value's register is
-// reloaded for the next chunk as soon as it is converted.  ebt[c] is the largest exponent of column c in
-// these rows.  At the end of a group the lanes' integer totals meet by warp reductions and
-// lane 0 stores them in slot[set][warp][c] (every slot is written once per super-tile).
-// Bound by the loads and the integer pipes together: per element 6 IMAD.WIDE and about 12
-// simple integer operations, where 2 FP64 multiply-adds hold their pipe for 64 issue slots each
-// (q1-n1024, GMRES(50), a step of the whole kernel: 228 us with FP64 multiply-adds in dots and
-// update, 162 us in fixed point; 4.2M rows, GMRES(40): 690 to 470 us; 3 columns a pass and 6
-// loads in flight in the update spill nothing, 4 and 8 were 2 to 3 % slower).
-template <int NSET, int G>
-__device__ __forceinline__ void arn_dots_fx(int4* slot, const double* V, long long ldv, int k,
-                                            long long s0, int nch, const int4* Wf,
-                                            const int4* Uf, const int* ebt, int warp, int lane) {
-  const int nqw = warp < nch ? (nch - 1 - warp) / kArnWarps + 1 : 0;  // chunks of this warp
-  if (nqw == 0) {
-    for (int q = lane; q < NSET * k; q += 32)
-      slot[(size_t)((q / k) * kArnWarps + warp) * kMaxK + q % k] = make_int4(0, 0, 0, 0);
-    return;
-  }
-  const double* const base = V + s0 + (size_t)warp * 64 + (size_t)lane * 2;
-  const double* pn = base;  // the next unit (a group's columns at one chunk) to load
-  int ln = 0, gn = 0;       // its chunk and first column
-  double b[G][2];
+// and u_j (Uf), both already operands (limbs of two rows per int4).  The first kf columns are
+// fixed-point integers, a last column kf (k = kf + 1), not converted yet, FP64 (largest exponent
+// ej; its dot with w only).  Row order: per pass a warp takes a group of G columns at the same
+// 64 rows (one 16-byte load per column and lane), D such units in flight; each value's register
+// is reloaded for a later unit as soon as it is used.  At the end of a group the lanes' integer totals meet by warp
+// reductions and lane 0 stores them in slot[set][first chunk][c] (once per super-tile).
+// Bound by the loads; per element 6 IMAD.WIDE and a few simple integer operations, where 2 FP64
+// multiply-adds hold their pipe for 64 issue slots each (q1-n1024, GMRES(50), a step of the whole
+// kernel: 228 us with FP64 multiply-adds in dots and update, 151 us in fixed point; 4.2M rows,
+// GMRES(40): 690 to 450 us).
+template <int NSET, int G, int D>
+__device__ __forceinline__ void arn_dots_fx(int4* slot, const double* V, long long ldv, int kf,
+                                            int k, int ej, long long s0, int nch, const int4* Wf,
+                                            const int4* Uf, int lane) {
+  const ArnSplit sp = arn_split(nch);
+  if (!sp.live) return;
+  const int nqw = (nch - 1 - sp.q0) / kArnWarps + 1;  // chunks of this warp
+  const long long at = s0 + (long long)sp.q0 * 64 + lane * 2;
+  const long long* const base = reinterpret_cast<const long long*>(V) + at;
+  // a unit: a group's columns at one chunk.  D units are in flight (b), reloaded as they are used
+  int ln = 0, gn = sp.p * G;  // chunk and first column of the next unit to load
+  const long long* pn = base + (size_t)gn * ldv;
+  auto advance = [&] {
+    pn += kArnWarps * 64;
+    if (++ln == nqw) {  // on to the next group's first chunk
+      ln = 0;
+      gn += G * sp.S;
+      pn = base + (size_t)gn * ldv;
+    }
+  };
+  uint4 b[D][G];
 #pragma unroll
-  for (int u = 0; u < G; ++u)
-    if (u < k) arn_ldg<double, double, 2>(pn + (size_t)u * ldv, b[u]);
-  for (int g0 = 0; g0 < k; g0 += G) {
-    const int gc = k - g0;
-    long long hh[NSET][G], cr[NSET][G];
-    int ll[NSET][G];
+  for (int d = 0; d < D; ++d) {
 #pragma unroll
     for (int u = 0; u < G; ++u) {
-#pragma unroll
-      for (int s = 0; s < NSET; ++s) hh[s][u] = cr[s][u] = ll[s][u] = 0;
+      b[d][u] = make_uint4(0, 0, 0, 0);
+      if (gn + u < kf) arn_ldfx(pn + (size_t)u * ldv, b[d][u]);
     }
-    const int4* pw = Wf + (size_t)warp * 32 + lane;
-    const int4* pu = Uf + (size_t)warp * 32 + lane;
+    advance();
+  }
+  auto store = [&](int set, int c, const FxDot& a) {
+    const FxSum t = fx_warp_sum(a);
+    if (lane == 0)
+      slot[(size_t)(set * kArnWarps + sp.q0) * kMaxK + c] =
+          make_int4((int)t.s, (int)(t.s >> 32), (int)t.f, (int)(t.f >> 32));
+  };
+  FxDot acc[NSET][G];
+#pragma unroll
+  for (int u = 0; u < G; ++u)
+#pragma unroll
+    for (int s = 0; s < NSET; ++s) acc[s][u] = FxDot{0, 0, 0, 0};
+  int g0 = sp.p * G, qi = 0;  // first column and chunk of the unit in use
+  const int at0 = sp.q0 * 32 + lane;
 #pragma unroll 1
-    for (int qi = 0; qi < nqw; ++qi) {
-      pn += kArnWarps * 64;
-      if (++ln == nqw) {  // on to the next group's first chunk
-        ln = 0;
-        gn += G;
-        pn = base + (size_t)gn * ldv;
-      }
-      const int4 w = *pw;
-      int4 uu = make_int4(0, 0, 0, 0);
-      if (NSET == 2) uu = *pu;
-      pw += kArnWarps * 32;
-      pu += kArnWarps * 32;
+  while (g0 < kf) {
 #pragma unroll
-      for (int u = 0; u < G; ++u) {
-        // (an absent column's stale values and exponent meet its accumulators only)
-        const int e = ebt[g0 + u] + 7;
-        const Fx v0 = fx_conv(b[u][0], e), v1 = fx_conv(b[u][1], e);
-        if (gn + u < k) arn_ldg<double, double, 2>(pn + (size_t)u * ldv, b[u]);
-        fx_fma(hh[0][u], cr[0][u], ll[0][u], v0, w.x, w.y);
-        fx_fma(hh[0][u], cr[0][u], ll[0][u], v1, w.z, w.w);
+    for (int d = 0; d < D; ++d) {
+      if (D > 1 && g0 >= kf) break;
+      const int4 w = Wf[at0 + qi * (kArnWarps * 32)];
+      int4 uu = make_int4(0, 0, 0, 0);
+      if (NSET == 2) uu = Uf[at0 + qi * (kArnWarps * 32)];
+#pragma unroll
+      for (int u = 0; u < G; ++u) {  // (an absent column's stale values meet its sums only)
+        const Fx v0 = fx_limbs(b[d][u].x, b[d][u].y), v1 = fx_limbs(b[d][u].z, b[d][u].w);
+        if (gn + u < kf) arn_ldfx(pn + (size_t)u * ldv, b[d][u]);
+        fx_dot(acc[0][u], v0, make_int2(w.x, w.y));
+        fx_dot(acc[0][u], v1, make_int2(w.z, w.w));
         if (NSET == 2) {
-          fx_fma(hh[NSET - 1][u], cr[NSET - 1][u], ll[NSET - 1][u], v0, uu.x, uu.y);
-          fx_fma(hh[NSET - 1][u], cr[NSET - 1][u], ll[NSET - 1][u], v1, uu.z, uu.w);
+          fx_dot(acc[NSET - 1][u], v0, make_int2(uu.x, uu.y));
+          fx_dot(acc[NSET - 1][u], v1, make_int2(uu.z, uu.w));
         }
+      }
+      advance();
+      if (++qi == nqw) {  // the group's last chunk in this warp
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+#pragma unroll
+          for (int s = 0; s < NSET; ++s) {
+            if (g0 + u < kf) store(s, g0 + u, acc[s][u]);
+            acc[s][u] = FxDot{0, 0, 0, 0};
+          }
+        qi = 0;
+        g0 += G * sp.S;
       }
     }
-#pragma unroll
-    for (int u = 0; u < G; ++u)
-      if (u < gc)
-#pragma unroll
-        for (int s = 0; s < NSET; ++s) {
-          const FxSum t = fx_warp_sum(hh[s][u], cr[s][u], ll[s][u]);
-          if (lane == 0)
-            slot[(size_t)(s * kArnWarps + warp) * kMaxK + g0 + u] =
-                make_int4((int)t.s, (int)(t.s >> 32), (int)t.f, 0);
-        }
+  }
+  if (kf < k && sp.p == sp.S - 1) {  // the FP64 column
+    FxDot a{0, 0, 0, 0};
+    for (int qi = 0; qi < nqw; ++qi) {
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(V + (size_t)kf * ldv + at +
+                                                                (long long)qi * (kArnWarps * 64)));
+      const int4 w = Wf[(size_t)(sp.q0 + qi * kArnWarps) * 32 + lane];
+      fx_dot(a, fx_limbs(fx_basis(v.x, ej)), make_int2(w.x, w.y));
+      fx_dot(a, fx_limbs(fx_basis(v.y, ej)), make_int2(w.z, w.w));
+    }
+    store(0, kf, a);
+    if (NSET == 2) store(1, kf, FxDot{0, 0, 0, 0});
   }
 }
 
@@ -544,7 +612,7 @@ __device__ __forceinline__ void arn_dia_rows(TACC (&acc)[B], long long row0, lon
 // of the general banded instantiation, which takes 5.)
 template <int ND> constexpr int arn_group() { return ND == 9 ? 6 : 5; }
 
-template <typename TV, typename TACC, int G>
+template <typename TV, typename TACC, int NSET, int G>
 __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long long ldv, int k,
                                               long long s0, int nch, const TACC* Ws,
                                               const TACC* Us, int warp, int lane) {
@@ -576,28 +644,34 @@ __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long lo
     const size_t off = (size_t)(warp + qi * kArnWarps) * 32 * VN;
     TACC wv[VN], uv[VN];
     ld_acc<VN>(Ws + off + lane * VN, wv);
-    ld_acc<VN>(Us + off + lane * VN, uv);
+    if (NSET == 2) ld_acc<VN>(Us + off + lane * VN, uv);
 #pragma unroll
     for (int u = 0; u < G; ++u)
       if (u < gc)
 #pragma unroll
         for (int e = 0; e < VN; ++e) {
           a1[u] += b[u][e] * wv[e];
-          a2[u] += b[u][e] * uv[e];
+          if (NSET == 2) a2[u] += b[u][e] * uv[e];
         }
     if (qi == nqw - 1) {  // the group's last chunk in this warp
 #pragma unroll
       for (int u = 0; u < G; ++u) {
         if (u < gc) {
-          const TACC t1 = warp_sum(a1[u]), t2 = warp_sum(a2[u]);
+          const TACC t1 = warp_sum(a1[u]);
           if (lane == 0) {
             float2* p1 = reinterpret_cast<float2*>(wsum) + (size_t)warp * kMaxK + g0 + u;
-            float2* p2 = reinterpret_cast<float2*>(wsum) + (size_t)(kArnWarps + warp) * kMaxK + g0 + u;
-            float2 a1v = *p1, a2v = *p2;
+            float2 a1v = *p1;
             arn_df_add(a1v.x, a1v.y, (float)t1, 0.f);
-            arn_df_add(a2v.x, a2v.y, (float)t2, 0.f);
             *p1 = a1v;
-            *p2 = a2v;
+          }
+          if (NSET == 2) {
+            const TACC t2 = warp_sum(a2[u]);
+            if (lane == 0) {
+              float2* p2 = reinterpret_cast<float2*>(wsum) + (size_t)(kArnWarps + warp) * kMaxK + g0 + u;
+              float2 a2v = *p2;
+              arn_df_add(a2v.x, a2v.y, (float)t2, 0.f);
+              *p2 = a2v;
+            }
           }
         }
         a1[u] = 0;
@@ -615,21 +689,104 @@ __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long lo
   }
 }
 
+// The same rows of a CSR operator: a thread per row (ten entries' loads, then their gathers, in
+// flight at once), or 8 lanes per row for long rows (two rows of up to 64 entries in flight per
+// lane group; 4 lanes: 24.8 against 22.2 ms on the 274,625-unknown Bratu matrix, 100 steps).  With one block of 16 warps per multiprocessor the loads in flight per thread
+// stand in for the occupancy of a kernel of its own.
+template <typename TV, typename TACC>
+__device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj, long long s0,
+                                        long long s1, TACC* Ws, TACC* Us, int tid, int nthr) {
+  const long long N = a.N;
+  if (!a.vec) {
+    constexpr int U = 10;
+    for (long long row = s0 + tid; row < s1; row += nthr) {
+      TACC acc = 0, x = 0;
+      if (row < N) {
+        const int rs = __ldg(a.rowptr + row), re = __ldg(a.rowptr + row + 1);
+        x = ld_as<TACC, TV>(xj + row);
+        for (int q = rs; q < re; q += U) {
+          int c[U];
+          TACC v[U], xv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            c[u] = q + u < re ? __ldg(a.col + q + u) : 0;
+            v[u] = q + u < re ? __ldg(a.val + q + u) : (TACC)0;
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) xv[u] = q + u < re ? ld_as<TACC, TV>(xj + c[u]) : (TACC)0;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (q + u < re) acc += v[u] * xv[u];
+        }
+      }
+      Ws[row - s0] = acc;
+      Us[row - s0] = x;
+    }
+    return;
+  }
+  constexpr int L = 8, U = 8;  // lanes per row, entries per lane and trip
+  const int sub = tid & (L - 1);
+  // (a warp's lane groups take 8 consecutive rows: the loop is uniform in a warp)
+  for (long long r0 = s0 + 2 * (tid / L); r0 < s1; r0 += 2 * (nthr / L)) {
+    TACC acc[2] = {0, 0};
+    int q[2], re[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      q[h] = r0 + h < N ? __ldg(a.rowptr + r0 + h) + sub : 0;
+      re[h] = r0 + h < N ? __ldg(a.rowptr + r0 + h + 1) : 0;
+    }
+    while (q[0] < re[0] || q[1] < re[1]) {
+      int c[2][U];
+      TACC v[2][U];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = q[h] + L * u;
+          c[h][u] = e < re[h] ? __ldg(a.col + e) : -1;
+          v[h][u] = e < re[h] ? __ldg(a.val + e) : (TACC)0;
+        }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        TACC xv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) xv[u] = c[h][u] >= 0 ? ld_as<TACC, TV>(xj + c[h][u]) : (TACC)0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (c[h][u] >= 0) acc[h] += v[h][u] * xv[u];
+        q[h] += L * U;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int o = L / 2; o > 0; o >>= 1) acc[h] += __shfl_xor_sync(0xffffffffu, acc[h], o);
+    if (sub < 2) {
+      Ws[r0 + sub - s0] = sub ? acc[1] : acc[0];
+      Us[r0 + sub - s0] = r0 + sub < N ? ld_as<TACC, TV>(xj + r0 + sub) : (TACC)0;
+    }
+  }
+}
+
 // Diagonal part of step j's SpMV for the rows [s0, s1) of a super-tile: (A v_j) into Ws and
 // u_j into Us (shared memory, from row s0; zeros past N)
 template <int ND, typename TV, typename TACC>
 __device__ __forceinline__ void arn_diag(const ArnArgs<TV, TACC>& a, int j, long long s0,
-                                         long long s1, TACC* Ws, TACC* Us) {
+                                         long long s1, TACC* Ws, TACC* Us, int tid, int nthr) {
   constexpr int B = sizeof(TACC) == 8 ? 2 : 4;  // SpMV rows per thread and batch
   const long long N = a.N;
   const TV* xj = a.V + (size_t)j * a.ldv;
+  if constexpr (ND == kArnCsr) {
+    arn_csr<TV, TACC>(a, xj, s0, s1, Ws, Us, tid, nthr);
+    return;
+  }
   const int nd = ND > 0 ? ND : a.dia.nd;
-  for (long long i0 = s0 + threadIdx.x; i0 < s1; i0 += (long long)B * kArnThreads) {
+  for (long long i0 = s0 + tid; i0 < s1; i0 += (long long)B * nthr) {
     TACC v[B];
-    arn_dia_rows<B, ND, TV, TACC>(v, i0, kArnThreads, N, nd, a.dia.off, a.ldd, a.dval, xj);
+    arn_dia_rows<B, (ND > 0 ? ND : 0), TV, TACC>(v, i0, nthr, N, nd, a.dia.off, a.ldd, a.dval, xj);
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-      const long long row = i0 + (long long)b * kArnThreads;
+      const long long row = i0 + (long long)b * nthr;
       if (row < s1) {
         Ws[row - s0] = row < N ? v[b] : (TACC)0;
         Us[row - s0] = row < N ? ld_as<TACC, TV>(xj + row) : (TACC)0;
@@ -638,12 +795,32 @@ __device__ __forceinline__ void arn_diag(const ArnArgs<TV, TACC>& a, int j, long
   }
 }
 
+// The block's column sums of a fixed-point multi-dot over nch chunks: the warps' integer totals, then FP64 once
+// per super-tile (added to the earlier super-tiles' unless first)
+template <int NSET>
+__device__ __forceinline__ void arn_slot_sums(const int4* slot, int nch, int k, const int* sE,
+                                              int ew, int eu, bool first, double* sred) {
+  const int rows = nch < kArnWarps ? nch : kArnWarps;
+  for (int q = threadIdx.x; q < NSET * k; q += kArnThreads) {
+    const int set = q / k, c = q % k;
+    long long sum = 0, f = 0;
+#pragma unroll 4
+    for (int w = 0; w < rows; ++w) {
+      const int4 v = slot[(size_t)(set * kArnWarps + w) * kMaxK + c];
+      sum += ((long long)v.y << 32) | (unsigned)v.x;
+      f += ((long long)v.w << 32) | (unsigned)v.z;
+    }
+    const double d = fx_value(sum, f, sE[c], set ? eu : ew);
+    sred[q] = first ? d : sred[q] + d;
+  }
+}
+
 // SpMV, coarse correction and multi-dot of step j over the block's super-tiles (a function
 // of its own, so that the cycle loop's state stays out of these loops' registers)
-template <typename TV, typename TACC, int ND, bool DF>
+template <typename TV, typename TACC, int ND, int MODE>
 __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TACC sig, bool waited,
                                        bool first_diag_done, TACC* Ws, TACC* Us, TACC* Ss,
-                                       double* sbuf, int* sEb, int* semax, double* sred) {
+                                       double* sbuf, const int* sE, int* semax, double* sred) {
   constexpr int VN = ArnVec<TV>::n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = threadIdx.x;
@@ -658,7 +835,7 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
     const long long s1 = s0 + a.RS < R1 ? s0 + a.RS : R1;
     // ---- 1. SpMV of the super-tile's rows: w and u_j into shared memory (the first
     // super-tile's may have been formed during the previous step's coarse solve) ---------
-    if (!(first_diag_done && s0 == R0)) arn_diag<ND, TV, TACC>(a, j, s0, s1, Ws, Us);
+    if (!(first_diag_done && s0 == R0)) arn_diag<ND, TV, TACC>(a, j, s0, s1, Ws, Us, t, kArnThreads);
     // + A W s' (the row's A W entries, s' from shared memory), the scale sigma_j; w also to
     // global memory when the update reads it there.
     if constexpr (sizeof(TACC) == 8) {
@@ -673,9 +850,9 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
       }
       if (a.defl && s0 == R0)
         for (int q = t; q < a.r; q += kArnThreads) Ss[q] = sig * __ldcg(a.sdefl + q);
-      if (t < 2) semax[t] = 0;
+      if (t == 0) semax[0] = 0;
       __syncthreads();
-      int mw = 0, mu = 0;  // high words of the largest |w|, |u_j| of the super-tile
+      int mw = 0;  // high word of the largest |w| of the super-tile
       constexpr int AWR = kArnAwRows64;
       for (long long i0 = s0 + t; i0 < s1; i0 += (long long)AWR * kArnThreads) {
         int e0[AWR], e1[AWR];
@@ -707,16 +884,11 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
             }
             Ws[row - s0] = wv;
             mw = max(mw, fx_mag(wv));
-            mu = max(mu, fx_mag(Us[row - s0]));
           }
         }
       }
       mw = __reduce_max_sync(0xffffffffu, mw);
-      mu = __reduce_max_sync(0xffffffffu, mu);
-      if (lane == 0) {
-        atomicMax(&semax[0], mw);
-        atomicMax(&semax[1], mu);
-      }
+      if (lane == 0) atomicMax(&semax[0], mw);
     } else {
       // FP32: a row's first two A W entries from the row-indexed planes (one level of loads,
       // kArnAwRows32 rows per thread at once); the first batch's loads are issued before s'
@@ -774,14 +946,12 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
     }
     __syncthreads();
     const int nch = (int)((s1 - s0) / (32 * VN));
+    constexpr int NSET = MODE == kArnCgs2 ? 1 : 2;  // w alone, or w and u_j
     if constexpr (sizeof(TV) == 8) {
-      // w and u_j to fixed point in place (relative to their largest exponents in the
-      // super-tile), then the dots with every column; the columns' exponents are kept per
-      // super-tile (the last slot is shared by all later ones, as their maximum)
-      const int ew = semax[0] >> 20, eu = semax[1] >> 20;
-      int* ebt = sEb + (tile < kArnEbTiles ? tile : kArnEbTiles - 1) * kMaxK;
-      if (t == 0) ebt[j] = tile < kArnEbTiles ? eu : max(ebt[j], eu);
-      if constexpr (DF) {
+      // w and u_j to fixed point in place (relative to the largest exponent of w in the
+      // super-tile, of u_j as a whole), then the dots with every column
+      const int ew = semax[0] >> 20, eu = sE[j];
+      if constexpr (MODE == kArnLowsyncDf) {
         // w and u_j split in place (float2 hi, lo in the 8 bytes of each double)
         for (int q = t; q < (int)(s1 - s0); q += kArnThreads) {
           float h1, l1, h2, l2;
@@ -798,112 +968,222 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
         continue;
       }
       for (int q = t; q < (int)(s1 - s0); q += kArnThreads) {
-        const Fx fw = fx_conv((double)Ws[q], ew + 8);
-        const Fx fu = fx_conv((double)Us[q], eu + 8);
-        reinterpret_cast<int2*>(Ws)[q] = make_int2(fw.h, fw.l);
-        reinterpret_cast<int2*>(Us)[q] = make_int2(fu.h, fu.l);
+        reinterpret_cast<int2*>(Ws)[q] = fx_operand((double)Ws[q], ew);
+        if (NSET == 2) reinterpret_cast<int2*>(Us)[q] = fx_operand((double)Us[q], eu);
       }
       __syncthreads();
       int4* slot = reinterpret_cast<int4*>(sbuf);
-      arn_dots_fx<2, kArnFxGroup>(slot, reinterpret_cast<const double*>(a.V), a.ldv, k, s0, nch,
-                                  reinterpret_cast<const int4*>(Ws),
-                                  reinterpret_cast<const int4*>(Us), ebt, warp, lane);
+      arn_dots_fx<NSET, (NSET == 2 ? kArnFxGroup : kArnFxGroup1), kArnFxDepth>(
+          slot, reinterpret_cast<const double*>(a.V), a.ldv, j, k, eu, s0, nch,
+          reinterpret_cast<const int4*>(Ws), reinterpret_cast<const int4*>(Us), lane);
       __syncthreads();
-      // the block's column sums: the 16 warps' integer totals, then FP64 once per super-tile
-      for (int q = t; q < 2 * k; q += kArnThreads) {
-        const int set = q / k, c = q % k;
-        long long sum = 0;
-        unsigned long long f = 0;
-#pragma unroll 4
-        for (int w = 0; w < kArnWarps; ++w) {
-          const int4 v = slot[(size_t)(set * kArnWarps + w) * kMaxK + c];
-          sum += ((long long)v.y << 32) | (unsigned)v.x;
-          f += (unsigned)v.z;
-        }
-        sum += (long long)(f >> 32);
-        const double d = fx_value(sum, (unsigned)f, ebt[c], (set ? eu : ew) + 1);
-        sred[q] = tile == 0 ? d : sred[q] + d;
-      }
+      arn_slot_sums<NSET>(slot, nch, k, sE, ew, eu, tile == 0, sred);
     } else {
-        arn_dots_rows<TV, TACC, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, Ws, Us, warp, lane);
+      arn_dots_rows<TV, TACC, NSET, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, Ws, Us, warp, lane);
     }
     __syncthreads();  // the slices are rewritten by the next super-tile
   }
 }
 
-// The same update of an FP64 basis in fixed point (fixed.cuh), super-tile by super-tile from the
-// last: the coefficients, each times its column's unit, become integers K_c relative to the
-// largest of them, a row's sum of M_c K_c (at most kMaxK terms) stays in integer
-// accumulators, and FP64 enters once per row, u = w - scale * sum.  Bound by the basis loads;
-// FP64 multiply-adds would cost 64 issue slots per entry, this form about 16.
-__device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, double* vout,
-                                                const double* w, int RS, long long R0,
-                                                long long R1, int k, const double* scoef,
-                                                const int* sEb, int4* sK, double* sscale,
-                                                double* ush) {
-  constexpr int U = 6;  // basis loads in flight per lane
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double nrm = 0.0;
-  const int tiles = (int)((R1 - R0 + RS - 1) / RS);
-  for (int tile = tiles - 1; tile >= 0; --tile) {
-    const long long s0 = R0 + (long long)tile * RS;
-    const long long s1 = s0 + RS < R1 ? s0 + RS : R1;
-    const int* ebt = sEb + (tile < kArnEbTiles ? tile : kArnEbTiles - 1) * kMaxK;
-    __syncthreads();
-    if (warp == 0) {
-      int m = 0;
-      bool bad = false;
-      for (int c = lane; c < k; c += 32) {
-        const int e = fx_mag(scoef[c]) >> 20;
-        bad |= e == 2047 || ebt[c] == 2047;
-        m = max(m, e + ebt[c]);
-      }
-      m = __reduce_max_sync(0xffffffffu, m);
-      bad = __any_sync(0xffffffffu, bad);
-      for (int c = lane; c < k; c += 32) {
-        const int3 f = fx_coef(scoef[c], m, ebt[c]);
-        sK[c] = make_int4(f.x, f.y, f.z, ebt[c] + 3);
-      }
-      if (lane == 0)
-        *sscale = bad ? __longlong_as_double(0x7ff8000000000000ll) : -ldexp(1.0, m - 2098);
+// The update's part of the reduction scratch: the coefficients at its end, past one dot set's slots
+// (CGS2's second multi-dot) and the split update's partial sums
+__device__ __forceinline__ int4* arn_sk(double* sbuf) {
+  static_assert(kArnScratch >= (15 * 32 * 3 + kMaxK) * 16, "partial sums and coefficients");
+  static_assert(kArnScratch >= (kArnWarps + 1) * kMaxK * 16, "slots and coefficients");
+  return reinterpret_cast<int4*>(sbuf) + kArnScratch / 16 - kMaxK;
+}
+
+// w - V (sigma o h) of the rows [s0, s1) (an FP64 basis): a row's sum of M_c K_c (at most kMaxK
+// terms) stays in integer accumulators, and FP64 enters once per row; put(r, value of row r, of
+// row r + 1) takes the results.  FIXED: the first kf columns are fixed-point integers, a last one
+// (k = kf + 1) is FP64 and is converted in place on the way (no other block reads it any more:
+// the SpMV is behind the last grid barrier); else all columns are FP64 and stay so.  Each loaded
+// value's register is reloaded U columns on (past the last column: from the warp's next chunk)
+// as soon as it is used.  With fewer than 16 chunks the warps of a chunk share its columns and
+// add their integer sums through sP.  Bound by the basis loads; FP64 multiply-adds would cost 64
+// issue slots per entry, this form about 7.  Called by all threads.
+constexpr int kArnUpdLoads = 6;  // basis loads in flight per lane
+
+template <bool FIXED, typename F>
+__device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ldv,
+                                                   const double* w, long long s0, long long s1,
+                                                   int kf, int k, const int* sE, const int4* sK,
+                                                   double nscale, longlong2* sP, F&& put) {
+  constexpr int U = kArnUpdLoads;
+  const int lane = threadIdx.x & 31;
+  const int nch = (int)((s1 - s0) >> 6);
+  const ArnSplit sp = arn_split(nch);
+  const int c0 = sp.p * kf / sp.S, c1 = (sp.p + 1) * kf / sp.S;
+  long long r = s0 + (long long)(nch - 1 - sp.q0) * 64 + lane * 2;
+  const bool one = sp.S > 1;
+  const long long* const Vi = reinterpret_cast<const long long*>(V);
+  // the FP64 column's part of the rows at r, then the finished rows
+  auto finish = [&](FxAcc& a0, FxAcc& a1) {
+    const double2 wv = __ldcg(reinterpret_cast<const double2*>(w + r));
+    if (FIXED && kf < k) {
+      double* pj = const_cast<double*>(V) + (size_t)kf * ldv + r;
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(pj));
+      const long long m0 = fx_basis(v.x, sE[kf]), m1 = fx_basis(v.y, sE[kf]);
+      *reinterpret_cast<longlong2*>(pj) = make_longlong2(m0, m1);
+      fx_axpy(a0, fx_limbs(m0), sK[kf]);
+      fx_axpy(a1, fx_limbs(m1), sK[kf]);
     }
-    __syncthreads();
-    const double nscale = *sscale;
-    const int nch = (int)((s1 - s0) >> 6);
-    for (int q = nch - 1 - warp; q >= 0; q -= kArnWarps) {
-      const long long r = s0 + (long long)q * 64 + lane * 2;
-      const double2 wv = __ldcg(reinterpret_cast<const double2*>(w + r));
-      FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
-      for (int b = 0; b < k; b += U) {
-        double v[U][2];
+    // rows past N: w and the basis are zero there
+    put(r, fx_axpy_add(a0, wv.x, nscale), fx_axpy_add(a1, wv.y, nscale));
+  };
+  FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
+  if (sp.live && (!one || c0 < c1)) {
+    int nb = c0;  // column and row of the next load
+    long long nr = r;
+    const long long* pn = Vi + (size_t)c0 * ldv + r;
+    uint4 v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (b + u < k) arn_ldg<double, double, 2>(V + (size_t)(b + u) * ldv + r, v[u]);
+    for (int u = 0; u < U; ++u) {
+      v[u] = make_uint4(0, 0, 0, 0);
+      if (nb + u < c1) arn_ldfx(pn + (size_t)u * ldv, v[u]);
+    }
+    for (; r >= s0; r -= kArnWarps * 64) {
+      if (!one) a0 = a1 = FxAcc{0, 0, 0, 0};
+#pragma unroll 1
+      for (int b = c0; b < c1; b += U) {
+        nb += U;
+        pn += (size_t)U * ldv;
+        if (nb >= c1) {  // on to the next chunk
+          nb = c0;
+          nr -= kArnWarps * 64;
+          pn = Vi + (size_t)c0 * ldv + nr;
+        }
+        const bool more = nr >= s0 && (!one || nb > c0);
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (b + u < k) {
-            const int4 kc = sK[b + u];
-            fx_axpy(a0, fx_conv_near(v[u][0], kc.w), kc);
-            fx_axpy(a1, fx_conv_near(v[u][1], kc.w), kc);
+        for (int u = 0; u < U; ++u) {
+          const bool on = b + u < c1;
+          Fx f0, f1;
+          if (FIXED) {
+            f0 = fx_limbs(v[u].x, v[u].y);
+            f1 = fx_limbs(v[u].z, v[u].w);
+          } else {
+            const int e = sE[on ? b + u : c0];
+            f0 = fx_limbs(fx_basis(__hiloint2double((int)v[u].y, (int)v[u].x), e));
+            f1 = fx_limbs(fx_basis(__hiloint2double((int)v[u].w, (int)v[u].z), e));
           }
+          if (more && nb + u < c1) arn_ldfx(pn + (size_t)u * ldv, v[u]);
+          if (on) {
+            const int4 kc = sK[b + u];
+            fx_axpy(a0, f0, kc);
+            fx_axpy(a1, f1, kc);
+          }
+        }
       }
-      // rows past N: w and the basis are zero there
-      double un[2];
-      un[0] = fx_axpy_sub(a0, wv.x, nscale);
-      un[1] = fx_axpy_sub(a1, wv.y, nscale);
-      *reinterpret_cast<double2*>(vout + r) = make_double2(un[0], un[1]);
-      if (ush) *reinterpret_cast<double2*>(ush + (r - R0)) = make_double2(un[0], un[1]);
-      nrm = fma(un[0], un[0], fma(un[1], un[1], nrm));
+      if (one) break;
+      finish(a0, a1);
     }
   }
+  if (!one) return;
+  // sP[part][chunk][lane][3]: hh, hl with the leading l kl, lh of both rows
+  if (sp.live && sp.p > 0) {
+    longlong2* q = sP + ((size_t)((sp.p - 1) * nch + sp.q0) * 32 + lane) * 3;
+    q[0] = make_longlong2(a0.hh, a1.hh);
+    q[1] = make_longlong2(a0.hl + 4ll * a0.ll, a1.hl + 4ll * a1.ll);
+    q[2] = make_longlong2(a0.lh, a1.lh);
+  }
+  __syncthreads();
+  if (sp.live && sp.p == 0) {
+    for (int p = 1; p < sp.S; ++p) {
+      const longlong2* q = sP + ((size_t)((p - 1) * nch + sp.q0) * 32 + lane) * 3;
+      const longlong2 hh = q[0], hl = q[1], lh = q[2];
+      a0.hh += hh.x; a0.hl += hl.x; a0.lh += lh.x;
+      a1.hh += hh.y; a1.hl += hl.y; a1.lh += lh.y;
+    }
+    finish(a0, a1);
+  }
+}
+
+// the coefficients (sK) and minus the unit of the sum (sscale), the same in every block; called by
+// all threads, ends with a barrier
+__device__ __forceinline__ void arn_fx_coefs(int k, const double* scoef, const int* sE, int4* sK,
+                                             double* sscale) {
+  if (threadIdx.x < 32) {
+    const double s = fx_coefs(k, scoef, sE, sK);
+    if (threadIdx.x == 0) *sscale = -s;
+  }
+  __syncthreads();
+}
+
+// u_{j+1} of the block's rows into vout (and ush, indexed from R0); returns the warp's part of
+// ||u_{j+1}||^2, and in mx the high word of the thread's largest |u_{j+1}|.  kf: the columns
+// already in fixed point
+template <bool FIXED>
+__device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, double* vout,
+                                                const double* w, long long R0, long long R1,
+                                                int kf, int k, const double* scoef,
+                                                const int* sE, double* sbuf, double* sscale,
+                                                double* ush, int& mx) {
+  int4* sK = arn_sk(sbuf);
+  double nrm = 0.0;
+  int m = 0;
+  arn_fx_coefs(k, scoef, sE, sK, sscale);
+  arn_rows_update_fx<FIXED>(
+      V, ldv, w, R0, R1, kf, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
+      [&](long long r, double u0, double u1) {
+        *reinterpret_cast<double2*>(vout + r) = make_double2(u0, u1);
+        if (ush) *reinterpret_cast<double2*>(ush + (r - R0)) = make_double2(u0, u1);
+        nrm = fma(u0, u0, fma(u1, u1, nrm));
+        m = max(m, max(fx_mag(u0), fx_mag(u1)));
+      });
+  mx = m;
   return warp_sum(nrm);
 }
 
-// u_{j+1} = w - V (sigma o h) over the block's rows of an FP32 basis (also into ush, indexed from
+// CGS2, first update and second multi-dot of an FP64 basis: per super-tile (from the last) w -= V
+// (sigma o h) into w and shared memory (the newest column becomes fixed-point on the way), its
+// operand form, then V^T w into sred
+__device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, double* w, int RS,
+                                             long long R0, long long R1, int k,
+                                             const double* scoef, const int* sE, double* Ws,
+                                             double* sbuf, int* semax, double* sscale,
+                                             double* sred) {
+  const int lane = threadIdx.x & 31;
+  int4* slot = reinterpret_cast<int4*>(sbuf);
+  int4* sK = arn_sk(sbuf);
+  const int tiles = (int)((R1 - R0 + RS - 1) / RS);
+  __syncthreads();  // scoef
+  arn_fx_coefs(k, scoef, sE, sK, sscale);
+  for (int tile = tiles - 1; tile >= 0; --tile) {
+    const long long s0 = R0 + (long long)tile * RS;
+    const long long s1 = s0 + RS < R1 ? s0 + RS : R1;
+    if (threadIdx.x == 0) semax[0] = 0;
+    __syncthreads();
+    int mw = 0;
+    arn_rows_update_fx<true>(
+        V, ldv, w, s0, s1, k - 1, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
+        [&](long long r, double u0, double u1) {
+          *reinterpret_cast<double2*>(w + r) = make_double2(u0, u1);
+          *reinterpret_cast<double2*>(Ws + (r - s0)) = make_double2(u0, u1);
+          mw = max(mw, max(fx_mag(u0), fx_mag(u1)));
+        });
+    mw = __reduce_max_sync(0xffffffffu, mw);
+    if (lane == 0) atomicMax(&semax[0], mw);
+    __syncthreads();
+    const int ew = semax[0] >> 20;
+    for (int q = threadIdx.x; q < (int)(s1 - s0); q += kArnThreads)
+      reinterpret_cast<int2*>(Ws)[q] = fx_operand(Ws[q], ew);
+    __syncthreads();
+    const int nch = (int)((s1 - s0) >> 6);
+    arn_dots_fx<1, kArnFxGroup1, kArnFxDepth>(slot, V, ldv, k, k, 0, s0, nch,
+                                 reinterpret_cast<const int4*>(Ws), nullptr, lane);
+    __syncthreads();
+    arn_slot_sums<1>(slot, nch, k, sE, ew, 0, tile == tiles - 1, sred);
+  }
+  __syncthreads();
+}
+
+// u_{j+1} = w - V (sigma o h) over the block's rows of an FP32 or BF16 basis (also into ush, indexed from
 // the block's first row, when given); returns the warp's part of ||u_{j+1}||^2 (in every lane)
-template <typename TV, typename TACC>
-__device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, const TACC* Ws,
-                                          const TACC* scoef, TACC* ush) {
+// (PASS2: only the rows [base, end), w back into Ws, indexed from base, and global memory)
+template <typename TV, typename TACC, bool PASS2>
+__device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
+                                          const TACC* scoef, TACC* ush, long long base,
+                                          long long end) {
   constexpr int VN = ArnVec<TV>::n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = gridDim.x, bid = blockIdx.x;
@@ -913,12 +1193,12 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
   TV* __restrict__ vout = const_cast<TV*>(a.V) + (size_t)k * a.ldv;
   float ns = 0.f, nc = 0.f;  // a double-FP32 pair (FP64 adds are dear)
   {
-    constexpr int U = 8;  // basis loads in flight per lane
+    constexpr int U = PASS2 ? 4 : 8;  // basis loads in flight per lane
     const int chunk = 32 * VN;
-    const long long nch = (R1 - R0) / chunk;
+    const long long nch = (end - base) / chunk;
     const bool wsm = R1 - R0 <= a.RS;  // the block's w is still in shared memory
     for (long long q = nch - 1 - warp; q >= 0; q -= kArnWarps) {
-      const long long r = R0 + q * chunk + (long long)lane * VN;
+      const long long r = base + q * chunk + (long long)lane * VN;
       TACC wv[VN], p[VN];
       if (wsm) {
         ld_acc<VN>(Ws + (r - R0), wv);
@@ -944,7 +1224,20 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
       TACC un[VN];
 #pragma unroll
       for (int e = 0; e < VN; ++e) un[e] = wv[e] - p[e];
+      if constexpr (PASS2) {  // CGS2's first update: w stays where it came from
+        if (wsm) {
+          acc_store<VN>(Ws + (r - R0), un);
+        } else {
+          acc_store<VN>(a.w + r, un);
+          acc_store<VN>(Ws + (r - base), un);
+        }
+        continue;
+      }
       arn_stv<TV, TACC, VN>(vout + r, un);
+      if constexpr (sizeof(TV) == 2) {  // the stored (rounded) values count
+#pragma unroll
+        for (int e = 0; e < VN; ++e) un[e] = __bfloat162float(__float2bfloat16_rn(un[e]));
+      }
       if (ush) acc_store<VN>(ush + (r - R0), un);  // for the piece sums
       TACC s = 0;
 #pragma unroll
@@ -962,12 +1255,37 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
   return (double)ns + (double)nc;
 }
 
+// CGS2, first update and second multi-dot of an FP32 or BF16 basis: per super-tile (from the last)
+// w -= V (sigma o h), then V^T w into the per-warp pairs.  A call of its own: inlined, the two
+// loops' registers spilled (240 to 690 bytes a thread).
+template <typename TV, typename TACC, int ND>
+__device__ __noinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
+                                            const TACC* scoef, double* sbuf) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int G = gridDim.x, bid = blockIdx.x;
+  const long long R0 = (long long)bid * a.units / G * kArnUnit;
+  const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
+  for (int q = threadIdx.x; q < kMaxK * kArnWarps; q += kArnThreads) sbuf[q] = 0.0;
+  const int tiles = (int)((R1 - R0 + a.RS - 1) / a.RS);
+  for (int tile = tiles - 1; tile >= 0; --tile) {
+    const long long s0 = R0 + (long long)tile * a.RS;
+    const long long s1 = s0 + a.RS < R1 ? s0 + a.RS : R1;
+    __syncthreads();
+    arn_update<TV, TACC, true>(a, k, Ws, scoef, nullptr, s0, s1);
+    __syncthreads();
+    arn_dots_rows<TV, TACC, 1, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0,
+                                                (int)((s1 - s0) / (32 * ArnVec<TV>::n)), Ws,
+                                                nullptr, warp, lane);
+  }
+  __syncthreads();
+}
+
 // Sums of u_{j+1} over this block's aggregate pieces (c of the next step's coarse solve, by
 // pieces, a warp each).  The pieces' bounds are loaded up front (lane i < 8 holds the
 // warp's i-th piece), then per piece the node indexes and the values: from the shared-memory
 // copy of the block's rows when there is one (ush, from row R0), else through L2 (this
 // block wrote them just before).  Fixed order throughout.
-template <typename TV, typename TACC>
+template <bool C32, typename TV, typename TACC>
 __device__ __forceinline__ void arn_piece_sums(const ArnArgs<TV, TACC>& a, const TV* vout,
                                                const TACC* ush, long long R0) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1002,7 +1320,7 @@ __device__ __forceinline__ void arn_piece_sums(const ArnArgs<TV, TACC>& a, const
       }
       const double sum = warp_sum(acc[0] + acc[1]);
       if (lane == 0) {
-        if constexpr (sizeof(TACC) == 8) {
+        if constexpr (!C32) {
           __stcg(a.ctl.cpart + p, sum);
         } else {  // the pair the FP32 coarse solve reads
           const float hs = (float)sum;
@@ -1018,21 +1336,21 @@ __device__ __forceinline__ void arn_piece_sums(const ArnArgs<TV, TACC>& a, const
 // pipe, exact to about 2^-48 of the sum's magnitude), rounded to FP64 once per piece.
 constexpr int kArnMaxBlkPieces = 256;
 
-template <typename TACC>
+template <bool C32, typename TACC>
 __device__ __forceinline__ void arn_piece_sums_staged(double* cpart, const TACC* ush,
                                                       const unsigned short* snode,
                                                       const int* spid, const int* spls, int np) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = warp; i < np; i += kArnWarps) {
     const int ls = spls[i], le = spls[i + 1];
-    double sum;
-    if constexpr (sizeof(TACC) == 8) {
+    if constexpr (!C32) {
       double acc[2] = {0.0, 0.0};
       for (int q = ls + lane; q < le; q += 64) {
         acc[0] += (double)ush[snode[q]];
         if (q + 32 < le) acc[1] += (double)ush[snode[q + 32]];
       }
-      sum = warp_sum(acc[0] + acc[1]);
+      const double sum = warp_sum(acc[0] + acc[1]);
+      if (lane == 0) __stcg(cpart + spid[i], sum);
     } else {
       float hs = 0.f, hc = 0.f;
       for (int q = ls + lane; q < le; q += 32) arn_df_add(hs, hc, (float)ush[snode[q]], 0.f);
@@ -1044,25 +1362,74 @@ __device__ __forceinline__ void arn_piece_sums_staged(double* cpart, const TACC*
       }
       // an FP32 basis keeps the pair (two floats in the slot) for the FP32 coarse solve
       if (lane == 0) __stcg(reinterpret_cast<float2*>(cpart + spid[i]), make_float2(hs, hc));
-      continue;
     }
-    if (lane == 0) __stcg(cpart + spid[i], sum);
   }
 }
 
-template <typename TV, typename TACC, int ND, bool DF>
+// The block's largest high word of |u| (the warp's lanes hold the candidates) into its slot of the
+// partials, and after a grid barrier the largest exponent over all blocks (one warp each)
+__device__ __forceinline__ void arn_put_max(Ctl& ctl, int m) {
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0)
+    __stcg(&ctl.part[(size_t)blockIdx.x * ctl.ldp + kArnMaxCol], __hiloint2double(0, m));
+}
+__device__ __forceinline__ int arn_get_max(const Ctl& ctl) {
+  int m = 0;
+  for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32)
+    m = max(m, __double2loint(__ldcg(&ctl.part[(size_t)b * ctl.ldp + kArnMaxCol])));
+  return __reduce_max_sync(0xffffffffu, m) >> 20;
+}
+
+// The 16 warps' pairs of ncols columns (sets of k) in warp order: double-FP32 multi-dots of an
+// FP64 basis rounded to FP64 once, sums of an FP32 or BF16 basis kept as pairs
+template <typename TV, int MODE>
+__device__ __forceinline__ void arn_block_sums(const double* sbuf, int ncols, int k, double* sred) {
+  if constexpr (sizeof(TV) == 8 && MODE == kArnLowsyncDf) {
+    for (int q = threadIdx.x; q < ncols; q += kArnThreads) {
+      const int set = q / k, c = q % k;
+      const float* dfp = reinterpret_cast<const float*>(sbuf);
+      float s = 0.f, cc = 0.f;
+      for (int w = 0; w < kArnWarps; ++w) {
+        const float* p = dfp + ((size_t)w * kMaxK + c) * 4 + 2 * set;
+        arn_df_add(s, cc, p[0], p[1]);
+      }
+      sred[q] = (double)s + (double)cc;
+    }
+  } else if constexpr (sizeof(TV) < 8) {
+    for (int q = threadIdx.x; q < ncols; q += kArnThreads) {
+      const int set = q / k, c = q % k;
+      const float2* ws = reinterpret_cast<const float2*>(sbuf);
+      float hs = 0.f, hc = 0.f;
+      for (int w = 0; w < kArnWarps; ++w) {
+        const float2 v = ws[(size_t)(set * kArnWarps + w) * kMaxK + c];
+        arn_df_add(hs, hc, v.x, v.y);
+      }
+      reinterpret_cast<float2*>(sred)[q] = make_float2(hs, hc);
+    }
+  }
+  __syncthreads();
+}
+
+template <typename TV, typename TACC, int ND, int MODE>
 __global__ void __launch_bounds__(kArnThreads, 1)
     k_arnoldi(const __grid_constant__ ArnArgs<TV, TACC> a) {
-  static_assert(std::is_same<TV, TACC>::value, "w and u_j slices share the basis element type");
-  static_assert(!DF || sizeof(TV) == 8, "the double-FP32 multi-dot takes an FP64 basis");
+  static_assert(MODE != kArnLowsyncDf || sizeof(TV) == 8, "the double-FP32 multi-dot takes an FP64 basis");
+  static_assert(MODE == kArnCgs2 || sizeof(TV) == sizeof(TACC), "BF16 bases use CGS2");
+  // the FP32 one-reduction step of a banded operator runs its coarse solve in FP32, every
+  // other instantiation in FP64
+  constexpr bool C32 = sizeof(TV) == 4 && MODE == kArnLowsync && ND != kArnCsr;
+  constexpr int NSET = MODE == kArnCgs2 ? 1 : 2;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double tot[2 * kMaxK + 1];
   __shared__ double sred[2 * kMaxK];
   __shared__ double sg[kMaxK];
   __shared__ TACC scoef[kMaxK];
   __shared__ double snrm[kArnWarps];
+  __shared__ int smax[kArnWarps];
   __shared__ double ssig[kMaxK + 1];
-  __shared__ int semax[2];
+  // FP64: the columns' largest exponents, of w in a super-tile, and the unit of an update
+  __shared__ int sE[kMaxK + 1];
+  __shared__ int semax[1];
   __shared__ double sscale;
   // the control block is read from the grid-constant parameter (no register copy)
   Ctl& ctl = const_cast<Ctl&>(a.ctl);
@@ -1080,7 +1447,6 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   double* scratch = reinterpret_cast<double*>(
       smem + ((2 * (size_t)a.RS + (size_t)a.r) * sizeof(TACC) + 127) / 128 * 128);
   double* sL = scratch + kArnScratch / sizeof(double);
-  int* sEb = reinterpret_cast<int*>(sL + (size_t)kMaxK * kMaxK);  // FP64: [tile][column]
   double* sbuf = scratch;
   double* sc = reinterpret_cast<double*>(smem);  // c of the coarse solve (w, u_j are dead)
 
@@ -1151,7 +1517,7 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   int* sap = nullptr;       // agg_piece, r + 1
   float* sus = nullptr;     // uscale, r
   float* stinv = nullptr;   // the block's rows of T^-1 (warp w: row (b - 1) + (G - 1) w)
-  if constexpr (sizeof(TACC) == 4) {
+  if constexpr (C32) {
     const int nwr = G == 1 ? kArnWarps : (G - 1) * kArnWarps;  // warps sharing the rows
     const int rows = (a.defl && bid > 0 && a.r <= nwr && bid - 1 < a.r)
                          ? min(kArnWarps, (a.r - (bid - 1) + G - 2) / (G - 1)) : 0;
@@ -1169,6 +1535,28 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     }
   }
   bool waited = !a.pre;
+  if constexpr (sizeof(TV) == 8) {  // the exponent of u_0: one more grid barrier per cycle
+    if (!waited) {
+      pdl_wait();
+      pdl_trigger();
+      waited = true;
+    }
+    int mx = 0;
+    for (long long r = R0 + t; r < R1; r += kArnThreads) mx = max(mx, fx_mag(__ldcg(a.V + r)));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) smax[warp] = mx;
+    __syncthreads();
+    if (warp == 0) arn_put_max(ctl, lane < kArnWarps ? smax[lane] : 0);
+    if (!arn_grid_sync(a.gbar, gen++)) {
+      arn_timeout(ctl);
+      return;
+    }
+    if (warp == 0) {
+      const int e = arn_get_max(ctl);
+      if (lane == 0) sE[0] = e;
+      if (lane == 0 && bid == 0) ctl.vexp[0] = e;
+    }
+  }
   __syncthreads();
 
   for (int j = 0; j < a.jmax; ++j) {
@@ -1177,52 +1565,56 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // partial sums of the multi-dot in shared memory, so that they persist across
     // super-tiles (FP64: lane-wise per column; FP32: per warp and column; double-FP32:
     // pairs per warp and column)
-    if constexpr (sizeof(TV) == 4 || DF)
+    if constexpr (sizeof(TV) < 8 || MODE == kArnLowsyncDf)
       for (int q = t; q < 2 * kMaxK * 33; q += kArnThreads) sbuf[q] = 0.0;
-    if (sizeof(TV) == 8 && t == 0)
-      sEb[(kArnEbTiles - 1) * kMaxK + j] = 0;  // a running maximum
-    arn_front<TV, TACC, ND, DF>(a, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sEb, semax, sred);
+    arn_front<TV, TACC, ND, MODE>(a, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sE, semax, sred);
     waited = true;
-    // per-block column sums (fixed order)
-    if constexpr (DF) {  // the 16 warps' pairs of each column in warp order, then FP64 once
-      for (int q = t; q < 2 * k; q += kArnThreads) {
-        const int set = q / k, c = q % k;
-        const float* dfp = reinterpret_cast<const float*>(sbuf);
-        float s = 0.f, cc = 0.f;
-        for (int w = 0; w < kArnWarps; ++w) {
-          const float* p = dfp + ((size_t)w * kMaxK + c) * 4 + 2 * set;
-          arn_df_add(s, cc, p[0], p[1]);
-        }
-        sred[q] = (double)s + (double)cc;
-      }
-    } else if constexpr (sizeof(TV) == 4) {  // the 16 warps' pairs in warp order, kept as a pair
-      for (int q = t; q < 2 * k; q += kArnThreads) {
-        const int set = q / k, c = q % k;
-        const float2* ws = reinterpret_cast<const float2*>(sbuf);
-        float hs = 0.f, hc = 0.f;
-        for (int w = 0; w < kArnWarps; ++w) {
-          const float2 v = ws[(size_t)(set * kArnWarps + w) * kMaxK + c];
-          arn_df_add(hs, hc, v.x, v.y);
-        }
-        reinterpret_cast<float2*>(sred)[q] = make_float2(hs, hc);
-      }
-    }
-    __syncthreads();
-    // the partials: FP64 values, or double-FP32 pairs (two floats in the slot) for an FP32
-    // basis, whose cross-block sums then run on the FP32 pipe
-    for (int c = t; c < 2 * k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
-    // ---- 3. grid barrier; identical totals in every block; (I + L) h = g ----------------
+    // per-block column sums (fixed order; a fixed-point multi-dot leaves them in sred)
+    arn_block_sums<TV, MODE>(sbuf, NSET * k, k, sred);
+    // the partials: FP64 values, or double-FP32 pairs (two floats in the slot) for an FP32 or
+    // BF16 basis, whose cross-block sums then run on the FP32 pipe
+    for (int c = t; c < NSET * k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
+    // ---- 3. grid barrier; identical totals in every block -------------------------------
     if (!arn_grid_sync(a.gbar, gen++)) {
       arn_timeout(ctl);
       return;
     }
-    if constexpr (sizeof(TV) == 4)
+    if constexpr (sizeof(TV) < 8)
       // (a thread's 152 / 8 rows of partials in one batch of loads)
-      arn_reduce_cols_df<24>(ctl.part, G, 2 * k, ctl.ldp, tot);  // ends with __syncthreads
+      arn_reduce_cols_df<24>(ctl.part, G, NSET * k, ctl.ldp, tot);  // ends with __syncthreads
     else
-      arn_reduce_cols(ctl.part, G, 2 * k, ctl.ldp, tot);
-    {
-      // the new row of L: v_j . v_c = sigma_j sigma_c (u_j . u_c), c < j; g_c = sigma_c (u_c . w)
+      arn_reduce_cols(ctl.part, G, NSET * k, ctl.ldp, tot);
+    if constexpr (MODE == kArnCgs2) {
+      // h = V^T w, first update and second multi-dot, one more barrier, h += h'
+      for (int c = t; c < k; c += kArnThreads) {
+        sg[c] = ssig[c] * tot[c];
+        scoef[c] = (TACC)(ssig[c] * sg[c]);
+      }
+      if constexpr (sizeof(TV) == 8) {
+        arn_pass2_fx(a.V, a.ldv, a.w, a.RS, R0, R1, k, scoef, sE, Ws,
+                     sbuf, semax, &sscale, sred);
+      } else {
+        arn_pass2_rows<TV, TACC, ND>(a, k, Ws, scoef, sbuf);
+      }
+      arn_block_sums<TV, MODE>(sbuf, k, k, sred);
+      for (int c = t; c < k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
+      if (!arn_grid_sync(a.gbar, gen++)) {
+        arn_timeout(ctl);
+        return;
+      }
+      if constexpr (sizeof(TV) < 8)
+        arn_reduce_cols_df<24>(ctl.part, G, k, ctl.ldp, tot);
+      else
+        arn_reduce_cols(ctl.part, G, k, ctl.ldp, tot);
+      for (int c = t; c < k; c += kArnThreads) {
+        const double h2 = ssig[c] * tot[c];
+        scoef[c] = (TACC)(ssig[c] * h2);
+        if (bid == 0) ctl.h[c] = sg[c] + h2;
+      }
+      __syncthreads();
+    } else {
+      // (I + L) h = g; the new row of L: v_j . v_c = sigma_j sigma_c (u_j . u_c), c < j;
+      // g_c = sigma_c (u_c . w)
       const double sj = ssig[k - 1];
       for (int c = t; c < k; c += kArnThreads) {
         if (c < k - 1) sL[(size_t)(k - 1) * kMaxK + c] = sj * ssig[c] * tot[k + c];
@@ -1264,28 +1656,35 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // super-tile (u_j's slice is dead by now)
     TACC* ush = (a.defl && k < a.jmax && R1 - R0 <= a.RS) ? Us : nullptr;
     double nrm;
+    int mx = 0;
     if constexpr (sizeof(TV) == 8)
-      nrm = arn_update_fx(a.V, a.ldv, vout, a.w, a.RS, R0, R1, k, scoef, sEb,
-                          reinterpret_cast<int4*>(sbuf), &sscale, ush);
+      nrm = arn_update_fx<MODE != kArnLowsyncDf>(
+          a.V, a.ldv, vout, a.w, R0, R1, MODE == kArnLowsync ? k - 1 : k, k, scoef, sE, sbuf,
+          &sscale, ush, mx);
     else
-      nrm = arn_update<TV, TACC>(a, k, Ws, scoef, ush);
+      nrm = arn_update<TV, TACC, false>(a, k, Ws, scoef, ush, R0, R1);
     // ---- 5. norm partial; partial sums of u_{j+1} over this block's aggregate pieces ----
     {
       // the warp sums (formed by the update), then warp 0 adds the 16 of them (a block-wide
       // final loop would issue 16 FP64 adds in every warp)
       if (lane == 0) snrm[warp] = nrm;
+      if constexpr (sizeof(TV) == 8) {
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) smax[warp] = mx;
+      }
       __syncthreads();  // also orders this block's stores of u_{j+1} before the piece sums
       if (warp == 0) {
         double bs = lane < kArnWarps ? snrm[lane] : 0.0;
 #pragma unroll
         for (int o = kArnWarps / 2; o > 0; o >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, o);
         if (lane == 0) __stcg(&ctl.part[(size_t)bid * ctl.ldp + kArnNormCol], bs);
+        if constexpr (sizeof(TV) == 8) arn_put_max(ctl, lane < kArnWarps ? smax[lane] : 0);
       }
       if (a.defl && k < a.jmax) {
         if (staged && ush)
-          arn_piece_sums_staged(ctl.cpart, ush, snode, spid, spls, bp1 - bp0);
+          arn_piece_sums_staged<C32>(ctl.cpart, ush, snode, spid, spls, bp1 - bp0);
         else
-          arn_piece_sums(a, vout, ush, R0);
+          arn_piece_sums<C32>(a, vout, ush, R0);
       }
     }
     if (!arn_grid_sync(a.gbar, gen++)) {
@@ -1295,18 +1694,25 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     const bool coarse = a.defl && k < a.jmax && (bid > 0 || G == 1);
     // ---- 6. ||u_{j+1}|| and the plane rotations with the stopping tests (block 0); the next
     // step's coarse solve s' = U (|mu| T^-1 - I) U^T u_{j+1} (the other blocks) -------------
-    if (bid == 0) {
-      arn_reduce_cols(ctl.part + kArnNormCol, G, 1, ctl.ldp, tot);
-      givens_step(ctl, j, a.m, sqrt(tot[0]));
+    const bool split0 = bid == 0 && G > 1;  // warp 0 alone: the others go on to the next SpMV
+    if (bid == 0 && warp == 0) {
+      double v = 0.0;
+      for (int b = lane; b < G; b += 32) v += __ldcg(&ctl.part[(size_t)b * ctl.ldp + kArnNormCol]);
+      givens_step(ctl, j, a.m, sqrt(warp_sum(v)));
+      __syncwarp();
+      if (split0 && lane == 0) {
+        __threadfence();
+        atomicAdd(&a.gbar[2], 1u);
+      }
     }
     if (coarse) {
       // y = T^-1 c: a warp per row, the rows dealt round-robin over blocks 1 .. G-1 (warp w
       // of block b takes rows (b - 1) + (G - 1) (w + 16 i)) so that each block has few; all
       // to block 0 when it is alone.  TQ loads in flight per lane (a whole row up to 1024)
-      constexpr int TQ = 32;
+      constexpr int TQ = sizeof(TACC) == 4 && !C32 ? 16 : 32;
       const int gw = G == 1 ? warp : (bid - 1) + (G - 1) * warp;
       const int nw = G == 1 ? kArnWarps : (G - 1) * kArnWarps;
-      if constexpr (sizeof(TACC) == 8) {
+      if constexpr (!C32) {
         // c_a = uscale_a (sum of a's pieces, in piece order), every aggregate in every block
         for (int q = t; q < a.r; q += kArnThreads) {
           const int p0 = __ldg(a.agg_piece + q), p1 = __ldg(a.agg_piece + q + 1);
@@ -1396,8 +1802,19 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // diagonal part of the next step's SpMV for the first super-tile, which needs only
     // u_{j+1} (complete since the barrier), not s' or sigma_{j+1} (it overwrites c); then
     // wait for every block's arrival
-    arn_arrive(&a.gbar[2]);
-    if (k < a.jmax) arn_diag<ND, TV, TACC>(a, k, R0, R0 + a.RS < R1 ? R0 + a.RS : R1, Ws, Us);
+    if (!split0) arn_arrive(&a.gbar[2]);
+    // the exponent of column j + 1 (one warp; the slots are written again only after this block's
+    // next arrival)
+    if constexpr (sizeof(TV) == 8) {
+      if (warp == kArnWarps - 1) {
+        const int e = arn_get_max(ctl);
+        if (lane == 0) sE[k] = e;
+        if (lane == 0 && bid == 0) ctl.vexp[k] = e;
+      }
+    }
+    if (k < a.jmax && (!split0 || warp > 0))
+      arn_diag<ND, TV, TACC>(a, k, R0, R0 + a.RS < R1 ? R0 + a.RS : R1, Ws, Us,
+                             split0 ? t - 32 : t, split0 ? kArnThreads - 32 : kArnThreads);
     if (!arn_wait(&a.gbar[2], cbase + (unsigned)G * (unsigned)k)) {
       arn_timeout(ctl);
       return;
@@ -1410,23 +1827,24 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   }
 }
 
+// rows of a super-tile: w and u_j slices, s' and the reduction scratch in kArnSmem
+inline long long arn_super_rows(int r, size_t esz) {
+  const size_t fixed = ((size_t)r * esz + 127) / 128 * 128 + kArnScratch +
+                       sizeof(double) * kMaxK * kMaxK + 256;
+  if (fixed >= kArnSmem) return 0;
+  return (long long)((kArnSmem - fixed) / (2 * esz)) / kArnUnit * kArnUnit;
+}
+
 template <typename TV, typename TACC>
 struct Arn {
-  // rows of a super-tile: w and u_j slices, s' and the reduction scratch in kArnSmem
-  static long long super_rows(int r) {
-    const size_t fixed = ((size_t)r * sizeof(TACC) + 127) / 128 * 128 + kArnScratch +
-                         sizeof(double) * kMaxK * kMaxK + kArnEbBytes + 256;
-    if (fixed >= kArnSmem) return 0;
-    return (long long)((kArnSmem - fixed) / (2 * sizeof(TACC))) / kArnUnit * kArnUnit;
-  }
-  template <int ND, bool DF>
+  template <int ND, int MODE>
   static cudaError_t prepare() {
-    return cudaFuncSetAttribute(k_arnoldi<TV, TACC, ND, DF>,
+    return cudaFuncSetAttribute(k_arnoldi<TV, TACC, ND, MODE>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kArnSmem);
   }
-  template <int ND, bool DF>
+  template <int ND, int MODE>
   static cudaError_t launch_nd(const CycleArgs& c, const ArnArgs<TV, TACC>& p, cudaStream_t st) {
-    static cudaError_t prep = prepare<ND, DF>();
+    static cudaError_t prep = prepare<ND, MODE>();
     if (prep != cudaSuccess) return prep;
     const int grid = p.units < c.sms ? p.units : c.sms;
     cudaLaunchConfig_t cfg = {};
@@ -1444,12 +1862,12 @@ struct Arn {
     // pair, the kernel runs cooperatively in plain stream order from then on (same result)
     static bool pdl_ok = true;
     cfg.numAttrs = (c.pdl && pdl_ok) ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_arnoldi<TV, TACC, ND, DF>, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_arnoldi<TV, TACC, ND, MODE>, p);
     if (e != cudaSuccess && cfg.numAttrs == 2) {
       (void)cudaGetLastError();
       pdl_ok = false;
       cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, k_arnoldi<TV, TACC, ND, DF>, p);
+      e = cudaLaunchKernelEx(&cfg, k_arnoldi<TV, TACC, ND, MODE>, p);
     }
     return e;
   }
@@ -1462,7 +1880,7 @@ struct Arn {
     p.pre = (defl && c.pdl) ? 1 : 0;
     p.defl = defl ? 1 : 0;
     p.r = defl ? c.op.defl.r : 0;
-    p.RS = (int)super_rows(p.r);
+    p.RS = (int)arn_super_rows(p.r, sizeof(TACC));
     if (p.RS < kArnUnit) return cudaErrorInvalidValue;  // arnoldi_fusable rules this out
     p.ldv = c.ldv;
     p.ldd = c.op.ldd;
@@ -1493,42 +1911,30 @@ struct Arn {
     p.tinv32 = c.op.defl.tinv32;
     p.ctl = c.ctl;
     p.gbar = c.gbar;
-    // the 9-point stencils of the Q1 systems take an unrolled instantiation
+    p.rowptr = c.op.rowptr;
+    p.col = c.op.col;
+    p.vec = c.op.vec;
+    if constexpr (sizeof(TACC) == 8) p.val = c.op.val;
+    else p.val = c.op.val32;
+    if (c.ortho == GMRES_ORTHO_CGS2) return launch_op<kArnCgs2>(c, p, st);
     if constexpr (sizeof(TV) == 8) {
-      if (c.dot_arith == GMRES_DOT_DF32)
-        return c.op.dia.nd == 9 ? launch_nd<9, true>(c, p, st) : launch_nd<0, true>(c, p, st);
+      // (a CSR operator takes the fixed-point multi-dot whatever dot_arith says)
+      if (c.dot_arith == GMRES_DOT_DF32 && c.op.dia.nd > 0)
+        return c.op.dia.nd == 9 ? launch_nd<9, kArnLowsyncDf>(c, p, st)
+                                : launch_nd<0, kArnLowsyncDf>(c, p, st);
     }
-    return c.op.dia.nd == 9 ? launch_nd<9, false>(c, p, st) : launch_nd<0, false>(c, p, st);
+    if constexpr (sizeof(TV) == sizeof(TACC)) return launch_op<kArnLowsync>(c, p, st);
+    else return cudaErrorInvalidValue;
+  }
+  // the 9-point stencils of the Q1 systems take an unrolled instantiation
+  template <int MODE>
+  static cudaError_t launch_op(const CycleArgs& c, const ArnArgs<TV, TACC>& p, cudaStream_t st) {
+    return c.op.dia.nd == 9  ? launch_nd<9, MODE>(c, p, st)
+           : c.op.dia.nd > 0 ? launch_nd<0, MODE>(c, p, st)
+                             : launch_nd<kArnCsr, MODE>(c, p, st);
   }
 };
 
 }  // namespace
-
-bool arnoldi_fusable(const CycleArgs& a) {
-  if (!(a.ortho == GMRES_ORTHO_MGS_LOWSYNC && a.op.dia.nd > 0 && !a.proj &&
-        a.op.defl.qd == 0 && a.ldv % kArnUnit == 0 && a.m + 1 <= kMaxK &&
-        (a.prec == P_FP64 || a.prec == P_FP32)))
-    return false;
-  const int r = a.op.defl.r;
-  // with deflation: the pieces split at this kernel's block rows (built at setup for a
-  // grid of min(units, SMs) blocks)
-  if (r > 0 && (!a.op.defl.blk_piece_start ||
-                a.op.defl.blk_grid != (int)std::min<long long>(a.ldv / kArnUnit, a.sms)))
-    return false;
-  if (r > 0 && a.prec == P_FP32 && !a.op.defl.tinv32) return false;  // its FP32 coarse solve
-  const long long rs = a.prec == P_FP64 ? Arn<double, double>::super_rows(r)
-                                        : Arn<float, float>::super_rows(r);
-  // c (r doubles) lives where w and u_j do
-  const size_t esz = a.prec == P_FP64 ? sizeof(double) : sizeof(float);
-  return rs >= kArnUnit && (size_t)r * sizeof(double) <= 2 * (size_t)rs * esz;
-}
-
-cudaError_t launch_arnoldi(const CycleArgs& a, int jmax, bool defl, cudaStream_t st) {
-  switch (a.prec) {
-    case P_FP64: return Arn<double, double>::launch(a, jmax, defl, st);
-    case P_FP32: return Arn<float, float>::launch(a, jmax, defl, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
 
 }  // namespace gg

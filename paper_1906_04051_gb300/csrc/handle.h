@@ -201,7 +201,8 @@ inline Ctl make_ctl(gmres_s* h) {
   c.y = d; d += ldh + 1;
   c.sigma = d; d += ldh + 1;
   c.h = d; d += ldh + 1;
-  c.coef = d;
+  c.coef = d; d += ldh + 1;
+  c.vexp = reinterpret_cast<int*>(d);
   Meta* m = h->meta.as<Meta>();
   c.scal = m->scal;
   c.counts = m->counts;

@@ -111,6 +111,7 @@ struct CycleArgs {
   int pdl;               // step kernels with programmatic dependent launch
   int ortho;             // gmres_ortho
   int dot_arith;         // gmres_dot_arith (the fused FP64 step's multi-dot)
+  int fixv;              // the cycle leaves its basis columns in fixed point (fixed.cuh)
   unsigned* gbar;        // grid barrier words of the MGS and fused kernels (4 words)
 };
 
@@ -128,7 +129,7 @@ enum Phase {
   PH_PROJ_FINAL,    // projector: x = xh + U T^-1 U^T (b - A xh)
   PH_ADAPT,         // adaptive deflation: update of U, A U, T, T^-1 after a cycle
   PH_MGS,           // modified Gram-Schmidt step (one cooperative kernel)
-  PH_ARNOLDI,       // the Arnoldi steps of a cycle in one persistent kernel (fused.cu)
+  PH_ARNOLDI,       // the Arnoldi steps of a cycle in one persistent kernel (fused.cuh)
   PH_COUNT
 };
 // c = M^T x over ncols FP64 columns of M (leading dimension ldm), pipelined multi-dot with
@@ -137,9 +138,11 @@ cudaError_t launch_udots(const CycleArgs& a, const double* M, long long ldm, int
                          const double* x, DotEpi epi, cudaStream_t st);
 cudaError_t launch_phase(const CycleArgs& a, int ph, int j, bool defl, double* x,
                          const double* b, cudaStream_t st, int* launches);
-// fused.cu: SpMV, one-reduction MGS projections, ||w|| and the rotations of step j in one
-// cooperative kernel (diagonal storage, EBP deflation or none, FP64 or FP32)
+// fused_*.cu: the steps of a restart cycle (SpMV, CGS2 or one-reduction MGS, ||w||, rotations) in
+// one cooperative kernel (EBP deflation or none)
 bool arnoldi_fusable(const CycleArgs& a);
+// whether that kernel leaves the basis columns of the cycle's steps in fixed point
+bool arnoldi_fixed(const CycleArgs& a);
 // one launch runs the jmax steps of a restart cycle (fewer when the cycle ends early)
 cudaError_t launch_arnoldi(const CycleArgs& a, int jmax, bool defl, cudaStream_t st);
 // Control-block initialisation for a new solve.

@@ -105,8 +105,9 @@ gmres_status run(gmres_s* h, OpHost& o, const double* b, const double* x0, int m
   const bool ada = h->opts.deflation_mode == GMRES_DEFL_ADAPTIVE;  // U grows from empty
   const bool dw = h->dense_r > 0;  // U from the caller's dense columns, fixed
   if (ada) h->aq = 0;
-  // the whole step in one persistent kernel where it applies (fused.cu)
+  // the whole step in one persistent kernel where it applies (fused.cuh)
   const bool fused = !mgs && !ada && !dw && arnoldi_fusable(a);
+  a.fixv = fused && arnoldi_fixed(a) ? 1 : 0;
   if (fused) CK(h, cudaMemsetAsync(h->gbar.p, 0, 4 * sizeof(unsigned), st));
   const int mu_mode = h->opts.mu_mode;
   double mu = 0.0;
@@ -286,8 +287,11 @@ gmres_status run_noalloc(gmres_s* h, OpHost& o, const double* b, const double* x
   CK(h, noalloc_scratch(&base));
   cudaStream_t st = h->stream;
   // everything that must start at zero (the previous call's contents are otherwise kept):
-  // ticket counters, and the basis and working vector, whose padding rows past n are read
-  CK(h, cudaMemsetAsync(base + oTick, 0, sizeof(unsigned) * (1 + kMaxGroups), st));
+  // ticket counters with the grid barrier words behind them (in the same 512-byte piece), and
+  // the basis and working vector, whose padding rows past n are read
+  constexpr size_t kTickBytes = sizeof(unsigned) * (1 + kMaxGroups), kBarAt = 320;
+  static_assert(kTickBytes <= kBarAt && kTickBytes > 256 && kBarAt + 16 <= 512, "one piece");
+  CK(h, cudaMemsetAsync(base + oTick, 0, kBarAt + 4 * sizeof(unsigned), st));
   CK(h, cudaMemsetAsync(base + oV, 0, oW + sizeof(double) * (size_t)ldv - oV, st));
   const size_t nb = sizeof(double) * (size_t)h->n;
   if (x != x0) {
@@ -306,7 +310,8 @@ gmres_status run_noalloc(gmres_s* h, OpHost& o, const double* b, const double* x
   c.y = d; d += m + 1;
   c.sigma = d; d += m + 1;
   c.h = d; d += m + 1;
-  c.coef = d;
+  c.coef = d; d += m + 1;
+  c.vexp = reinterpret_cast<int*>(d);
   Meta* meta = reinterpret_cast<Meta*>(base + oMeta);
   c.scal = meta->scal;
   c.counts = meta->counts;
@@ -330,6 +335,9 @@ gmres_status run_noalloc(gmres_s* h, OpHost& o, const double* b, const double* x
   a.grid_small = h->r > 0 ? grid_for(h->r, 8, h->sms) : 1;
   a.pdl = h->prof_on ? 0 : 1;  // per-phase events would serialise the launches anyway
   a.proj = (h->r > 0 && h->opts.deflation_mode == GMRES_DEFL_PROJECTOR) ? 1 : 0;
+  a.gbar = reinterpret_cast<unsigned*>(base + oTick + kBarAt);
+  const bool fused = arnoldi_fusable(a);
+  a.fixv = fused && arnoldi_fixed(a) ? 1 : 0;
 
   const bool ebp = h->r > 0 && h->opts.deflation_mode == GMRES_DEFL_EBP;
   const int mu_mode = h->opts.mu_mode;
@@ -358,7 +366,8 @@ gmres_status run_noalloc(gmres_s* h, OpHost& o, const double* b, const double* x
     if (defl_cycle) CK(h, launch_phase(a, PH_DEFL, 0, true, x, b, st, nullptr));
     const long long left = maxit - hm.counts[C_STEPS];
     const int jmax = (int)(left < m ? left : m);
-    for (int j = 0; j < jmax; ++j) {
+    if (fused && jmax > 0) CK(h, launch_phase(a, PH_ARNOLDI, jmax, defl_cycle, x, b, st, nullptr));
+    for (int j = 0; j < (fused ? 0 : jmax); ++j) {
       CK(h, launch_phase(a, PH_SPMV, j, defl_cycle, x, b, st, nullptr));
       CK(h, launch_phase(a, PH_DOT1, j, defl_cycle, x, b, st, nullptr));
       CK(h, launch_phase(a, PH_UPD1DOT2, j, defl_cycle, x, b, st, nullptr));

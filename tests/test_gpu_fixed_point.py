@@ -46,6 +46,45 @@ def test_power_of_two_scaling_is_exact(G, orc, shift):
     assert torch.equal(x1, torch.ldexp(x2, torch.tensor(-shift, device=x2.device)))
 
 
+# the fused CGS2 cycles: both update passes over a converted basis, operators in diagonals and in
+# CSR (short and long rows), every basis precision, row counts at the edges of units and chunks
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("n,kind", [(3, "dia"), (15, "dia"), (100, "dia"), (15, "csr"),
+                                    (100, "csr"), (2, "long"), (6, "long")])
+def test_fused_cgs2_matches_oracle(G, orc, n, kind, prec):
+    if kind == "long":
+        A, b = orc.q2_bratu_assemble(n, 3.0, np.zeros((2 * n + 1) ** 3))
+        agg = (np.arange(A.n) // max(1, A.n // 3)).clip(max=2).astype(np.int32)
+        r = 3
+    else:
+        p = W.convdiff(n, pe=20.0, sigma=0.5, seed=40 + n, px=2, py=1)
+        A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+        agg, r = p.agg, p.r
+        if kind == "csr":  # a symmetric permutation leaves no diagonals
+            perm = np.random.default_rng(n).permutation(A.n)
+            inv = np.argsort(perm)
+            rows = [sorted(zip(inv[A.col[A.rowptr[i]:A.rowptr[i + 1]]],
+                               A.val[A.rowptr[i]:A.rowptr[i + 1]])) for i in perm]
+            A = orc.CSR(np.cumsum([0] + [len(q) for q in rows]),
+                        np.array([c for q in rows for c, _ in q]),
+                        np.array([v for q in rows for _, v in q]))
+            b, agg = b[perm], agg[perm]
+    steps = min(24, max(1, A.n // 3))
+    kw = dict(mu_mode=1, mu_user=4.0)
+    if prec == 0:
+        s = gpu_solver_from_oracle(G, A, agg, r, fixed_iterations=True, **kw)
+        xg, ig = s.solve(to_dev(b), m=10, tol=0.0, maxit=steps)
+        xo, _ = orc.gmres(A, b, defl=orc.Deflation(A, agg, r), m=10, tol=0.0, maxit=steps,
+                          fixed_iterations=True, **kw)
+        assert ig["iters"] == steps
+        assert relerr(xg.cpu().numpy(), xo) <= 1e-9
+    else:  # FP32 and BF16 inner cycles, refined: the true residual
+        s = gpu_solver_from_oracle(G, A, agg, r, precision=prec, **kw)
+        xg, ig = s.solve(to_dev(b), m=20, tol=1e-10, maxit=20000)
+        assert ig["status"] == 0
+        assert np.linalg.norm(b - A.matvec(xg.cpu().numpy())) <= 1.01e-10 * np.linalg.norm(b)
+
+
 def test_wide_range_of_entries(G, orc):
     """Right-hand side entries over 60 binary orders, one block of rows far below the rest."""
     p = W.convdiff(120, pe=5.0, sigma=0.5, seed=12, px=1, py=1)
