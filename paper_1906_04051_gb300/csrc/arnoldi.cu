@@ -18,6 +18,8 @@
 // true residual r = b - A x in FP64 (Eq. 15), which also starts the next cycle.
 //
 // All floating-point reductions are formed in a fixed order (deterministic).
+#include <cooperative_groups.h>
+
 #include <utility>
 
 #include "fixed.cuh"
@@ -971,16 +973,100 @@ __global__ void __launch_bounds__(kSpmvRows)
 }
 
 // --------------------------------------------------------------------------------------
-// |mu| from the Ritz values of H_k (Sec. 3.3): eigenvalues of the k x k Hessenberg matrix
-// by the Francis double-shift QR iteration, one warp; lanes share the row and column
-// updates of each reflector.
+// |mu| from the Ritz values of H_k (Sec. 3.3): the spectral radius of the k x k Hessenberg matrix
+// by repeated squaring, rho = lim ||H^m||^(1/m) (Gelfand).  With N_0 = H, e_i the exponent of
+// N_i's largest entry and N_{i+1} = (N_i 2^-e_i)^2, log2 rho = sum_i e_i 2^-i: after p squarings
+// the rest is log2 ||.|| 2^-p, below the rounding of the sum at p = 56 for any matrix of order
+// 64, real or complex dominant eigenvalue, simple or not.  A rounding error of squaring i enters
+// log rho halved i times over, so the result is as accurate as an eigenvalue from the QR
+// algorithm (backward error times the eigenvalue's condition number).
+// The Francis QR iteration in one warp this replaces is a chain of some 10^5 dependent FP64
+// operations (4.2 ms at k = 50); here a cluster of 8 blocks shares the rows of each square, every
+// block keeping the whole matrix in shared memory (0.41 ms at k = 50).
 // --------------------------------------------------------------------------------------
-__global__ void k_ritz(Ctl ctl) {
-  __shared__ double A[kMaxM * kMaxM];
-  __shared__ double smod;
-  __shared__ int sfail;
-  if (ctl.flags[F_STOP]) return;
-  ritz_warp(ctl, A, smod, sfail);
+constexpr int kRitzCluster = 8;
+constexpr int kRitzThreads = 512;                      // 8 rows x 64 columns
+constexpr int kRitzSquarings = 56;
+constexpr int kRitzRows = kMaxM / kRitzCluster;
+constexpr size_t kRitzSmem = 2 * kMaxM * kMaxM * sizeof(double);
+
+__global__ void __cluster_dims__(kRitzCluster, 1, 1) __launch_bounds__(kRitzThreads)
+    k_ritz(Ctl ctl) {
+  extern __shared__ __align__(16) double sN[];  // two copies, alternating
+  __shared__ int smax[kRitzThreads / 32];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  if (ctl.flags[F_STOP]) return;  // the same in every block
+  const int n = ctl.flags[F_K];
+  if (n <= 0) return;
+  const int t = threadIdx.x, rank = (int)cl.block_rank(), ldh = ctl.ldh;
+  // the Hessenberg block as built; entries below the subdiagonal are never written, so they
+  // are taken as the zeros they are (not read from memory)
+  for (int q = t; q < kMaxM * kMaxM; q += kRitzThreads) {
+    const int i = q / kMaxM, c = q % kMaxM;
+    sN[q] = (i < n && c < n && i <= c + 1) ? ctl.Hr[(size_t)i * ldh + c] : 0.0;
+    sN[kMaxM * kMaxM + q] = 0.0;
+  }
+  cl.sync();  // (no block writes into another's copies before it is ready)
+  const int rows = (n + kRitzCluster - 1) / kRitzCluster;  // rows of this block: rank * rows ..
+  const int j = t % kMaxM, i = rank * rows + t / kMaxM;
+  const bool live = t / kMaxM < rows && i < n && (j & ~31) < n;
+  double s = 0.0, w = 1.0;
+  int e0 = 0;
+  bool ok = true;
+  for (int p = 0; p <= kRitzSquarings; ++p) {
+    const double* N = sN + (p & 1) * (kMaxM * kMaxM);
+    // the largest exponent (the high words order like the magnitudes)
+    int m = 0;
+    for (int q = t; q < n * kMaxM; q += kRitzThreads) m = max(m, __double2hiint(N[q]) & 0x7fffffff);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((t & 31) == 0) smax[t >> 5] = m;
+    __syncthreads();
+    m = smax[t & (kRitzThreads / 32 - 1)];
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((m >> 20) == 0 || (m >> 20) == 2047) {  // zero (nilpotent H) or not finite
+      ok = false;
+      break;  // the same in every block: all hold the same matrix
+    }
+    const int e = (m >> 20) - 1023;
+    if (p == 0) e0 = e;  // kept apart: the fraction then keeps all its bits
+    else s += w * e;
+    w *= 0.5;
+    if (p == kRitzSquarings) break;
+    // scaled in place where the exponent is large (N_0's may be anything), else with the product
+    const bool now = p == 0 || e < -16 || e > 16;
+    if (now) {
+      double* Np = sN + (p & 1) * (kMaxM * kMaxM);
+      for (int q = t; q < n * kMaxM; q += kRitzThreads) Np[q] = ldexp(Np[q], -e);
+      __syncthreads();
+    }
+    const double sc = now ? 1.0 : __hiloint2double((1023 - 2 * e) << 20, 0);
+    if (live) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+      const double* row = N + i * kMaxM;
+      int c = 0;
+      for (; c + 3 < n; c += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = fma(row[c + u], N[(c + u) * kMaxM + j], a[u]);
+      for (; c < n; ++c) a[0] = fma(row[c], N[c * kMaxM + j], a[0]);
+      const double v = ((a[0] + a[1]) + (a[2] + a[3])) * sc;
+      double* out = sN + ((p + 1) & 1) * (kMaxM * kMaxM) + i * kMaxM + j;
+      if (j < n)
+#pragma unroll
+        for (int b = 0; b < kRitzCluster; ++b) *cl.map_shared_rank(out, b) = v;
+    }
+    cl.sync();
+  }
+  cl.sync();  // no block leaves while another may still write to it
+  if (rank == 0 && t == 0) {
+    const double mu = ok ? ldexp(exp2(s), e0) : 0.0;
+    if (!(mu > 0.0) || !isfinite(mu)) {
+      ctl.flags[F_STATUS] = GMRES_ERR_SINGULAR_COARSE;
+      ctl.flags[F_STOP] = 1;
+    } else {
+      ctl.scal[S_MU] = mu;
+    }
+  }
 }
 
 __global__ void k_init(Ctl ctl, double tol, double inner_tol, double r0ref, double mu,
@@ -1315,7 +1401,7 @@ struct Kern {
         break;
       }
       case PH_RITZ:
-        k_ritz<<<1, 32, 0, st>>>(a.ctl);
+        k_ritz<<<kRitzCluster, kRitzThreads, kRitzSmem, st>>>(a.ctl);
         nl = 1;
         break;
       case PH_ARNOLDI: {  // the steps of a cycle in one persistent kernel (fused.cuh; j = steps)
@@ -1362,7 +1448,9 @@ using K16 = Kern<__nv_bfloat16, float, float>;
 
 static cudaError_t prepare_all() {
   static cudaError_t once = [] {
-    cudaError_t e = K64::prepare();
+    cudaError_t e = cudaFuncSetAttribute(k_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kRitzSmem);
+    if (e == cudaSuccess) e = K64::prepare();
     if (e == cudaSuccess) e = K32::prepare();
     if (e == cudaSuccess) e = K16::prepare();
     return e;
