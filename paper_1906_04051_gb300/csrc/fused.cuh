@@ -599,93 +599,111 @@ __device__ __forceinline__ void arn_dia_rows(TACC (&acc)[B], long long row0, lon
   }
 }
 
-// Multi-dot in row-chunk order (FP32 basis): warp w takes the chunks w, w + 16, ... of the
-// super-tile and, per unit, a group of up to G columns at one chunk: one 16-byte load per
-// column and lane for the same rows, so the loads in flight of a warp fall in one row window
-// of many columns (on GB300 this streams about twice as fast as a warp reading one column
-// through many consecutive chunks).  Units run group by group, the warp's chunks in order,
-// and the next unit's G loads are issued before the current one is consumed (two units in
-// flight).  At a group's last chunk the lanes' partial sums of each column are added by a
-// shuffle tree and lane 0 accumulates them into wsum[set][warp][c].  (G = 6 with two units
-// in flight: measured on q1-n1024, 20 us at k = 26 against 21 for 10 columns, one unit at a
-// time; 8 columns do not fit the register budget, nor 6 beside the run-time diagonal count
-// of the general banded instantiation, which takes 5.)
+// warps that share a chunk in every block of the system: 16 / the most chunks of a block
+template <typename TV, typename TACC>
+__device__ __forceinline__ int arn_share(const ArnArgs<TV, TACC>& a, int G) {
+  constexpr int per = kArnUnit / (32 * ArnVec<TV>::n);  // chunks per unit
+  const int most = ((a.units + G - 1) / G) * per;
+  return most < kArnWarps ? kArnWarps / most : 1;
+}
+
+// Multi-dot in row-chunk order (FP32 or BF16 basis): per unit, a warp takes a group of up to G
+// columns at one chunk: one 16-byte (BF16: 8-byte) load per column and lane for the same rows, so
+// the loads in flight of a warp fall in one row window of many columns (on GB300 this streams
+// about twice as fast as a warp reading one column through many consecutive chunks).  Units run
+// group by group, the warp's chunks in order, two units in flight, each value's register reloaded
+// as it is used.  S warps share a chunk's groups where the blocks have few chunks (arn_split32).
+// At a group's last chunk the lanes' partial sums of each column are added by a shuffle tree and
+// lane 0 accumulates them into wsum[set][first chunk][c].
 template <int ND> constexpr int arn_group() { return ND == 9 ? 6 : 5; }
+
+// S: warps per chunk, the same in every block of the system (so that equal rows are summed in the
+// same order everywhere): 16 / the most chunks a block holds, at least 1
+__device__ __forceinline__ ArnSplit arn_split32(int S, int nch) {
+  const int warp = threadIdx.x >> 5;
+  if (S <= 1) return ArnSplit{1, warp, 0, kArnWarps, warp < nch};
+  const int w = kArnWarps / S;  // chunk places
+  return ArnSplit{S, warp % w, warp / w, w, warp / w < S && warp % w < nch};
+}
 
 template <typename TV, typename TACC, int NSET, int G>
 __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long long ldv, int k,
-                                              long long s0, int nch, const TACC* Ws,
-                                              const TACC* Us, int warp, int lane) {
-  constexpr int VN = ArnVec<TV>::n;
-  const int nqw = warp < nch ? (nch - 1 - warp) / kArnWarps + 1 : 0;  // chunks of this warp
-  const int ng = (k + G - 1) / G;
-  const int TU = ng * nqw;
-  if (TU == 0) return;
-  TACC a1[G], a2[G];
-#pragma unroll
-  for (int u = 0; u < G; ++u) {
-    a1[u] = 0;
-    a2[u] = 0;
-  }
-  auto load_unit = [&](int un, TACC (&b)[G][VN]) {
-    const int g = un / nqw, qi = un - g * nqw;
-    const int g0 = g * G;
-    const int gc = k - g0 < G ? k - g0 : G;
-    const TV* col = V + (size_t)g0 * ldv + s0 + (size_t)lane * VN +
-                    (size_t)(warp + qi * kArnWarps) * 32 * VN;
-#pragma unroll
-    for (int u = 0; u < G; ++u)
-      if (u < gc) arn_ldg<TV, TACC, VN>(col + (size_t)u * ldv, b[u]);
-  };
-  auto consume = [&](int un, const TACC (&b)[G][VN]) {
-    const int g = un / nqw, qi = un - g * nqw;
-    const int g0 = g * G;
-    const int gc = k - g0 < G ? k - g0 : G;
-    const size_t off = (size_t)(warp + qi * kArnWarps) * 32 * VN;
-    TACC wv[VN], uv[VN];
-    ld_acc<VN>(Ws + off + lane * VN, wv);
-    if (NSET == 2) ld_acc<VN>(Us + off + lane * VN, uv);
-#pragma unroll
-    for (int u = 0; u < G; ++u)
-      if (u < gc)
-#pragma unroll
-        for (int e = 0; e < VN; ++e) {
-          a1[u] += b[u][e] * wv[e];
-          if (NSET == 2) a2[u] += b[u][e] * uv[e];
-        }
-    if (qi == nqw - 1) {  // the group's last chunk in this warp
-#pragma unroll
-      for (int u = 0; u < G; ++u) {
-        if (u < gc) {
-          const TACC t1 = warp_sum(a1[u]);
-          if (lane == 0) {
-            float2* p1 = reinterpret_cast<float2*>(wsum) + (size_t)warp * kMaxK + g0 + u;
-            float2 a1v = *p1;
-            arn_df_add(a1v.x, a1v.y, (float)t1, 0.f);
-            *p1 = a1v;
-          }
-          if (NSET == 2) {
-            const TACC t2 = warp_sum(a2[u]);
-            if (lane == 0) {
-              float2* p2 = reinterpret_cast<float2*>(wsum) + (size_t)(kArnWarps + warp) * kMaxK + g0 + u;
-              float2 a2v = *p2;
-              arn_df_add(a2v.x, a2v.y, (float)t2, 0.f);
-              *p2 = a2v;
-            }
-          }
-        }
-        a1[u] = 0;
-        a2[u] = 0;
-      }
+                                              long long s0, int nch, int S, const TACC* Ws,
+                                              const TACC* Us, int lane) {
+  constexpr int VN = ArnVec<TV>::n, D = 2;
+  const ArnSplit sp = arn_split32(S, nch);
+  if (!sp.live) return;
+  const int nqw = S > 1 ? 1 : (nch - 1 - sp.q0) / kArnWarps + 1;  // chunks of this warp
+  const long long step = (long long)kArnWarps * 32 * VN;
+  const TV* const base = V + s0 + (size_t)sp.q0 * 32 * VN + (size_t)lane * VN;
+  int ln = 0, gn = sp.p * G;
+  const TV* pn = base + (size_t)gn * ldv;
+  auto advance = [&] {
+    pn += step;
+    if (++ln == nqw) {
+      ln = 0;
+      gn += G * sp.S;
+      pn = base + (size_t)gn * ldv;
     }
   };
-  TACC bA[G][VN], bB[G][VN];
-  load_unit(0, bA);
-  for (int un = 0; un < TU; un += 2) {
-    if (un + 1 < TU) load_unit(un + 1, bB);
-    consume(un, bA);
-    if (un + 2 < TU) load_unit(un + 2, bA);
-    if (un + 1 < TU) consume(un + 1, bB);
+  TACC b[D][G][VN];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+#pragma unroll
+      for (int e = 0; e < VN; ++e) b[d][u][e] = 0;
+      if (gn + u < k) arn_ldg<TV, TACC, VN>(pn + (size_t)u * ldv, b[d][u]);
+    }
+    advance();
+  }
+  TACC acc[NSET][G];
+#pragma unroll
+  for (int u = 0; u < G; ++u)
+#pragma unroll
+    for (int t = 0; t < NSET; ++t) acc[t][u] = 0;
+  int g0 = sp.p * G, qi = 0;
+  const int at = (sp.q0 * 32 + lane) * VN;
+#pragma unroll 1
+  while (g0 < k) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      if (g0 >= k) break;
+      TACC wv[VN], uv[VN];
+      ld_acc<VN>(Ws + at + qi * step, wv);
+      if (NSET == 2) ld_acc<VN>(Us + at + qi * step, uv);
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        if (g0 + u < k)
+#pragma unroll
+          for (int e = 0; e < VN; ++e) {
+            acc[0][u] += b[d][u][e] * wv[e];
+            if (NSET == 2) acc[NSET - 1][u] += b[d][u][e] * uv[e];
+          }
+        if (gn + u < k) arn_ldg<TV, TACC, VN>(pn + (size_t)u * ldv, b[d][u]);
+      }
+      advance();
+      if (++qi == nqw) {  // the group's last chunk in this warp
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+#pragma unroll
+          for (int t = 0; t < NSET; ++t) {
+            if (g0 + u < k) {
+              const TACC v = warp_sum(acc[t][u]);
+              if (lane == 0) {
+                float2* pw = reinterpret_cast<float2*>(wsum) +
+                             (size_t)(t * kArnWarps + sp.q0) * kMaxK + g0 + u;
+                float2 o = *pw;
+                arn_df_add(o.x, o.y, (float)v, 0.f);
+                *pw = o;
+              }
+            }
+            acc[t][u] = 0;
+          }
+        qi = 0;
+        g0 += G * sp.S;
+      }
+    }
   }
 }
 
@@ -979,7 +997,8 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
       __syncthreads();
       arn_slot_sums<NSET>(slot, nch, k, sE, ew, eu, tile == 0, sred);
     } else {
-      arn_dots_rows<TV, TACC, NSET, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, Ws, Us, warp, lane);
+      arn_dots_rows<TV, TACC, NSET, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, arn_share(a, G),
+                                                     Ws, Us, lane);
     }
     __syncthreads();  // the slices are rewritten by the next super-tile
   }
@@ -1183,56 +1202,42 @@ __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, dou
 template <typename TV, typename TACC, bool PASS2>
 __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
                                           const TACC* scoef, TACC* ush, long long base,
-                                          long long end) {
+                                          long long end, float* sP) {
   constexpr int VN = ArnVec<TV>::n;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int U = PASS2 ? 6 : 8;  // basis loads in flight per lane, reloaded as they are used
+  constexpr int chunk = 32 * VN;
+  const int lane = threadIdx.x & 31;
   const int G = gridDim.x, bid = blockIdx.x;
   const long long R0 = (long long)bid * a.units / G * kArnUnit;
   const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
   const long long N = a.N;
   TV* __restrict__ vout = const_cast<TV*>(a.V) + (size_t)k * a.ldv;
   float ns = 0.f, nc = 0.f;  // a double-FP32 pair (FP64 adds are dear)
-  {
-    constexpr int U = PASS2 ? 4 : 8;  // basis loads in flight per lane
-    const int chunk = 32 * VN;
-    const long long nch = (end - base) / chunk;
-    const bool wsm = R1 - R0 <= a.RS;  // the block's w is still in shared memory
-    for (long long q = nch - 1 - warp; q >= 0; q -= kArnWarps) {
-      const long long r = base + q * chunk + (long long)lane * VN;
-      TACC wv[VN], p[VN];
+  const int nch = (int)((end - base) / chunk);
+  const bool wsm = R1 - R0 <= a.RS;  // the block's w is still in shared memory
+  const ArnSplit sp = arn_split32(arn_share(a, G), nch);
+  const bool one = sp.S > 1;
+  const int c0 = sp.p * k / sp.S, c1 = (sp.p + 1) * k / sp.S;
+  long long r = base + (long long)(nch - 1 - sp.q0) * chunk + (long long)lane * VN;
+  TACC p[VN];
+  auto finish = [&] {
+    TACC wv[VN], un[VN];
+    if (wsm) {
+      ld_acc<VN>(Ws + (r - R0), wv);
+    } else {
+#pragma unroll
+      for (int e = 0; e < VN; ++e) wv[e] = r + e < N ? __ldcg(a.w + r + e) : (TACC)0;
+    }
+#pragma unroll
+    for (int e = 0; e < VN; ++e) un[e] = wv[e] - p[e];
+    if constexpr (PASS2) {  // CGS2's first update: w stays where it came from
       if (wsm) {
-        ld_acc<VN>(Ws + (r - R0), wv);
+        acc_store<VN>(Ws + (r - R0), un);
       } else {
-#pragma unroll
-        for (int e = 0; e < VN; ++e) wv[e] = r + e < N ? __ldcg(a.w + r + e) : (TACC)0;
+        acc_store<VN>(a.w + r, un);
+        acc_store<VN>(Ws + (r - base), un);
       }
-#pragma unroll
-      for (int e = 0; e < VN; ++e) p[e] = 0;
-      for (int c0 = 0; c0 < k; c0 += U) {
-        TACC v[U][VN];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (c0 + u < k) arn_ldg<TV, TACC, VN>(a.V + (size_t)(c0 + u) * a.ldv + r, v[u]);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (c0 + u < k) {
-            const TACC cf = scoef[c0 + u];
-#pragma unroll
-            for (int e = 0; e < VN; ++e) p[e] += v[u][e] * cf;
-          }
-      }
-      TACC un[VN];
-#pragma unroll
-      for (int e = 0; e < VN; ++e) un[e] = wv[e] - p[e];
-      if constexpr (PASS2) {  // CGS2's first update: w stays where it came from
-        if (wsm) {
-          acc_store<VN>(Ws + (r - R0), un);
-        } else {
-          acc_store<VN>(a.w + r, un);
-          acc_store<VN>(Ws + (r - base), un);
-        }
-        continue;
-      }
+    } else {
       arn_stv<TV, TACC, VN>(vout + r, un);
       if constexpr (sizeof(TV) == 2) {  // the stored (rounded) values count
 #pragma unroll
@@ -1244,7 +1249,59 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
       for (int e = 0; e < VN; ++e) s += un[e] * un[e];
       arn_df_add(ns, nc, s, 0.f);
     }
+  };
+#pragma unroll
+  for (int e = 0; e < VN; ++e) p[e] = 0;
+  if (sp.live) {
+    int nb = c0;  // column and row of the next load
+    long long nr = r;
+    TACC v[U][VN];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int e = 0; e < VN; ++e) v[u][e] = 0;
+      if (nb + u < c1) arn_ldg<TV, TACC, VN>(a.V + (size_t)(nb + u) * a.ldv + nr, v[u]);
+    }
+    for (; r >= base; r -= (long long)kArnWarps * chunk) {
+#pragma unroll
+      for (int e = 0; e < VN; ++e) p[e] = 0;
+#pragma unroll 1
+      for (int b = c0; b < c1; b += U) {
+        nb += U;
+        if (nb >= c1) {  // on to the warp's next chunk
+          nb = c0;
+          nr -= (long long)kArnWarps * chunk;
+        }
+        const bool more = nr >= base && (!one || nb > c0);
+        const TV* pn = a.V + (size_t)nb * a.ldv + nr;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (b + u < c1) {
+            const TACC cf = scoef[b + u];
+#pragma unroll
+            for (int e = 0; e < VN; ++e) p[e] += v[u][e] * cf;
+          }
+          if (more && nb + u < c1) arn_ldg<TV, TACC, VN>(pn + (size_t)u * a.ldv, v[u]);
+        }
+      }
+      if (one) break;
+      finish();
+    }
   }
+  if (one) {  // the shares' partial sums, added in order
+    if (sp.live && sp.p > 0) acc_store<VN>(sP + ((size_t)((sp.p - 1) * sp.rows + sp.q0) * 32 + lane) * VN, p);
+    __syncthreads();
+    if (sp.live && sp.p == 0) {
+      for (int q = 1; q < sp.S; ++q) {
+        TACC o[VN];
+        ld_acc<VN>(sP + ((size_t)((q - 1) * sp.rows + sp.q0) * 32 + lane) * VN, o);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) p[e] += o[e];
+      }
+      finish();
+    }
+  }
+  if constexpr (PASS2) return 0.0;
   // the warp's total in double-FP32, rounded once
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -1256,26 +1313,28 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
 }
 
 // CGS2, first update and second multi-dot of an FP32 or BF16 basis: per super-tile (from the last)
-// w -= V (sigma o h), then V^T w into the per-warp pairs.  A call of its own: inlined, the two
-// loops' registers spilled (240 to 690 bytes a thread).
+// w -= V (sigma o h), then V^T w into the per-warp pairs
 template <typename TV, typename TACC, int ND>
-__device__ __noinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
+__device__ __forceinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
                                             const TACC* scoef, double* sbuf) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = gridDim.x, bid = blockIdx.x;
   const long long R0 = (long long)bid * a.units / G * kArnUnit;
   const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
-  for (int q = threadIdx.x; q < kMaxK * kArnWarps; q += kArnThreads) sbuf[q] = 0.0;
   const int tiles = (int)((R1 - R0 + a.RS - 1) / a.RS);
   for (int tile = tiles - 1; tile >= 0; --tile) {
     const long long s0 = R0 + (long long)tile * a.RS;
     const long long s1 = s0 + a.RS < R1 ? s0 + a.RS : R1;
     __syncthreads();
-    arn_update<TV, TACC, true>(a, k, Ws, scoef, nullptr, s0, s1);
+    arn_update<TV, TACC, true>(a, k, Ws, scoef, nullptr, s0, s1, reinterpret_cast<float*>(sbuf));
     __syncthreads();
+    if (tile == tiles - 1) {  // (the shares of a chunk, one super-tile only, used sbuf)
+      for (int q = threadIdx.x; q < kMaxK * kArnWarps; q += kArnThreads) sbuf[q] = 0.0;
+      __syncthreads();
+    }
     arn_dots_rows<TV, TACC, 1, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0,
-                                                (int)((s1 - s0) / (32 * ArnVec<TV>::n)), Ws,
-                                                nullptr, warp, lane);
+                                                (int)((s1 - s0) / (32 * ArnVec<TV>::n)),
+                                                arn_share(a, G), Ws, nullptr, lane);
   }
   __syncthreads();
 }
@@ -1662,7 +1721,8 @@ __global__ void __launch_bounds__(kArnThreads, 1)
           a.V, a.ldv, vout, a.w, R0, R1, MODE == kArnLowsync ? k - 1 : k, k, scoef, sE, sbuf,
           &sscale, ush, mx);
     else
-      nrm = arn_update<TV, TACC, false>(a, k, Ws, scoef, ush, R0, R1);
+      nrm = arn_update<TV, TACC, false>(a, k, Ws, scoef, ush, R0, R1,
+                                          reinterpret_cast<float*>(sbuf));
     // ---- 5. norm partial; partial sums of u_{j+1} over this block's aggregate pieces ----
     {
       // the warp sums (formed by the update), then warp 0 adds the 16 of them (a block-wide
