@@ -1,23 +1,30 @@
 // batch.cu -- many independent deflated GMRES(m) solves in one CUDA-graph launch.
 //
-// Every phase kernel runs over a flattened list of row tiles drawn from all systems, so
-// each launch spreads every system's work over all SMs (on GB300 one SM retires only two
-// FP64 FMAs per clock: a system of 66k unknowns cannot be left to one SM).  Block b owns
-// the contiguous tile range [b T / G, (b+1) T / G); it accumulates a system's partial sums
-// over its tiles of that system and, when the system changes, stores them in the
-// system's slot b - (first block touching the system).  The last block to fill a
-// system's slots (per-system ticket) reduces them in slot order and runs the system's
-// epilogue (projection coefficients, plane rotations, restart decision), so results are
-// deterministic and no block waits on another.
+// The steps of a restart cycle run in the fused step kernel (fused.cuh), one thread-block cluster
+// per running system: the two or three barriers of a step are then cluster barriers among a few
+// blocks, systems do not wait for each other inside a cycle, and the step's launches (six to
+// eight, over all systems) are gone.  Batches it does not cover (a system of more than kClusterRows
+// rows, operators of different forms, an option without a fused step) run the steps as phase
+// kernels.  The rest of a cycle (x update, corrections, residual, restart decision) is phase
+// kernels in either case.
 //
-// All systems advance in lock step through restart cycles; a system that converged or
-// ended its cycle early is skipped by every tile of it.  The cycle's kernel sequence is
-// captured once into the body of a conditional `while` graph node, and a last kernel sets
-// the loop condition (any system still running), so the whole solve is one graph launch.
+// A phase kernel runs over a flattened list of row tiles drawn from all systems, so each launch
+// spreads every system's work over all SMs.  Block b owns the contiguous tile range
+// [b T / G, (b+1) T / G); it accumulates a system's partial sums over its tiles of that system
+// and, when the system changes, stores them in the system's slot b - (first block touching the
+// system).  The last block to fill a system's slots (per-system ticket) reduces them in slot
+// order and runs the system's epilogue (projection coefficients, plane rotations, restart
+// decision), so results are deterministic and no block waits on another.
+//
+// All systems advance in lock step through restart cycles; a system that converged is left out
+// (its tiles are skipped, kb_list gives it no cluster).  The cycle's kernel sequence is captured
+// once into the body of a conditional `while` graph node, and a last kernel sets the loop
+// condition (any system still running), so the whole solve is one graph launch.
 #include <algorithm>
 #include <map>
 #include <memory>
 
+#include "fixed.cuh"
 #include "handle.h"
 #include "kernels.cuh"
 
@@ -530,19 +537,19 @@ __global__ void __launch_bounds__(kThreads) kb_pass3(BTab tab, int k) {
 }
 
 // ---- deflation: U^T x per system (warp per piece), then the coarse correction ----------
-// mode 0: x = basis column j of a system in its cycle, scale sigma_j;
-// mode 1: x = t of a live system at the cycle end, scale 1.
+// mode 0: x = basis column j of a system in its cycle, scale sigma_j (mode 2: scale 1, the fused
+// cycle's form); mode 1: x = t of a live system at the cycle end, scale 1.
 template <typename TV>
 __global__ void __launch_bounds__(kThreads) kb_aggsum(BTab tab, int j, int mode) {
   const int lane = threadIdx.x & 31;
   const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (p >= tab.P) return;
   const BSys& S = tab.sys[tab.piece_sys[p]];
-  if (!S.ctl.flags[F_DEFL_ON] || (mode == 0 ? !sys_step_active(S) : !sys_live(S))) return;
+  if (!S.ctl.flags[F_DEFL_ON] || (mode != 1 ? !sys_step_active(S) : !sys_live(S))) return;
   const int lp = p - S.piece0;
   const int s = S.defl.piece_start[lp], e = S.defl.piece_start[lp + 1];
   double acc = 0.0;
-  if (mode == 0) {
+  if (mode != 1) {
     const TV* x = static_cast<const TV*>(S.V) + (size_t)j * S.ldv;
     for (int q = s + lane; q < e; q += 32) acc += ld_as<double, TV>(x + S.defl.perm[q]);
   } else {
@@ -555,7 +562,7 @@ __global__ void __launch_bounds__(kThreads) kb_aggsum(BTab tab, int j, int mode)
 __global__ void __launch_bounds__(kThreads) kb_coarse(BTab tab, int j, int mode) {
   extern __shared__ double sc[];
   const BSys& S = tab.sys[blockIdx.x];
-  if (!S.ebp || !S.ctl.flags[F_DEFL_ON] || (mode == 0 ? !sys_step_active(S) : !sys_live(S)))
+  if (!S.ebp || !S.ctl.flags[F_DEFL_ON] || (mode != 1 ? !sys_step_active(S) : !sys_live(S)))
     return;
   const Defl& d = S.defl;
   const double scale = mode == 0 ? S.ctl.sigma[j] : 1.0;
@@ -622,6 +629,38 @@ __global__ void __launch_bounds__(kThreads) kb_xupdate(BTab tab) {
   }
 }
 
+// the same from bases in fixed point (fixed.cuh)
+__global__ void __launch_bounds__(kThreads) kb_xupdate_fx(BTab tab) {
+  __shared__ int4 sK[kMaxK];
+  __shared__ double sscale;
+  const int T = tab.T_s;
+  const int lo = range_lo(blockIdx.x, gridDim.x, T), hi = range_lo(blockIdx.x + 1, gridDim.x, T);
+  int cur = -1;
+  for (int t = lo; t < hi; ++t) {
+    const int s = tab.tile_sys_s[t];
+    const BSys& S = tab.sys[s];
+    if (!sys_live(S)) continue;
+    const int k = S.ctl.flags[F_K];
+    if (s != cur) {
+      __syncthreads();
+      if (threadIdx.x < 32) {
+        const double sc = fx_coefs(k, S.ctl.coef, S.ctl.vexp, sK);
+        if (threadIdx.x == 0) sscale = sc;
+      }
+      __syncthreads();
+      cur = s;
+    }
+    const int row = (t - S.tile0_s) * kSpmvRows + threadIdx.x;
+    if (row >= S.n) continue;
+    const long long* V = static_cast<const long long*>(S.V) + row;
+    FxAcc a{0, 0, 0, 0};
+#pragma unroll 8
+    for (int c = 0; c < k; ++c) fx_axpy(a, fx_limbs(__ldg(V + (size_t)c * S.ldv)), sK[c]);
+    if (S.ctl.flags[F_DEFL_ON]) S.t[row] = fx_axpy_add(a, 0.0, sscale);
+    else S.x[row] = fx_axpy_add(a, S.x[row], sscale);
+  }
+}
+
 __global__ void __launch_bounds__(kThreads) kb_xapply(BTab tab) {
   const int T = tab.T_s;
   const int lo = range_lo(blockIdx.x, gridDim.x, T), hi = range_lo(blockIdx.x + 1, gridDim.x, T);
@@ -647,6 +686,30 @@ __global__ void kb_ritz(BTab tab) {
   ritz_warp(ctl, A, smod, sfail);
   __syncwarp();
   if (threadIdx.x == 0 && !ctl.flags[F_STOP]) ctl.flags[F_DEFL_ON] = 1;
+}
+
+// the systems still running, in the order given (by size): their count, then their positions
+__global__ void __launch_bounds__(256) kb_list(BTab tab, const int* __restrict__ order,
+                                               int* __restrict__ list) {
+  __shared__ int wsum[8];
+  int base = 0;
+  for (int q0 = 0; q0 < tab.count; q0 += 256) {
+    const int q = q0 + (int)threadIdx.x;
+    const bool live = q < tab.count && sys_live(tab.sys[order[q]]);
+    const unsigned bal = __ballot_sync(0xffffffffu, live);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) wsum[warp] = __popc(bal);
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) before += wsum[w];
+      all += wsum[w];
+    }
+    if (live) list[1 + base + before + __popc(bal & ((1u << lane) - 1u))] = q;
+    base += all;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) list[0] = base;
 }
 
 // loop condition of the graph: any system still running
@@ -686,20 +749,39 @@ struct BKern {
   }
   // one restart cycle of every system; returns the number of kernels enqueued, or -1
   // with *err / *where set when a launch fails
-  static int cycle(const BTab& tab, int sms, int bps_pass, int max_r, bool lowsync,
-                   cudaStream_t st, cudaError_t* err, const char** where) {
+  static int cycle(const BTab& tab, int sms, int bps_pass, int max_r, int ortho,
+                   const FusedBatch& fb, const int* fb_order, int* fb_list, cudaStream_t st,
+                   cudaError_t* err, const char** where) {
+    const bool lowsync = ortho == GMRES_ORTHO_MGS_LOWSYNC;
     const int m = tab.m;
     auto grid = [&](int T, int per_sm) { return std::max(1, std::min(T, per_sm * sms)); };
     const int gs = grid(tab.T_s, 4);
     const int gpieces = std::max(1, (tab.P + 7) / 8);
     const size_t csm = sizeof(double) * (size_t)std::max(1, max_r);
     int nl = 0;
-    kb_aggsum<TV><<<gpieces, kThreads, 0, st>>>(tab, 0, 0);
+    const int mode0 = fb.tiers ? 2 : 0;
+    kb_aggsum<TV><<<gpieces, kThreads, 0, st>>>(tab, 0, mode0);
     if ((*err = cudaGetLastError()) != cudaSuccess) { *where = "kb_aggsum"; return -1; }
-    kb_coarse<<<tab.count, kThreads, csm, st>>>(tab, 0, 0);
+    kb_coarse<<<tab.count, kThreads, csm, st>>>(tab, 0, mode0);
     if ((*err = cudaGetLastError()) != cudaSuccess) { *where = "kb_coarse"; return -1; }
     nl += 2;
-    for (int j = 0; j < m; ++j) {
+    if (fb.tiers) {
+      kb_list<<<1, 256, 0, st>>>(tab, fb_order, fb_list);
+      if ((*err = cudaGetLastError()) != cudaSuccess) { *where = "kb_list"; return -1; }
+      for (int t = 0; t < fb.tiers; ++t) {  // one of them does the work
+        const int hi = t == 0 ? tab.count : fb.upto[t];
+        const int lo = t + 1 < fb.tiers ? fb.upto[t + 1] : 0;
+        if (tab.count <= lo) continue;
+        const int nc = std::min(tab.count, hi);
+        *err = sizeof(TV) == 8   ? launch_arnoldi_batch_fp64(fb, nc, lo, hi, fb.G[t], st)
+               : sizeof(TV) == 4 ? launch_arnoldi_batch_fp32(fb, nc, lo, hi, fb.G[t], st)
+                                 : launch_arnoldi_batch_bf16(fb, nc, lo, hi, fb.G[t], st);
+        if (*err != cudaSuccess) { *where = "k_arnoldi_batch"; return -1; }
+        nl += 1;
+      }
+      nl += 1;
+    }
+    for (int j = 0; j < (fb.tiers ? 0 : m); ++j) {
       const int k = j + 1;
       const size_t rs = ring_smem(k, tab.TR);
       kb_spmv<TA, TV, TACC><<<gs, kSpmvRows, 0, st>>>(tab, j);
@@ -735,7 +817,8 @@ struct BKern {
     }
     kb_backsolve<<<tab.count, 128, 0, st>>>(tab);
     if ((*err = cudaGetLastError()) != cudaSuccess) { *where = "kb_backsolve"; return -1; }
-    kb_xupdate<TV><<<gs, kThreads, 0, st>>>(tab);
+    if (sizeof(TV) == 8 && fb.tiers) kb_xupdate_fx<<<gs, kThreads, 0, st>>>(tab);
+    else kb_xupdate<TV><<<gs, kThreads, 0, st>>>(tab);
     if ((*err = cudaGetLastError()) != cudaSuccess) { *where = "kb_xupdate"; return -1; }
     kb_aggsum<TV><<<gpieces, kThreads, 0, st>>>(tab, 0, 1);
     if ((*err = cudaGetLastError()) != cudaSuccess) { *where = "kb_aggsum"; return -1; }
@@ -757,10 +840,21 @@ struct BKern {
   }
 };
 
+// Most rows (padded) of a system that runs in a cluster.  A cluster has at most 16 of the 152 SMs,
+// so what it gains over the phase kernels shrinks as systems grow: two systems of 73,000 to 79,000
+// rows take 23.8 ms against 26.3 (FP64, 300 steps), 40 of them 92 against 132.
+constexpr long long kClusterRows = 80000;
+// Running systems above which clusters of 4 give way to clusters of 2, in waves of the former.
+// 256 systems (300 steps, FP64) take 150 ms with clusters of 2 and 168 with 4; with 64 systems,
+// under two waves of 4, the largest of them holds up a single wave of 2 (39 ms against 27).
+constexpr int kClusterWaves = 2;
+
 struct BatchCtx {
   std::vector<gmres_s*> hs;
   int m = 0, prec = 0, TR = 0, bps = 0, max_r = 0, count = 0, ortho = 0;
   BTab tab{};
+  FusedBatch fb;
+  DevMem dargs, dlist;  // dlist: systems by size (count), then the list (1 + count)
   DevMem dsys, dtile_s, dtile_p, dpiece;
   std::vector<BSys> hsys;
   cudaGraph_t graph = nullptr;
@@ -783,7 +877,7 @@ std::vector<std::unique_ptr<BatchCtx>>& batch_cache() {
 
 template <typename K>
 int run_cycle(const BatchCtx& c, int sms, cudaStream_t st, cudaError_t* err, const char** where) {
-  return K::cycle(c.tab, sms, c.bps, c.max_r, c.ortho == GMRES_ORTHO_MGS_LOWSYNC, st, err, where);
+  return K::cycle(c.tab, sms, c.bps, c.max_r, c.ortho, c.fb, c.dlist.as<int>(), c.dlist.as<int>() + c.count, st, err, where);
 }
 
 int dispatch_cycle(const BatchCtx& c, int sms, cudaStream_t st, cudaError_t* err,
@@ -849,6 +943,86 @@ cudaError_t build_tables(BatchCtx& c, cudaStream_t st) {
   c.tab.P = (int)ps.size();
   c.tab.TR = c.TR;
   c.tab.m = c.m;
+  return cudaStreamSynchronize(st);
+}
+
+// Whether the systems of the batch can run their cycles in clusters (fused.cuh), and in which
+// sizes.  While many systems run, clusters of 2 or 4 blocks (the most systems at once, the least
+// waiting inside a system); when the running systems fit the device in clusters of 8, and of 16,
+// those: the last systems of a batch are a chain of short steps.  The phase kernels took 301 ms
+// (FP64) and 209 ms (FP32) for 256 systems of 1,000 to 66,000 rows and 300 steps, clusters of 2
+// at first take 150 and 114; three systems of 23,000 to 40,000 rows take 23.4 ms, 36.7 with
+// clusters of 4 only, 22.8 with 8, 16.4 with 16.
+FusedBatch plan_fused(const BatchCtx& c) {
+  FusedBatch f, none;
+  f.nd = c.hs[0]->fwd.dia.nd;
+  f.ortho = c.ortho;
+  for (gmres_s* h : c.hs) {
+    CycleArgs a{};
+    a.op = make_op(h, h->fwd);
+    a.ldv = h->ldv;
+    a.m = c.m;
+    a.prec = c.prec;
+    a.ortho = c.ortho;
+    a.sms = h->sms;
+    if (h->opts.deflation_mode != GMRES_DEFL_EBP) a.op.defl.r = 0;
+    const bool same = h->fwd.dia.nd == f.nd ||  // one operator form for all
+                      (f.nd > 0 && f.nd != 9 && h->fwd.dia.nd > 0 && h->fwd.dia.nd != 9);
+    if (!same || h->ldv > kClusterRows || !arnoldi_fusable(a)) return none;
+  }
+  const int sizes[kBatchTiers] = {2, 4, 8, 16};
+  for (int t = 0; t < kBatchTiers; ++t) {
+    int fit = 0;
+    f.fit = &fit;
+    const cudaError_t e = c.prec == P_FP64   ? launch_arnoldi_batch_fp64(f, 0, 0, 0, sizes[t], nullptr)
+                          : c.prec == P_FP32 ? launch_arnoldi_batch_fp32(f, 0, 0, 0, sizes[t], nullptr)
+                                             : launch_arnoldi_batch_bf16(f, 0, 0, 0, sizes[t], nullptr);
+    f.fit = nullptr;
+    if (e != cudaSuccess || fit < 1) break;
+    f.G[f.tiers] = sizes[t];
+    f.upto[f.tiers++] = sizes[t] == 4 ? kClusterWaves * fit : fit;
+  }
+  return f;
+}
+
+// the kernel arguments of every system's cycles, largest first, to the device
+cudaError_t upload_args(BatchCtx& c, cudaStream_t st) {
+  auto fill = [&](const CycleArgs& a, bool defl, void* dst) {
+    return c.prec == P_FP64   ? arnoldi_args_fp64(a, defl, dst)
+           : c.prec == P_FP32 ? arnoldi_args_fp32(a, defl, dst)
+                              : arnoldi_args_bf16(a, defl, dst);
+  };
+  const size_t each = fill(CycleArgs{}, false, nullptr);
+  std::vector<int> order(c.count);
+  for (int i = 0; i < c.count; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return c.hs[x]->n > c.hs[y]->n; });
+  std::vector<unsigned char> buf(each * (size_t)c.count);
+  for (int q = 0; q < c.count; ++q) {
+    gmres_s* h = c.hs[order[q]];
+    const BSys& S = c.hsys[order[q]];
+    CycleArgs a{};
+    a.op = make_op(h, h->fwd);
+    a.ctl = S.ctl;
+    a.V = S.V;
+    a.ldv = S.ldv;
+    a.w = S.w;
+    a.t = S.t;
+    a.prec = c.prec;
+    a.m = c.m;
+    a.sms = h->sms;
+    a.ortho = c.ortho;
+    fill(a, S.ebp != 0, buf.data() + each * (size_t)q);
+  }
+  cudaError_t e = c.dargs.ensure(buf.size());
+  if (e != cudaSuccess) return e;
+  if ((e = cudaMemcpyAsync(c.dargs.p, buf.data(), buf.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+    return e;
+  c.fb.args = c.dargs.p;
+  if ((e = c.dlist.ensure(sizeof(int) * (2 * (size_t)c.count + 1))) != cudaSuccess) return e;
+  if ((e = cudaMemcpyAsync(c.dlist.p, order.data(), sizeof(int) * (size_t)c.count,
+                           cudaMemcpyHostToDevice, st)) != cudaSuccess)
+    return e;
+  c.fb.list = c.dlist.as<int>() + c.count;
   return cudaStreamSynchronize(st);
 }
 
@@ -986,6 +1160,8 @@ gmres_status batch_solve_impl(int count, gmres_t const* hs, const double* const*
   }
   ctx->max_r = max_r;
   cudaError_t e;
+  if (fresh) ctx->fb = plan_fused(*ctx);
+  if (ctx->fb.tiers && (e = upload_args(*ctx, st)) != cudaSuccess) return cuda_fail(nullptr, e, "batch arguments");
   const bool mixed = prec != P_FP64;
   const double inner_tol = prec == P_BF16 ? 1e-2 : 1e-4;
   if (fresh) {
@@ -996,13 +1172,14 @@ gmres_status batch_solve_impl(int count, gmres_t const* hs, const double* const*
       for (int bps : {4, 2})
         if (ring_stage_bytes(m + 1, tr, basis_elem(prec), prec == P_FP64 ? 8 : 4) <= 48 * 1024)
           cand.push_back({tr, bps});
+    if (ctx->fb.tiers) cand.clear();  // the tiles and grids of the phase kernels are not used
     if (cand.empty()) cand.push_back({lo, 2});
     float best = 1e30f;
     int best_i = 0;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    for (size_t ci = 0; ci < cand.size(); ++ci) {
+    for (size_t ci = 0; ci < (cand.size() > 1 ? cand.size() : 0); ++ci) {
       ctx->TR = cand[ci].first;
       ctx->bps = cand[ci].second;
       if ((e = dispatch_prepare(prec, ctx->TR, m)) != cudaSuccess) return cuda_fail(nullptr, e, "batch prepare");

@@ -79,6 +79,7 @@ template <typename TV, typename TACC>
 struct ArnArgs {
   int N;          // rows of A
   int units;      // ldv / kArnUnit
+  int fine;       // ranges of units that the aggregate pieces are cut at (ArnRows)
   int jmax, m;    // steps of this cycle (<= m), restart length
   int pre;        // the predecessor is the coarse solve of step 0: the diagonal part of
                   // its SpMV may run before the wait
@@ -115,6 +116,25 @@ struct ArnArgs {
   unsigned* gbar;  // [0] arrivals, [1] generation
 };
 
+// Block `bid` of the G that share a system: its rows [R0, R1), whole fine ranges f0 .. f1 - 1 (fine
+// range f: the units [f U / F, (f + 1) U / F) of the U); one fine range per block where a grid of
+// F blocks runs the system, several where a cluster of fewer blocks does
+struct ArnRows {
+  int G, bid, f0, f1;
+  long long R0, R1;
+};
+template <typename A>
+__device__ __forceinline__ ArnRows arn_rows(const A& a, int G, int bid) {
+  ArnRows o;
+  o.G = G;
+  o.bid = bid;
+  o.f0 = (int)((long long)bid * a.fine / G);
+  o.f1 = (int)((long long)(bid + 1) * a.fine / G);
+  o.R0 = (long long)o.f0 * a.units / a.fine * kArnUnit;
+  o.R1 = (long long)o.f1 * a.units / a.fine * kArnUnit;
+  return o;
+}
+
 // rows VN elements at a time (16-byte loads of the basis type, 8-byte for BF16: a warp's chunk is
 // then at most kArnUnit rows)
 template <typename TV> struct ArnVec { static constexpr int n = sizeof(TV) == 8 ? 2 : 4; };
@@ -122,7 +142,23 @@ template <typename TV> struct ArnVec { static constexpr int n = sizeof(TV) == 8 
 // Grid barrier (cooperative launch: every block resident).  Thread 0 arrives on bar[0];
 // the last arrival resets it and advances the generation bar[1]; the others poll the
 // generation with a bound and report false when it never moves.
+// CL: the blocks are one thread-block cluster, whose hardware barrier (all its threads) takes
+// the place of the words in global memory.
+__device__ __forceinline__ void arn_cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void arn_cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <bool CL>
 __device__ __forceinline__ bool arn_grid_sync(unsigned* bar, unsigned gen) {
+  if constexpr (CL) {
+    __syncwarp();
+    arn_cluster_arrive();
+    arn_cluster_wait();
+    return true;
+  }
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -153,15 +189,26 @@ __device__ __forceinline__ bool arn_grid_sync(unsigned* bar, unsigned gen) {
 // of a phase is published, carries on with work that does not need the other blocks'
 // shares, and waits later until the counter reaches the target (G arrivals per phase,
 // counted from the value read at the kernel's start; compared modulo 2^32).
+template <bool CL>
 __device__ __forceinline__ void arn_arrive(unsigned* cnt) {
   __syncthreads();
+  if constexpr (CL) {
+    arn_cluster_arrive();
+    return;
+  }
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(cnt, 1u);
   }
 }
 
+template <bool CL>
 __device__ __forceinline__ bool arn_wait(const unsigned* cnt, unsigned target) {
+  if constexpr (CL) {
+    __syncwarp();
+    arn_cluster_wait();
+    return true;
+  }
   __shared__ int s_ok;
   if (threadIdx.x == 0) {
     int ok = 1;
@@ -382,7 +429,7 @@ struct ArnSplit {
 };
 __device__ __forceinline__ ArnSplit arn_split(int nch) {
   const int warp = threadIdx.x >> 5;
-  if (nch >= kArnWarps) return ArnSplit{1, warp, 0, kArnWarps, true};
+  if (nch >= kArnWarps || nch == 0) return ArnSplit{1, warp, 0, kArnWarps, nch > 0};
   const int S = kArnWarps / nch;
   return ArnSplit{S, warp % nch, warp / nch, nch, warp / nch < S};
 }
@@ -603,7 +650,7 @@ __device__ __forceinline__ void arn_dia_rows(TACC (&acc)[B], long long row0, lon
 template <typename TV, typename TACC>
 __device__ __forceinline__ int arn_share(const ArnArgs<TV, TACC>& a, int G) {
   constexpr int per = kArnUnit / (32 * ArnVec<TV>::n);  // chunks per unit
-  const int most = ((a.units + G - 1) / G) * per;
+  const int most = ((a.fine + G - 1) / G) * ((a.units + a.fine - 1) / a.fine) * per;
   return most < kArnWarps ? kArnWarps / most : 1;
 }
 
@@ -836,15 +883,13 @@ __device__ __forceinline__ void arn_slot_sums(const int4* slot, int nch, int k, 
 // SpMV, coarse correction and multi-dot of step j over the block's super-tiles (a function
 // of its own, so that the cycle loop's state stays out of these loops' registers)
 template <typename TV, typename TACC, int ND, int MODE>
-__device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TACC sig, bool waited,
+__device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnRows& g, int j, TACC sig, bool waited,
                                        bool first_diag_done, TACC* Ws, TACC* Us, TACC* Ss,
                                        double* sbuf, const int* sE, int* semax, double* sred) {
   constexpr int VN = ArnVec<TV>::n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = threadIdx.x;
-  const int G = gridDim.x, bid = blockIdx.x;
-  const long long R0 = (long long)bid * a.units / G * kArnUnit;
-  const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
+  const long long R0 = g.R0, R1 = g.R1;
   const long long N = a.N;
   const int k = j + 1;
   const bool multi = R1 - R0 > a.RS;  // w goes through global memory to the update
@@ -997,7 +1042,7 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, int j, TAC
       __syncthreads();
       arn_slot_sums<NSET>(slot, nch, k, sE, ew, eu, tile == 0, sred);
     } else {
-      arn_dots_rows<TV, TACC, NSET, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, arn_share(a, G),
+      arn_dots_rows<TV, TACC, NSET, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0, nch, arn_share(a, g.G),
                                                      Ws, Us, lane);
     }
     __syncthreads();  // the slices are rewritten by the next super-tile
@@ -1200,22 +1245,20 @@ __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, dou
 // the block's first row, when given); returns the warp's part of ||u_{j+1}||^2 (in every lane)
 // (PASS2: only the rows [base, end), w back into Ws, indexed from base, and global memory)
 template <typename TV, typename TACC, bool PASS2>
-__device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
+__device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, const ArnRows& g, int k, TACC* Ws,
                                           const TACC* scoef, TACC* ush, long long base,
                                           long long end, float* sP) {
   constexpr int VN = ArnVec<TV>::n;
   constexpr int U = PASS2 ? 6 : 8;  // basis loads in flight per lane, reloaded as they are used
   constexpr int chunk = 32 * VN;
   const int lane = threadIdx.x & 31;
-  const int G = gridDim.x, bid = blockIdx.x;
-  const long long R0 = (long long)bid * a.units / G * kArnUnit;
-  const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
+  const long long R0 = g.R0, R1 = g.R1;
   const long long N = a.N;
   TV* __restrict__ vout = const_cast<TV*>(a.V) + (size_t)k * a.ldv;
   float ns = 0.f, nc = 0.f;  // a double-FP32 pair (FP64 adds are dear)
   const int nch = (int)((end - base) / chunk);
   const bool wsm = R1 - R0 <= a.RS;  // the block's w is still in shared memory
-  const ArnSplit sp = arn_split32(arn_share(a, G), nch);
+  const ArnSplit sp = arn_split32(arn_share(a, g.G), nch);
   const bool one = sp.S > 1;
   const int c0 = sp.p * k / sp.S, c1 = (sp.p + 1) * k / sp.S;
   long long r = base + (long long)(nch - 1 - sp.q0) * chunk + (long long)lane * VN;
@@ -1315,18 +1358,17 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, int k, 
 // CGS2, first update and second multi-dot of an FP32 or BF16 basis: per super-tile (from the last)
 // w -= V (sigma o h), then V^T w into the per-warp pairs
 template <typename TV, typename TACC, int ND>
-__device__ __forceinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, int k, TACC* Ws,
+__device__ __forceinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, const ArnRows& g, int k, TACC* Ws,
                                             const TACC* scoef, double* sbuf) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int G = gridDim.x, bid = blockIdx.x;
-  const long long R0 = (long long)bid * a.units / G * kArnUnit;
-  const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
+  const long long R0 = g.R0, R1 = g.R1;
   const int tiles = (int)((R1 - R0 + a.RS - 1) / a.RS);
   for (int tile = tiles - 1; tile >= 0; --tile) {
     const long long s0 = R0 + (long long)tile * a.RS;
     const long long s1 = s0 + a.RS < R1 ? s0 + a.RS : R1;
     __syncthreads();
-    arn_update<TV, TACC, true>(a, k, Ws, scoef, nullptr, s0, s1, reinterpret_cast<float*>(sbuf));
+    arn_update<TV, TACC, true>(a, g, k, Ws, scoef, nullptr, s0, s1,
+                               reinterpret_cast<float*>(sbuf));
     __syncthreads();
     if (tile == tiles - 1) {  // (the shares of a chunk, one super-tile only, used sbuf)
       for (int q = threadIdx.x; q < kMaxK * kArnWarps; q += kArnThreads) sbuf[q] = 0.0;
@@ -1334,7 +1376,7 @@ __device__ __forceinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, int k
     }
     arn_dots_rows<TV, TACC, 1, arn_group<ND>()>(sbuf, a.V, a.ldv, k, s0,
                                                 (int)((s1 - s0) / (32 * ArnVec<TV>::n)),
-                                                arn_share(a, G), Ws, nullptr, lane);
+                                                arn_share(a, g.G), Ws, nullptr, lane);
   }
   __syncthreads();
 }
@@ -1346,10 +1388,10 @@ __device__ __forceinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, int k
 // block wrote them just before).  Fixed order throughout.
 template <bool C32, typename TV, typename TACC>
 __device__ __forceinline__ void arn_piece_sums(const ArnArgs<TV, TACC>& a, const TV* vout,
-                                               const TACC* ush, long long R0) {
+                                               const TACC* ush, const ArnRows& g) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int bid = blockIdx.x;
-  const int p0 = __ldg(a.blk_piece_start + bid), p1 = __ldg(a.blk_piece_start + bid + 1);
+  const long long R0 = g.R0;
+  const int p0 = __ldg(a.blk_piece_start + g.f0), p1 = __ldg(a.blk_piece_start + g.f1);
   for (int base = p0 + warp; base < p1; base += kArnWarps * 8) {
     const int pi = base + kArnWarps * lane;
     int mp = -1, ms = 0, me = 0;
@@ -1427,14 +1469,14 @@ __device__ __forceinline__ void arn_piece_sums_staged(double* cpart, const TACC*
 
 // The block's largest high word of |u| (the warp's lanes hold the candidates) into its slot of the
 // partials, and after a grid barrier the largest exponent over all blocks (one warp each)
-__device__ __forceinline__ void arn_put_max(Ctl& ctl, int m) {
+__device__ __forceinline__ void arn_put_max(Ctl& ctl, int bid, int m) {
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0)
-    __stcg(&ctl.part[(size_t)blockIdx.x * ctl.ldp + kArnMaxCol], __hiloint2double(0, m));
+    __stcg(&ctl.part[(size_t)bid * ctl.ldp + kArnMaxCol], __hiloint2double(0, m));
 }
-__device__ __forceinline__ int arn_get_max(const Ctl& ctl) {
+__device__ __forceinline__ int arn_get_max(const Ctl& ctl, int G) {
   int m = 0;
-  for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32)
+  for (int b = threadIdx.x & 31; b < G; b += 32)
     m = max(m, __double2loint(__ldcg(&ctl.part[(size_t)b * ctl.ldp + kArnMaxCol])));
   return __reduce_max_sync(0xffffffffu, m) >> 20;
 }
@@ -1469,9 +1511,9 @@ __device__ __forceinline__ void arn_block_sums(const double* sbuf, int ncols, in
   __syncthreads();
 }
 
-template <typename TV, typename TACC, int ND, int MODE>
-__global__ void __launch_bounds__(kArnThreads, 1)
-    k_arnoldi(const __grid_constant__ ArnArgs<TV, TACC> a) {
+// The cycle of one system by G blocks, this one bid; CL: the blocks are a cluster
+template <typename TV, typename TACC, int ND, int MODE, bool CL>
+__device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int G, const int bid) {
   static_assert(MODE != kArnLowsyncDf || sizeof(TV) == 8, "the double-FP32 multi-dot takes an FP64 basis");
   static_assert(MODE == kArnCgs2 || sizeof(TV) == sizeof(TACC), "BF16 bases use CGS2");
   // the FP32 one-reduction step of a banded operator runs its coarse solve in FP32, every
@@ -1494,10 +1536,8 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   Ctl& ctl = const_cast<Ctl&>(a.ctl);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = threadIdx.x;
-  const int G = gridDim.x, bid = blockIdx.x;
-  const long long R0 = (long long)bid * a.units / G * kArnUnit;
-  const long long R1 = (long long)(bid + 1) * a.units / G * kArnUnit;
-  const long long N = a.N;
+  const ArnRows g = arn_rows(a, G, bid);
+  const long long R0 = g.R0, R1 = g.R1;
   // shared memory: w and u_j of a super-tile, s' (r), reduction scratch, the rows of L
   // (stride kMaxK), the FP64 multi-dot staging
   TACC* Ws = reinterpret_cast<TACC*>(smem);
@@ -1522,10 +1562,10 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     }
     return;
   }
-  unsigned gen = *(volatile unsigned*)&a.gbar[1];  // advanced only once all arrive
+  unsigned gen = CL ? 0u : *(volatile unsigned*)&a.gbar[1];  // advanced only once all arrive
   // the split barrier's counter: no block arrives before every block has passed the first
   // grid barrier, so all read the same base
-  const unsigned cbase = *(volatile unsigned*)&a.gbar[2];
+  const unsigned cbase = CL ? 0u : *(volatile unsigned*)&a.gbar[2];
   for (int q = t; q < kMaxK * kMaxK; q += kArnThreads) sL[q] = 0.0;
   if (t == 0) ssig[0] = __ldcg(&ctl.sigma[0]);
   // the block's aggregate pieces for the whole cycle: their ids, local starts and nodes (as
@@ -1535,8 +1575,8 @@ __global__ void __launch_bounds__(kArnThreads, 1)
   __shared__ int spls[kArnMaxBlkPieces + 1];
   const long long nrows = R1 - R0;
   unsigned short* snode = reinterpret_cast<unsigned short*>(Us + nrows);
-  const int bp0 = a.defl ? __ldg(a.blk_piece_start + bid) : 0;
-  const int bp1 = a.defl ? __ldg(a.blk_piece_start + bid + 1) : 0;
+  const int bp0 = a.defl ? __ldg(a.blk_piece_start + g.f0) : 0;
+  const int bp1 = a.defl ? __ldg(a.blk_piece_start + g.f1) : 0;
   const bool staged = a.defl && bp1 - bp0 <= kArnMaxBlkPieces && nrows <= 65536 &&
                       (size_t)nrows * sizeof(TACC) + (size_t)nrows * 2 <= (size_t)a.RS * sizeof(TACC);
   if (staged) {
@@ -1605,13 +1645,13 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     mx = __reduce_max_sync(0xffffffffu, mx);
     if (lane == 0) smax[warp] = mx;
     __syncthreads();
-    if (warp == 0) arn_put_max(ctl, lane < kArnWarps ? smax[lane] : 0);
-    if (!arn_grid_sync(a.gbar, gen++)) {
+    if (warp == 0) arn_put_max(ctl, bid, lane < kArnWarps ? smax[lane] : 0);
+    if (!arn_grid_sync<CL>(a.gbar, gen++)) {
       arn_timeout(ctl);
       return;
     }
     if (warp == 0) {
-      const int e = arn_get_max(ctl);
+      const int e = arn_get_max(ctl, G);
       if (lane == 0) sE[0] = e;
       if (lane == 0 && bid == 0) ctl.vexp[0] = e;
     }
@@ -1626,15 +1666,17 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // pairs per warp and column)
     if constexpr (sizeof(TV) < 8 || MODE == kArnLowsyncDf)
       for (int q = t; q < 2 * kMaxK * 33; q += kArnThreads) sbuf[q] = 0.0;
-    arn_front<TV, TACC, ND, MODE>(a, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sE, semax, sred);
+    arn_front<TV, TACC, ND, MODE>(a, g, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sE, semax, sred);
     waited = true;
+    if (sizeof(TV) == 8 && R0 == R1)  // a block without rows (a small system's cluster)
+      for (int c = t; c < NSET * k; c += kArnThreads) sred[c] = 0.0;
     // per-block column sums (fixed order; a fixed-point multi-dot leaves them in sred)
     arn_block_sums<TV, MODE>(sbuf, NSET * k, k, sred);
     // the partials: FP64 values, or double-FP32 pairs (two floats in the slot) for an FP32 or
     // BF16 basis, whose cross-block sums then run on the FP32 pipe
     for (int c = t; c < NSET * k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
     // ---- 3. grid barrier; identical totals in every block -------------------------------
-    if (!arn_grid_sync(a.gbar, gen++)) {
+    if (!arn_grid_sync<CL>(a.gbar, gen++)) {
       arn_timeout(ctl);
       return;
     }
@@ -1653,11 +1695,13 @@ __global__ void __launch_bounds__(kArnThreads, 1)
         arn_pass2_fx(a.V, a.ldv, a.w, a.RS, R0, R1, k, scoef, sE, Ws,
                      sbuf, semax, &sscale, sred);
       } else {
-        arn_pass2_rows<TV, TACC, ND>(a, k, Ws, scoef, sbuf);
+        arn_pass2_rows<TV, TACC, ND>(a, g, k, Ws, scoef, sbuf);
       }
+      if (sizeof(TV) == 8 && R0 == R1)
+        for (int c = t; c < k; c += kArnThreads) sred[c] = 0.0;
       arn_block_sums<TV, MODE>(sbuf, k, k, sred);
       for (int c = t; c < k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
-      if (!arn_grid_sync(a.gbar, gen++)) {
+      if (!arn_grid_sync<CL>(a.gbar, gen++)) {
         arn_timeout(ctl);
         return;
       }
@@ -1721,7 +1765,7 @@ __global__ void __launch_bounds__(kArnThreads, 1)
           a.V, a.ldv, vout, a.w, R0, R1, MODE == kArnLowsync ? k - 1 : k, k, scoef, sE, sbuf,
           &sscale, ush, mx);
     else
-      nrm = arn_update<TV, TACC, false>(a, k, Ws, scoef, ush, R0, R1,
+      nrm = arn_update<TV, TACC, false>(a, g, k, Ws, scoef, ush, R0, R1,
                                           reinterpret_cast<float*>(sbuf));
     // ---- 5. norm partial; partial sums of u_{j+1} over this block's aggregate pieces ----
     {
@@ -1738,16 +1782,16 @@ __global__ void __launch_bounds__(kArnThreads, 1)
 #pragma unroll
         for (int o = kArnWarps / 2; o > 0; o >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, o);
         if (lane == 0) __stcg(&ctl.part[(size_t)bid * ctl.ldp + kArnNormCol], bs);
-        if constexpr (sizeof(TV) == 8) arn_put_max(ctl, lane < kArnWarps ? smax[lane] : 0);
+        if constexpr (sizeof(TV) == 8) arn_put_max(ctl, bid, lane < kArnWarps ? smax[lane] : 0);
       }
       if (a.defl && k < a.jmax) {
         if (staged && ush)
           arn_piece_sums_staged<C32>(ctl.cpart, ush, snode, spid, spls, bp1 - bp0);
         else
-          arn_piece_sums<C32>(a, vout, ush, R0);
+          arn_piece_sums<C32>(a, vout, ush, g);
       }
     }
-    if (!arn_grid_sync(a.gbar, gen++)) {
+    if (!arn_grid_sync<CL>(a.gbar, gen++)) {
       arn_timeout(ctl);
       return;
     }
@@ -1760,7 +1804,9 @@ __global__ void __launch_bounds__(kArnThreads, 1)
       for (int b = lane; b < G; b += 32) v += __ldcg(&ctl.part[(size_t)b * ctl.ldp + kArnNormCol]);
       givens_step(ctl, j, a.m, sqrt(warp_sum(v)));
       __syncwarp();
-      if (split0 && lane == 0) {
+      if (CL) {
+        if (split0) arn_cluster_arrive();
+      } else if (split0 && lane == 0) {
         __threadfence();
         atomicAdd(&a.gbar[2], 1u);
       }
@@ -1862,12 +1908,13 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     // diagonal part of the next step's SpMV for the first super-tile, which needs only
     // u_{j+1} (complete since the barrier), not s' or sigma_{j+1} (it overwrites c); then
     // wait for every block's arrival
-    if (!split0) arn_arrive(&a.gbar[2]);
+    if (!split0) arn_arrive<CL>(&a.gbar[2]);
+    else if (CL && warp > 0) arn_cluster_arrive();
     // the exponent of column j + 1 (one warp; the slots are written again only after this block's
     // next arrival)
     if constexpr (sizeof(TV) == 8) {
       if (warp == kArnWarps - 1) {
-        const int e = arn_get_max(ctl);
+        const int e = arn_get_max(ctl, G);
         if (lane == 0) sE[k] = e;
         if (lane == 0 && bid == 0) ctl.vexp[k] = e;
       }
@@ -1875,7 +1922,7 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     if (k < a.jmax && (!split0 || warp > 0))
       arn_diag<ND, TV, TACC>(a, k, R0, R0 + a.RS < R1 ? R0 + a.RS : R1, Ws, Us,
                              split0 ? t - 32 : t, split0 ? kArnThreads - 32 : kArnThreads);
-    if (!arn_wait(&a.gbar[2], cbase + (unsigned)G * (unsigned)k)) {
+    if (!arn_wait<CL>(&a.gbar[2], cbase + (unsigned)G * (unsigned)k)) {
       arn_timeout(ctl);
       return;
     }
@@ -1885,6 +1932,33 @@ __global__ void __launch_bounds__(kArnThreads, 1)
     __syncthreads();
     if (done) break;
   }
+}
+
+template <typename TV, typename TACC, int ND, int MODE>
+__global__ void __launch_bounds__(kArnThreads, 1)
+    k_arnoldi(const __grid_constant__ ArnArgs<TV, TACC> a) {
+  arn_cycle<TV, TACC, ND, MODE, false>(a, (int)gridDim.x, (int)blockIdx.x);
+}
+
+// The cycles of many systems, a cluster of G blocks each: cluster c runs the c-th system of the list
+// (list[0] systems still running, then their positions in args) when that count is in (lo, hi];
+// deflation as the system's flag says
+template <typename TV, typename TACC, int ND, int MODE>
+__global__ void __launch_bounds__(kArnThreads, 1)
+    k_arnoldi_batch(const ArnArgs<TV, TACC>* __restrict__ args, const int* __restrict__ list, int lo,
+                    int hi, int G) {
+  __shared__ ArnArgs<TV, TACC> a;
+  const int n = __ldg(list), c = (int)blockIdx.x / G;
+  if (n <= lo || n > hi || c >= n) return;  // the whole cluster
+  const int* src = reinterpret_cast<const int*>(args + __ldg(list + 1 + c));
+  for (int q = threadIdx.x; q < (int)(sizeof(a) / 4); q += kArnThreads)
+    reinterpret_cast<int*>(&a)[q] = __ldg(src + q);
+  __syncthreads();
+  const int on = __ldcg(&a.ctl.flags[F_DEFL_ON]);
+  __syncthreads();
+  if (threadIdx.x == 0) a.defl = a.defl && on;
+  __syncthreads();
+  arn_cycle<TV, TACC, ND, MODE, true>(a, G, (int)(blockIdx.x % G));
 }
 
 // rows of a super-tile: w and u_j slices, s' and the reduction scratch in kArnSmem
@@ -1897,6 +1971,59 @@ inline long long arn_super_rows(int r, size_t esz) {
 
 template <typename TV, typename TACC>
 struct Arn {
+  using Args = ArnArgs<TV, TACC>;
+  // many systems, a cluster of G blocks each (args, list: device arrays)
+  template <int ND, int MODE>
+  static cudaError_t batch_nd(const FusedBatch& f, int clusters, int lo, int hi, int G,
+                              cudaStream_t st) {
+    auto* kern = k_arnoldi_batch<TV, TACC, ND, MODE>;
+    static cudaError_t prep = [&] {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)kArnSmem);
+      return e == cudaSuccess
+                 ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
+                 : e;
+    }();
+    if (prep != cudaSuccess) return prep;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * G));
+    cfg.blockDim = dim3((unsigned)kArnThreads);
+    cfg.dynamicSmemBytes = kArnSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)G;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (clusters == 0) {  // query: the clusters of G blocks that fit the device at once
+      cfg.gridDim = dim3((unsigned)G);
+      int n = 0;
+      const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+      if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        n = 0;
+      }
+      *f.fit = n;
+      return cudaSuccess;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<const Args*>(f.args), f.list, lo, hi, G);
+  }
+  static cudaError_t batch(const FusedBatch& f, int clusters, int lo, int hi, int G,
+                           cudaStream_t st) {
+    if (f.ortho == GMRES_ORTHO_CGS2) return batch_op<kArnCgs2>(f, clusters, lo, hi, G, st);
+    if constexpr (sizeof(TV) == sizeof(TACC))
+      return batch_op<kArnLowsync>(f, clusters, lo, hi, G, st);
+    else
+      return cudaErrorInvalidValue;
+  }
+  template <int MODE>
+  static cudaError_t batch_op(const FusedBatch& f, int clusters, int lo, int hi, int G,
+                              cudaStream_t st) {
+    return f.nd == 9  ? batch_nd<9, MODE>(f, clusters, lo, hi, G, st)
+           : f.nd > 0 ? batch_nd<0, MODE>(f, clusters, lo, hi, G, st)
+                      : batch_nd<kArnCsr, MODE>(f, clusters, lo, hi, G, st);
+  }
   template <int ND, int MODE>
   static cudaError_t prepare() {
     return cudaFuncSetAttribute(k_arnoldi<TV, TACC, ND, MODE>,
@@ -1931,17 +2058,17 @@ struct Arn {
     }
     return e;
   }
-  static cudaError_t launch(const CycleArgs& c, int jmax, bool defl, cudaStream_t st) {
-    ArnArgs<TV, TACC> p{};
+  static Args fill(const CycleArgs& c, int jmax, bool defl) {
+    Args p{};
     p.N = c.op.n;
     p.units = (int)(c.ldv / kArnUnit);
+    p.fine = p.units < c.sms ? p.units : c.sms;
     p.jmax = jmax;
     p.m = c.m;
     p.pre = (defl && c.pdl) ? 1 : 0;
     p.defl = defl ? 1 : 0;
     p.r = defl ? c.op.defl.r : 0;
     p.RS = (int)arn_super_rows(p.r, sizeof(TACC));
-    if (p.RS < kArnUnit) return cudaErrorInvalidValue;  // arnoldi_fusable rules this out
     p.ldv = c.ldv;
     p.ldd = c.op.ldd;
     p.V = static_cast<const TV*>(c.V);
@@ -1976,6 +2103,11 @@ struct Arn {
     p.vec = c.op.vec;
     if constexpr (sizeof(TACC) == 8) p.val = c.op.val;
     else p.val = c.op.val32;
+    return p;
+  }
+  static cudaError_t launch(const CycleArgs& c, int jmax, bool defl, cudaStream_t st) {
+    const Args p = fill(c, jmax, defl);
+    if (p.RS < kArnUnit) return cudaErrorInvalidValue;  // arnoldi_fusable rules this out
     if (c.ortho == GMRES_ORTHO_CGS2) return launch_op<kArnCgs2>(c, p, st);
     if constexpr (sizeof(TV) == 8) {
       // (a CSR operator takes the fixed-point multi-dot whatever dot_arith says)

@@ -145,6 +145,29 @@ bool arnoldi_fusable(const CycleArgs& a);
 bool arnoldi_fixed(const CycleArgs& a);
 // one launch runs the jmax steps of a restart cycle (fewer when the cycle ends early)
 cudaError_t launch_arnoldi(const CycleArgs& a, int jmax, bool defl, cudaStream_t st);
+// The batched form: one thread-block cluster per system runs the system's cycle (fused_batch_*.cu)
+constexpr int kBatchTiers = 4;
+struct FusedBatch {
+  int tiers = 0;                // cluster sizes in use (0: the batch runs the phase kernels)
+  int G[kBatchTiers] = {};      // blocks per cluster
+  int upto[kBatchTiers] = {};   // and the most running systems a cluster size serves
+  int nd = 0, ortho = 0;       // diagonals of every operator (0: CSR), gmres_ortho
+  const void* args = nullptr;  // device: one system's kernel arguments each, largest system first
+  const int* list = nullptr;   // device: running systems, then their positions in args
+  int* fit = nullptr;          // host: the answer of a query (clusters = 0)
+};
+// one system's kernel arguments (written to dst unless null); returns their size
+size_t arnoldi_args_fp64(const CycleArgs& a, bool defl, void* dst);
+size_t arnoldi_args_fp32(const CycleArgs& a, bool defl, void* dst);
+size_t arnoldi_args_bf16(const CycleArgs& a, bool defl, void* dst);
+// `clusters` clusters of G blocks, in effect when the number of running systems is in (lo, hi];
+// clusters = 0 only asks how many fit the device at once
+cudaError_t launch_arnoldi_batch_fp64(const FusedBatch& f, int clusters, int lo, int hi, int G,
+                                      cudaStream_t st);
+cudaError_t launch_arnoldi_batch_fp32(const FusedBatch& f, int clusters, int lo, int hi, int G,
+                                      cudaStream_t st);
+cudaError_t launch_arnoldi_batch_bf16(const FusedBatch& f, int clusters, int lo, int hi, int G,
+                                      cudaStream_t st);
 // Control-block initialisation for a new solve.
 cudaError_t launch_init(const CycleArgs& a, double tol, double inner_tol, double r0ref,
                         double mu, int fixed, int mixed, long long maxit, cudaStream_t st);
