@@ -153,7 +153,10 @@ inline gmres_status ensure_workspace(gmres_s* h, int m, int prec) {
     CK(h, h->w.ensure(sizeof(double) * (size_t)ldv));
     CK(h, cudaMemsetAsync(h->w.p, 0, sizeof(double) * (size_t)ldv, h->stream));
   }
-  CK(h, h->t.ensure(sizeof(double) * (size_t)ldv));
+  if (!h->t.p) {  // (the multi-dot over a dense space copies whole tiles of it, like w's)
+    CK(h, h->t.ensure(sizeof(double) * (size_t)ldv));
+    CK(h, cudaMemsetAsync(h->t.p, 0, sizeof(double) * (size_t)ldv, h->stream));
+  }
   CK(h, h->part.ensure(sizeof(double) * (size_t)max_grid * kLdp));
   CK(h, h->part2.ensure(sizeof(double) * (size_t)kMaxGroups * kLdp));
   if (!h->tickets.p) {

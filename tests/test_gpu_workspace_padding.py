@@ -1,0 +1,30 @@
+"""The rows between n and the next multiple of 256 of a workspace vector: they are copied with
+whole tiles, so they have to hold zeros whatever the memory held before (the fixed-point basis of
+a closed handle, say: small negative integers read as NaNs)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from helpers import gpu_solver_from_oracle, to_dev
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("n", [39, 200])
+def test_adaptive_space_after_a_closed_handle(orc, n):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1906_04051_gb300 as G
+    p = W.convdiff(n, pe=10.0, sigma=0.5, seed=21, px=1, py=1)
+    A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+    for m in (20, 40, 60, 30, 50):
+        s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_NONE, fixed_iterations=True)
+        s.solve(to_dev(b), m=m, tol=0.0, maxit=m)
+        s.close()
+        s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_ADAPTIVE, rmax=6, ninv=2)
+        x, info = s.solve(to_dev(b), m=12, tol=1e-3, maxit=400)
+        assert info["rel_res_true"] < 1.0
+        true = np.linalg.norm(b - A.matvec(x.cpu().numpy())) / np.linalg.norm(b)
+        assert true == pytest.approx(info["rel_res_true"], rel=1e-6)
+        s.close()
