@@ -36,13 +36,10 @@ UNIT = "solves/s"
 # (inverse compact WY) form; CGS2 and column-by-column MGS are timed beside it
 ORTHO = 2  # GMRES_ORTHO_MGS_LOWSYNC
 M, TOL, MAXIT = 50, 1e-8, 20000
-# FP64 FMA peak of GB300: 2 DFMA/clk/SM (ncu sm__sass_thread_inst_executed_op_dfma
-# peak_sustained) x 152 SMs x 2.07 GHz x 2 flop
-FP64_PEAK_TFLOPS = 2 * 152 * 2.07e9 * 2 / 1e12
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the fused Arnoldi kernel
 # (a full 50-step deflated cycle) on this workload, FP64 and FP32 basis (one ncu capture
 # each, profiles/k_arnoldi_cycle_q1-n1024_*.txt); None once the kernel changes
-ARN_DRAM_BYTES_CYCLE50 = {8: 21.859e9, 4: 8.261e9}
+ARN_DRAM_BYTES_CYCLE50 = {8: None, 4: None}
 # Arnoldi steps the deflated GMRES(50) takes to 1e-8 on this workload (deterministic;
 # the GPU arm prints its own count): used only to project the CPU sample to a full solve
 PROJECT_ITERS = 782
@@ -148,18 +145,14 @@ def cycle_ks(iters, cycles, m):
 
 
 def arn_units(layout, n, ks, s, coarse_steps=0):
-    """Algorithmic FP64 FMAs and bytes of the fused Arnoldi kernel over steps with k basis
-    columns (s bytes per basis / operator element): the SpMV (nd diagonals, the A W rows,
-    x), the one-reduction MGS multi-dot (2 k FMA per row: V^T w and V^T u_j; the basis read
-    once), the update (k FMA per row; the basis read again, u_{j+1} written) and the norm;
-    w and u_j stay on chip.  coarse_steps of them also run the next step's coarse solve in
-    the kernel: the sums of u_{j+1} over the aggregates (n adds, from shared memory) and
-    y = T^-1 c (r^2 FMA, T^-1 read in the basis precision)."""
+    """Algorithmic bytes of the fused Arnoldi kernel over steps with k basis columns (s bytes
+    per basis / operator element): the SpMV (nd diagonals, the A W rows, x), the one-reduction
+    MGS multi-dot (the basis read once), the update (the basis read again, u_{j+1} written);
+    w and u_j stay on chip.  coarse_steps of them also run the next step's coarse solve in the
+    kernel (T^-1, r^2 elements, read in the basis precision)."""
     nd, nau, r = layout.get("ndiag", 0), layout.get("nau", 0), layout.get("r", 0)
-    fma = sum(nd * n + nau + 3.0 * k * n + n for k in ks) + coarse_steps * (r * r + 0.5 * n)
-    byt = (sum(s * (nd * n + n + 2.0 * k * n + n) + 4.0 * (n + 1) + (4.0 + s) * nau for k in ks)
-           + coarse_steps * s * r * r)
-    return fma, byt
+    return (sum(s * (nd * n + n + 2.0 * k * n + n) + 4.0 * (n + 1) + (4.0 + s) * nau for k in ks)
+            + coarse_steps * s * r * r)
 
 
 def cpu_baseline(p, budget_steps=M):
@@ -455,7 +448,7 @@ def main():
 
     # ---- roofline of the dominant kernel: the fused Arnoldi step (k_arnoldi) -------------
     # one launch per Arnoldi step: SpMV, the one-reduction MGS multi-dot, the update, the
-    # norm and the rotations; FP64 work bound by the FMA pipe
+    # norm and the rotations; the basis is read twice (multi-dot, update) from HBM
     N, nnz = p.N, p.nnz
     it = infos[-1]["iters"]
     cyc = infos[-1]["cycles"]
@@ -465,31 +458,27 @@ def main():
     # every step of a deflated cycle but its last also runs the next step's coarse solve;
     # the first cycle runs undeflated (|mu| comes from its Ritz values)
     coarse = max(0, (it - min(it, M)) - (cyc - 1))
-    fma, arn_bytes = arn_units(layout, N, ks, 8, coarse_steps=coarse)
+    arn_bytes = arn_units(layout, N, ks, 8, coarse_steps=coarse)
     # every timed step runs the same deterministic solve, so each launches what the
     # profiled one did
     launches = args.steps * sum(v[1] for v in profs[-1].values())
-    achieved = 2.0 * fma / (ms_arn / 1e3) / 1e12
+    arnoldi_gbs = arn_bytes / (ms_arn / 1e3) / 1e9
     hbm_peak, peak_kind = _peaks()
     # a launch is a restart cycle: per-launch figures average over the solve's cycles; the
     # captured traffic of a full cycle is scaled to them by their algorithmic bytes
     traffic = None
     if ARN_DRAM_BYTES_CYCLE50[8] is not None:
-        _, b50 = arn_units(layout, N, list(range(1, M + 1)), 8, coarse_steps=M - 1)
+        b50 = arn_units(layout, N, list(range(1, M + 1)), 8, coarse_steps=M - 1)
         traffic = ARN_DRAM_BYTES_CYCLE50[8] * (arn_bytes / cyc) / b50
     roofline = {"kernel": "k_arnoldi (one launch per restart cycle; per step the SpMV, the "
                           "one-reduction MGS multi-dot, update, norm, rotations and the next "
-                          "step's coarse solve)", "bound": "alu",
-                "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS,
+                          "step's coarse solve)", "bound": "hbm",
+                "achieved": arnoldi_gbs, "peak": hbm_peak, "unit": "GB/s",
+                "frac": arnoldi_gbs / hbm_peak,
                 "traffic": traffic, "traffic_unit": "bytes per launch",
                 "algorithmic_bytes_per_launch": arn_bytes / cyc,
                 "launches": "one per restart cycle",
-                "peak_kind": "derived FP64 FMA rate",
-                "hbm_gbs_same_kernel": arn_bytes / (ms_arn / 1e3) / 1e9}
-    # SpMV + Arnoldi algorithmic bytes over the whole solve (metric part 2): the fused
-    # kernel's time against the bytes the method must move
-    arnoldi_gbs = arn_bytes / (ms_arn / 1e3) / 1e9
+                "peak_kind": peak_kind}
 
     # ---- the same SpMV + Arnoldi with an FP32 basis and operator (the inner solve of the
     # mixed-precision method), 100 steps = two full GMRES(50) cycles of the fixed-iteration
@@ -507,11 +496,11 @@ def main():
             ph32 = s32.profile()
             s32.close()
             ks32 = cycle_ks(i32["iters"], i32["cycles"], M)
-            _, b32 = arn_units(layout, N, ks32, 4, coarse_steps=i32["iters"] - i32["cycles"])
+            b32 = arn_units(layout, N, ks32, 4, coarse_steps=i32["iters"] - i32["cycles"])
             ms32 = ph32["arnoldi"][0]
             t32 = None
             if ARN_DRAM_BYTES_CYCLE50[4] is not None:
-                _, b50 = arn_units(layout, N, list(range(1, M + 1)), 4, coarse_steps=M - 1)
+                b50 = arn_units(layout, N, list(range(1, M + 1)), 4, coarse_steps=M - 1)
                 t32 = ARN_DRAM_BYTES_CYCLE50[4] * (b32 / i32["cycles"]) / b50
             fp32_arnoldi = {"kernel": "k_arnoldi, one launch per restart cycle: SpMV, the next "
                                       "step's coarse solve, one-reduction MGS, update, "
@@ -634,9 +623,10 @@ def main():
             pr_ms = ev0.elapsed_time(ev1)
             bratu["protocol_100_cycles"] = {"ms": pr_ms, "iters": ib["iters"],
                                             "us_per_step": pr_ms * 1e3 / ib["iters"]}
-            # SpMV rate of the lane-per-row CSR kernel from a profiled cycle
+            # SpMV rate of the lane-per-row CSR kernel from a profiled cycle of the column-by-column
+            # MGS (the other forms run their SpMV inside the fused step kernel)
             sp = G.Solver(br, bc, bv, None, 0, deflation_mode=G.DEFL_NONE, fixed_iterations=True,
-                          profile=True)
+                          ortho=G.ORTHO_MGS, profile=True)
             sp.solve(bb, m=M, tol=0.0, maxit=M)
             ph_b = sp.profile()
             sp.close()
