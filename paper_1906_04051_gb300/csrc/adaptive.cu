@@ -206,17 +206,25 @@ __global__ void k_adapt_z(Ctl ctl, int ninv, double* __restrict__ zout, int* __r
   if (lane == 0) iv[0] = nvec;
 }
 
-// u = V_k z (the basis columns as stored, v_c = sigma_c u_c: z is scaled by sigma here)
+// u = V_k z (the basis columns as stored, v_c = sigma_c u_c: z is scaled by sigma here).
+// FIX: the cycle left its columns in fixed point (fixed.cuh), whose units go into z as well.
+template <bool FIX>
 __global__ void __launch_bounds__(kThreads)
     k_adapt_vz(int N, const double* __restrict__ V, long long ldv, const double* __restrict__ z,
                Ctl ctl, double* __restrict__ u) {
   __shared__ double sz[kMaxK];
   const int k = ctl.flags[F_K];
-  for (int c = threadIdx.x; c < k; c += blockDim.x) sz[c] = z[c] * ctl.sigma[c];
+  for (int c = threadIdx.x; c < k; c += blockDim.x) {
+    const double s = z[c] * ctl.sigma[c];
+    sz[c] = FIX ? ldexp(s, ctl.vexp[c] - 1083) : s;
+  }
   __syncthreads();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     double s = 0.0;
-    for (int c = 0; c < k; ++c) s += V[(size_t)c * ldv + i] * sz[c];
+    for (int c = 0; c < k; ++c) {
+      const double v = V[(size_t)c * ldv + i];
+      s += (FIX ? (double)__double_as_longlong(v) : v) * sz[c];
+    }
     u[i] = s;
   }
 }
@@ -707,8 +715,12 @@ gmres_status adapt_update(gmres_s* h, CycleArgs& a) {
   const int nvec = hiv[0];
   int q = h->aq;
   for (int v = 0; v < nvec; ++v) {
-    k_adapt_vz<<<grid, kThreads, 0, st>>>(N, static_cast<const double*>(a.V), ld,
-                                          z + (size_t)v * kMaxK, ctl, u);
+    if (a.fixv)
+      k_adapt_vz<true><<<grid, kThreads, 0, st>>>(N, static_cast<const double*>(a.V), ld,
+                                                  z + (size_t)v * kMaxK, ctl, u);
+    else
+      k_adapt_vz<false><<<grid, kThreads, 0, st>>>(N, static_cast<const double*>(a.V), ld,
+                                                   z + (size_t)v * kMaxK, ctl, u);
     k_adapt_norm<<<grid, kThreads, 0, st>>>(N, u, ctl, nrm);
     nl += 2;
     for (int pass = 0; pass < 2 && q > 0; ++pass) {

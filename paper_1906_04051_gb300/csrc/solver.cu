@@ -105,10 +105,10 @@ gmres_status run(gmres_s* h, OpHost& o, const double* b, const double* x0, int m
   const bool ada = h->opts.deflation_mode == GMRES_DEFL_ADAPTIVE;  // U grows from empty
   const bool dw = h->dense_r > 0;  // U from the caller's dense columns, fixed
   if (ada) h->aq = 0;
-  // the whole step in one persistent kernel where it applies (fused.cuh)
-  const bool fused = !mgs && !ada && !dw && arnoldi_fusable(a);
-  a.fixv = fused && arnoldi_fixed(a) ? 1 : 0;
-  if (fused) CK(h, cudaMemsetAsync(h->gbar.p, 0, 4 * sizeof(unsigned), st));
+  // the whole cycle in one persistent kernel where it applies (fused.cuh): not over a dense
+  // deflation space, but those solves' cycles before they have one
+  const bool fusable = !mgs && arnoldi_fusable(a);
+  if (fusable) CK(h, cudaMemsetAsync(h->gbar.p, 0, 4 * sizeof(unsigned), st));
   const int mu_mode = h->opts.mu_mode;
   double mu = 0.0;
   if (mu_mode == GMRES_MU_USER) mu = std::fabs(h->opts.mu_user);
@@ -143,6 +143,8 @@ gmres_status run(gmres_s* h, OpHost& o, const double* b, const double* x0, int m
       a.op.defl.ldu = h->ldv;
       a.op.defl.qd = defl_cycle ? h->aq : 0;
     }
+    const bool fused = fusable && a.op.defl.qd == 0;
+    a.fixv = fused && arnoldi_fixed(a) ? 1 : 0;
     if (defl_cycle) CK(h, phase(h, a, PH_DEFL, 0, true, x, b));
     const long long left = maxit - h->hmeta->counts[C_STEPS];
     const int jmax = (int)(left < m ? left : m);

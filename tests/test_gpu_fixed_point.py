@@ -106,3 +106,29 @@ def test_nonfinite_input_is_reported(G, orc, bad):
     s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_NONE, ortho=G.ORTHO_MGS_LOWSYNC)
     with pytest.raises(G.GmresError):
         s.solve(to_dev(b), m=10, tol=1e-8, maxit=50)
+
+
+# the cycles of an adaptive solve before it has a space are fused ones; its first vectors come from
+# their basis in fixed point (or in FP64: double-float dots over diagonals)
+@pytest.mark.parametrize("n,kind,ortho,df32", [(9, "dia", 0, 0), (40, "dia", 0, 0), (40, "csr", 0, 0),
+                                               (40, "dia", 2, 0), (40, "csr", 2, 0), (40, "dia", 2, 1)])
+def test_adaptive_space_from_a_fused_cycle(G, orc, n, kind, ortho, df32):
+    p = W.convdiff(n, pe=25.0, sigma=0.5, seed=140, px=1, py=1)
+    A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+    if kind == "csr":
+        perm = np.random.default_rng(n).permutation(A.n)
+        inv = np.argsort(perm)
+        rows = [sorted(zip(inv[A.col[A.rowptr[i]:A.rowptr[i + 1]]],
+                           A.val[A.rowptr[i]:A.rowptr[i + 1]])) for i in perm]
+        A = orc.CSR(np.cumsum([0] + [len(q) for q in rows]),
+                    np.array([c for q in rows for c, _ in q]),
+                    np.array([v for q in rows for _, v in q]))
+        b = b[perm]
+    kw = dict(mu_mode=1, mu_user=5.0, rmax=20, fixed_iterations=True)
+    s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_ADAPTIVE, ortho=ortho,
+                               dot_arith=G.DOT_DF32 if df32 else G.DOT_FP64, **kw)
+    xg, ig = s.solve(to_dev(b), m=15, tol=0.0, maxit=47)
+    xo, io = orc.gmres(A, b, m=15, tol=0.0, maxit=47, defl_mode=orc.DEFL_ADAPTIVE,
+                       **({"ortho": orc.MGS} if ortho else {}), **kw)
+    assert ig["iters"] == io["iters"] == 47
+    assert relerr(xg.cpu().numpy(), xo) <= (1e-7 if df32 else 1e-9)
