@@ -139,8 +139,9 @@ typedef enum {
 
 typedef enum {
   GMRES_DOT_FP64 = 0,  /* the basis multi-dot to FP64 accuracy (in the fused step as exact
-                          integer sums of fixed-point operands, 57 bits below the largest
-                          entry of each block's rows; in FP64 FMAs elsewhere) */
+                          integer sums of fixed-point operands, the basis to 61 bits of its
+                          column's largest entry, w to 54 bits of its largest in a block's
+                          rows; in FP64 FMAs elsewhere) */
   GMRES_DOT_DF32 = 1   /* the multi-dot V^T [w, v_j] of the one-reduction MGS step in
                           double-FP32 on the FP32 pipe: each FP64 operand split into two
                           floats (47 significant bits), products exact by FMA (Dekker's
@@ -185,8 +186,8 @@ typedef enum {
   GMRES_PH_PROJ_FINAL = 9,/* projector: x = xh + U T^-1 U^T (b - A xh) */
   GMRES_PH_ADAPT = 10,    /* adaptive deflation: the update of U, A U, T, T^-1 */
   GMRES_PH_MGS = 11,      /* modified Gram-Schmidt step: projections, ||w||, rotations */
-  GMRES_PH_ARNOLDI = 12,  /* a whole step in one kernel: SpMV, one-reduction MGS, ||w||,
-                             rotations (Eqs. 10, 12-14) */
+  GMRES_PH_ARNOLDI = 12,  /* a cycle's steps in one kernel: SpMV, CGS2 or one-reduction MGS,
+                             ||w||, rotations (Eqs. 10, 12-14) */
   GMRES_PH_COUNT = 13
 } gmres_phase;
 

@@ -9,10 +9,11 @@
 // 1.0, b_i = 0); the other rows keep their couplings to those columns (the pattern is the
 // mesh connectivity, which the paper's Table 1 counts).
 //
-// Assembly is row-parallel and gather-based (no atomics, bitwise deterministic): the
-// thread of row i visits the 1, 2, 4 or 8 elements around node i.  Per element it forms
-// the exp(u_h) values at the 3 x 3 x 3 Gauss-Legendre points by sum factorisation and the
-// row of the element Jacobian
+// Assembly is row-parallel and gather-based (no atomics, bitwise deterministic): a block
+// takes a brick of 8 x 8 x 4 nodes, forms w_g exp(u_h) at the 3 x 3 x 3 Gauss-Legendre points of
+// the elements around it once, contracts it in x and y with the products of basis functions, all
+// in shared memory, and the thread of row i then visits the 1, 2, 4 or 8 elements around node i
+// for the last contraction and the row of the element Jacobian
 //   J_e[l][m] = - int grad phi_m . grad phi_l + lambda int exp(u_h) phi_m phi_l,
 // the stiffness part from the exact 1-D integrals of the quadratic Lagrange functions
 // (h (S x M x M + M x S x M + M x M x S)), the exp part by the quadrature, again by sum
@@ -60,10 +61,11 @@ __device__ __forceinline__ long long q2_row_start(int n, int I, int J, int K) {
 }
 
 struct Q2Tab {
-  double P[3][3];  // P[g][a]: 1-D quadratic Lagrange function a at Gauss point g
-  double w[3];     // 1-D Gauss weights on [0, 1]
-  double S[3][3];  // exact int p_a' p_c' on [0, 1]
-  double Mm[3][3]; // exact int p_a p_c on [0, 1]
+  double P[3][3];      // P[g][a]: 1-D quadratic Lagrange function a at Gauss point g
+  double w[3];         // 1-D Gauss weights on [0, 1]
+  double S[3][3];      // exact int p_a' p_c' on [0, 1]
+  double Mm[3][3];     // exact int p_a p_c on [0, 1]
+  double PP[3][3][3];  // P[g][a] P[g][c] at [a][c][g]
 };
 
 __device__ void q2_tables(Q2Tab& t) {
@@ -84,25 +86,113 @@ __device__ void q2_tables(Q2Tab& t) {
     for (int c = 0; c < 3; ++c) {
       t.S[a][c] = S3[a][c] / 3.0;
       t.Mm[a][c] = M30[a][c] / 30.0;
+      for (int g = 0; g < 3; ++g) t.PP[a][c][g] = t.P[g][a] * t.P[g][c];
     }
 }
 
-// Row of J (values) and b = -R for the rows of the mesh; rowptr and col as well.
-__global__ void __launch_bounds__(128)
+// the brick of a block: nodes, the elements around them, the nodes of those elements
+constexpr int kQx = 8, kQy = 8, kQz = 4;
+constexpr int kQex = kQx / 2 + 1, kQey = kQy / 2 + 1, kQez = kQz / 2 + 1, kQel = kQex * kQey * kQez;
+constexpr int kQux = 2 * kQex + 1, kQuy = 2 * kQey + 1, kQuz = 2 * kQez + 1;
+constexpr int kQThreads = kQx * kQy * kQz;
+static_assert(kQThreads == 256, "a warp per class of nodes");
+// per element: E (27), then T (6 x 6 x 3, an odd stride) in its place; X (6 x 9)
+constexpr int kQT = 109, kQX = 54;
+constexpr size_t kQSmem = sizeof(double) * (27 * 27 + kQux * kQuy * kQuz + kQel * (kQT + kQX));
+
+// the six products p_a p_c (a <= c), in the order 00 01 02 11 12 22
+__device__ __forceinline__ int q2_pair(int a, int c) {
+  const int i = min(a, c), j = max(a, c);
+  return i * (5 - i) / 2 + j;
+}
+
+// Row of J (values) and b = -R for the rows of the mesh; rowptr and col as well.  Bound by the
+// FP64 pipe, so what several rows need is formed once per brick.  With the 27 exponentials of an
+// element and the contractions over its Gauss points in every row around it (some 1,500 FP64
+// operations per row and element) 9,261 rows took 400 us and 274,625 rows 3.5 ms; with the
+// exponentials and the stiffness per brick 240 us at 9,261 rows; now (189 operations) 170 us, and
+// 1.1 ms at 274,625.  A warp's nodes have the same parities, so that its lanes visit the same
+// number of elements; the warps of eight visits and of one share a scheduler.
+__global__ void __launch_bounds__(kQThreads, 2)
     k_q2_assemble(int n, double lambda, const double* __restrict__ u, int* __restrict__ rowptr,
                   int* __restrict__ col, double* __restrict__ val, double* __restrict__ b) {
+  extern __shared__ __align__(16) double sq2[];
   __shared__ Q2Tab tab;
-  if (threadIdx.x == 0) q2_tables(tab);
-  __syncthreads();
+  double* sK = sq2;                          // minus the element stiffness: [local row][local column]
+  double* su = sK + 27 * 27;                 // u at the nodes of the elements
+  double* sX = su + kQux * kQuy * kQuz;      // [element][x pair][gy, gz]
+  double* sT = sX + (size_t)kQel * kQX;      // [element][x pair][y pair][gz]
+  double* sE = sT;                           // lambda w_g h^3 exp(u_h(g)); replaced by sT
+  const int t = threadIdx.x;
   const int M = 2 * n + 1;
-  const long long N = (long long)M * M * M;
   const double h = 1.0 / n, h3 = h * h * h;
-  for (long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x; row < N;
-       row += (long long)gridDim.x * blockDim.x) {
-    const int I = (int)(row % M), J = (int)((row / M) % M), K = (int)(row / ((long long)M * M));
+  const int bx = (M + kQx - 1) / kQx, by = (M + kQy - 1) / kQy, bz = (M + kQz - 1) / kQz;
+  if (t == 0) q2_tables(tab);
+  __syncthreads();
+  for (int q = t; q < 27 * 27; q += kQThreads) {
+    const int l = q / 27, m = q % 27;
+    const int la = l % 3, lb = l / 3 % 3, lc = l / 9, a = m % 3, bb = m / 3 % 3, c = m / 9;
+    sK[q] = -h * (tab.S[la][a] * tab.Mm[lb][bb] * tab.Mm[lc][c] +
+                  tab.Mm[la][a] * tab.S[lb][bb] * tab.Mm[lc][c] +
+                  tab.Mm[la][a] * tab.Mm[lb][bb] * tab.S[lc][c]);
+  }
+  // this thread's node of a brick: parities by warp, position by lane
+  const int cls = 0x35674210 >> (4 * (t >> 5)) & 7;
+  const int ix = 2 * (t & 3) + (cls & 1), iy = 2 * (t >> 2 & 3) + (cls >> 1 & 1),
+            iz = 2 * (t >> 4 & 1) + (cls >> 2);
+  for (long long brick = blockIdx.x; brick < (long long)bx * by * bz; brick += gridDim.x) {
+    const int I0 = (int)(brick % bx) * kQx, J0 = (int)(brick / bx % by) * kQy,
+              K0 = (int)(brick / ((long long)bx * by)) * kQz;
+    // first element of the brick's neighbourhood and its first node (may lie outside)
+    const int e0x = I0 / 2 - 1, e0y = J0 / 2 - 1, e0z = K0 / 2 - 1;
+    __syncthreads();
+    for (int q = t; q < kQux * kQuy * kQuz; q += kQThreads) {
+      const int i = 2 * e0x + q % kQux, j = 2 * e0y + q / kQux % kQuy, k = 2 * e0z + q / (kQux * kQuy);
+      const bool in = i >= 0 && j >= 0 && k >= 0 && i < M && j < M && k < M;
+      su[q] = (u && in) ? u[((long long)k * M + j) * M + i] : 0.0;
+    }
+    __syncthreads();
+    for (int q = t; q < kQel * 27; q += kQThreads) {
+      const int e = q / 27, g = q % 27;
+      const int ex = e % kQex, ey = e / kQex % kQey, ez = e / (kQex * kQey);
+      const int gx = g % 3, gy = g / 3 % 3, gz = g / 9;
+      const double* ue = su + ((2 * ez) * kQuy + 2 * ey) * kQux + 2 * ex;
+      double ug = 0.0;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        double vy = 0.0;
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb) {
+          double vx = 0.0;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) vx += tab.P[gx][a] * ue[(c * kQuy + bb) * kQux + a];
+          vy += tab.P[gy][bb] * vx;
+        }
+        ug += tab.P[gz][c] * vy;
+      }
+      sE[e * 27 + g] = lambda * (tab.w[gx] * tab.w[gy] * tab.w[gz] * h3 * exp(ug));
+    }
+    __syncthreads();
+    for (int q = t; q < kQel * kQX; q += kQThreads) {
+      const int e = q / kQX, g = q % 9, pr = q / 9 % 6;
+      const int a = pr < 3 ? 0 : (pr < 5 ? 1 : 2), c = pr < 3 ? pr : (pr < 5 ? pr - 2 : 2);
+      const double* E = sE + e * 27 + 3 * g;
+      sX[q] = E[0] * tab.PP[a][c][0] + E[1] * tab.PP[a][c][1] + E[2] * tab.PP[a][c][2];
+    }
+    __syncthreads();
+    for (int q = t; q < kQel * 108; q += kQThreads) {
+      const int e = q / 108, f = q % 108, gz = f % 3, pr = f / 3 % 6, px = f / 18;
+      const int a = pr < 3 ? 0 : (pr < 5 ? 1 : 2), c = pr < 3 ? pr : (pr < 5 ? pr - 2 : 2);
+      const double* X = sX + e * kQX + px * 9 + 3 * gz;
+      sT[e * kQT + f] = X[0] * tab.PP[a][c][0] + X[1] * tab.PP[a][c][1] + X[2] * tab.PP[a][c][2];
+    }
+    __syncthreads();
+    const int I = I0 + ix, J = J0 + iy, K = K0 + iz;
+    if (I >= M || J >= M || K >= M) continue;
+    const long long row = ((long long)K * M + J) * M + I;
     const long long start = q2_row_start(n, I, J, K);
     rowptr[row] = (int)start;
-    if (row == N - 1) rowptr[N] = (int)(start + 1);
+    if (row == (long long)M * M * M - 1) rowptr[row + 1] = (int)(start + 1);
     if (I == 0 || J == 0 || I == M - 1 || J == M - 1) {  // x- and y-faces: du_i = 0
       col[start] = (int)row;
       val[start] = 1.0;
@@ -134,71 +224,32 @@ __global__ void __launch_bounds__(128)
       for (int ey = ey0; ey <= ey1; ++ey)
         for (int ex = ex0; ex <= ex1; ++ex) {
           const int la = I - 2 * ex, lb = J - 2 * ey, lc = K - 2 * ez;  // local node of the row
-          double ue[27];
-          for (int c = 0; c < 3; ++c)
-            for (int bb = 0; bb < 3; ++bb)
-              for (int a = 0; a < 3; ++a) {
-                const long long g = ((long long)(2 * ez + c) * M + 2 * ey + bb) * M + 2 * ex + a;
-                ue[a + 3 * bb + 9 * c] = u ? u[g] : 0.0;
+          const int lx = ex - e0x, ly = ey - e0y, lz = ez - e0z;        // element in the brick
+          const double* Te = sT + ((lz * kQey + ly) * kQex + lx) * kQT;
+          const double* ue = su + ((2 * lz) * kQuy + 2 * ly) * kQux + 2 * lx;
+          const double* Kl = sK + (la + 3 * lb + 9 * lc) * 27;
+          double* ve = val + start + ((2 * ez - c0) * ny + (2 * ey - b0)) * nx + (2 * ex - a0);
+          double ri = 0.0;  // lambda int exp(u) phi_l - (K_e u_e)_l
+#pragma unroll
+          for (int bb = 0; bb < 3; ++bb) {
+            const int py = q2_pair(lb, bb);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              const double* T = Te + (q2_pair(la, a) * 6 + py) * 3;
+              const double t0 = T[0], t1 = T[1], t2 = T[2];
+#pragma unroll
+              for (int c = 0; c < 3; ++c) {
+                // the functions of an element add up to one: their sum is int exp(u) phi_l
+                const double* pz = tab.PP[lc][c];
+                const double q = t0 * pz[0] + t1 * pz[1] + t2 * pz[2];
+                const double kl = Kl[a + 3 * bb + 9 * c];
+                ri += q;
+                ri += kl * ue[(c * kQuy + bb) * kQux + a];
+                ve[(c * ny + bb) * nx + a] += q + kl;
               }
-          // u_h at the Gauss points: contract x, then y, then z
-          double t1[27], t2[27];
-          for (int c = 0; c < 3; ++c)
-            for (int bb = 0; bb < 3; ++bb)
-              for (int gx = 0; gx < 3; ++gx) {
-                double s = 0.0;
-                for (int a = 0; a < 3; ++a) s += tab.P[gx][a] * ue[a + 3 * bb + 9 * c];
-                t1[gx + 3 * bb + 9 * c] = s;
-              }
-          for (int c = 0; c < 3; ++c)
-            for (int gy = 0; gy < 3; ++gy)
-              for (int gx = 0; gx < 3; ++gx) {
-                double s = 0.0;
-                for (int bb = 0; bb < 3; ++bb) s += tab.P[gy][bb] * t1[gx + 3 * bb + 9 * c];
-                t2[gx + 3 * gy + 9 * c] = s;
-              }
-          // E[g] = w_g exp(u_h(g)) phi_l(g) (row's local node l = (la, lb, lc))
-          double E[27], rexp = 0.0;
-          for (int gz = 0; gz < 3; ++gz)
-            for (int gy = 0; gy < 3; ++gy)
-              for (int gx = 0; gx < 3; ++gx) {
-                double ug = 0.0;
-                for (int c = 0; c < 3; ++c) ug += tab.P[gz][c] * t2[gx + 3 * gy + 9 * c];
-                const double e = tab.w[gx] * tab.w[gy] * tab.w[gz] * h3 * exp(ug) *
-                                 tab.P[gx][la] * tab.P[gy][lb] * tab.P[gz][lc];
-                E[gx + 3 * gy + 9 * gz] = e;
-                rexp += e;
-              }
-          // Q[m] = sum_g E[g] phi_m(g): contract gx -> a', gy -> b', gz -> c'
-          for (int gz = 0; gz < 3; ++gz)
-            for (int gy = 0; gy < 3; ++gy)
-              for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int gx = 0; gx < 3; ++gx) s += E[gx + 3 * gy + 9 * gz] * tab.P[gx][a];
-                t1[a + 3 * gy + 9 * gz] = s;
-              }
-          for (int gz = 0; gz < 3; ++gz)
-            for (int bb = 0; bb < 3; ++bb)
-              for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int gy = 0; gy < 3; ++gy) s += t1[a + 3 * gy + 9 * gz] * tab.P[gy][bb];
-                t2[a + 3 * bb + 9 * gz] = s;
-              }
-          double ku = 0.0;  // (K_e u_e)_l
-          for (int c = 0; c < 3; ++c)
-            for (int bb = 0; bb < 3; ++bb)
-              for (int a = 0; a < 3; ++a) {
-                double q = 0.0;
-                for (int gz = 0; gz < 3; ++gz) q += t2[a + 3 * bb + 9 * gz] * tab.P[gz][c];
-                const double kl = h * (tab.S[la][a] * tab.Mm[lb][bb] * tab.Mm[lc][c] +
-                                       tab.Mm[la][a] * tab.S[lb][bb] * tab.Mm[lc][c] +
-                                       tab.Mm[la][a] * tab.Mm[lb][bb] * tab.S[lc][c]);
-                ku += kl * ue[a + 3 * bb + 9 * c];
-                const int gi = 2 * ex + a, gj = 2 * ey + bb, gk = 2 * ez + c;
-                const long long slot = ((long long)(gk - c0) * ny + (gj - b0)) * nx + (gi - a0);
-                val[start + slot] += -kl + lambda * q;
-              }
-          bi -= -ku + lambda * rexp;  // b = -R, R_l = -(K u)_l + lambda int exp(u) phi_l
+            }
+          }
+          bi -= ri;
         }
     b[row] = bi;
   }
@@ -256,8 +307,13 @@ gmres_status q2_bratu_assemble(int32_t n, double lambda, const double* u, int32_
   if (!std::isfinite(lambda))
     return fail(nullptr, GMRES_ERR_INVALID_ARG, "q2_bratu_assemble: lambda must be finite");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  k_q2_assemble<<<grid_for(N, 128, 152 * 16), 128, 0, st>>>(n, lambda, u, rowptr, col, val, b);
-  const cudaError_t e = cudaGetLastError();
+  const long long bricks = ((M + kQx - 1) / kQx) * ((M + kQy - 1) / kQy) * ((M + kQz - 1) / kQz);
+  cudaError_t e = cudaFuncSetAttribute(k_q2_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kQSmem);
+  if (e != cudaSuccess) return cuda_fail(nullptr, e, "q2_bratu_assemble");
+  k_q2_assemble<<<grid_for(bricks, 1, 152 * 16), kQThreads, kQSmem, st>>>(n, lambda, u, rowptr, col,
+                                                                        val, b);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "q2_bratu_assemble");
   return GMRES_OK;
 }

@@ -20,8 +20,7 @@
 //      totals in every block) and solves (I + L) h = g itself.
 //   4. Update of its rows, u_{j+1} = w - V (sigma o h), in the reverse order of step 2 (the
 //      columns read last are the likeliest to be in L2; FP64 in fixed point); partial sums of
-//      ||u_{j+1}||^2 and
-//      of u_{j+1} over the block's pieces of aggregates (U^T u_{j+1}).
+//      ||u_{j+1}||^2 and of u_{j+1} over the block's pieces of aggregates (U^T u_{j+1}).
 //   5. Grid barrier 2; block 0 adds the norm partials and applies the rotations and the
 //      stopping tests; the other blocks form c = U^T u_{j+1} from the piece sums and share
 //      the rows of y = T^-1 c, giving s' for step j + 1.
@@ -32,8 +31,11 @@
 // first update w -= V h with the second multi-dot h' = V^T w (a pass over each super-tile's
 // rows, w' in shared memory in between), one more grid barrier, and coefficients h + h'.
 // Every reduction is formed in a fixed order: runs are bitwise reproducible.  The per-phase
-// register budgets (loads in flight) are set so that the kernel needs no local memory:
-// with 220 KB of shared memory per block, spilled registers would live in L2.
+// register budgets (loads in flight) are set so that no loop needs local memory: with 220 KB
+// of shared memory per block, spilled registers would live in L2.
+//
+// The batched form (k_arnoldi_batch) runs the same cycle for one system per thread-block
+// cluster, whose hardware barrier takes the place of the grid barriers.
 //
 // The basis is streamed with plain vectorised loads rather than bulk asynchronous copies:
 // measured on GB300, a multiprocessor fed by bulk copies reached about 10 bytes per clock,
@@ -756,8 +758,10 @@ __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long lo
 
 // The same rows of a CSR operator: a thread per row (ten entries' loads, then their gathers, in
 // flight at once), or 8 lanes per row for long rows (two rows of up to 64 entries in flight per
-// lane group; 4 lanes: 24.8 against 22.2 ms on the 274,625-unknown Bratu matrix, 100 steps).  With one block of 16 warps per multiprocessor the loads in flight per thread
-// stand in for the occupancy of a kernel of its own.
+// lane group; 4 lanes: 24.8 against 22.2 ms on the 274,625-unknown Bratu matrix, 100 steps).  With
+// one block of 16 warps per multiprocessor the loads in flight per thread stand in for the
+// occupancy of a kernel of its own.  Sharing the long rows out by entries instead of the basis'
+// row ranges, through w in global memory, did not pay (19.9 against 19.7 ms).
 template <typename TV, typename TACC>
 __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj, long long s0,
                                         long long s1, TACC* Ws, TACC* Us, int tid, int nthr) {

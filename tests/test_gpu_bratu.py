@@ -150,3 +150,15 @@ def test_newton_rejects_bad_arguments(G, orc):
         G.bratu_newton(0, LAM)
     with pytest.raises(G.GmresError):
         G.q2_bratu_assemble(2, float("nan"), device="cuda")
+
+
+# meshes whose nodes end inside, at and one past a brick of 8 x 8 x 4 nodes
+@pytest.mark.parametrize("n", [5, 7, 8, 9])
+def test_assembly_at_brick_edges(G, orc, n):
+    u = _u(n, 20 + n) * 0.4
+    A, b = orc.q2_bratu_assemble(n, LAM, u)
+    rp, cl, vl, bg = G.q2_bratu_assemble(n, LAM, to_dev(u))
+    assert np.array_equal(rp.cpu().numpy(), A.rowptr)
+    assert np.array_equal(cl.cpu().numpy(), A.col)
+    assert np.abs(vl.cpu().numpy() - A.val).max() <= 1e-13 * np.abs(A.val).max()
+    assert np.abs(bg.cpu().numpy() - b).max() <= 1e-13 * np.abs(b).max()
