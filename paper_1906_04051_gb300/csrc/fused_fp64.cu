@@ -1,5 +1,7 @@
 // fused_fp64.cu -- the fused Arnoldi cycle (fused.cuh) with an FP64 basis, and the rule that says
 // which solves it takes.
+#include <climits>
+
 #include "fused.cuh"
 
 namespace gg {
@@ -7,12 +9,33 @@ namespace gg {
 cudaError_t launch_arnoldi_fp32(const CycleArgs& a, int jmax, bool defl, cudaStream_t st);
 cudaError_t launch_arnoldi_bf16(const CycleArgs& a, int jmax, bool defl, cudaStream_t st);
 
+// Most rows (padded) up to which the fused cycle is the faster one; us a step against one kernel
+// per phase, 40 to 50 columns:
+//   FP64 diagonals, CGS2     4,225 rows 35 / 51, 262k 98 / 152, 4M 652 / 900
+//   FP64 CSR, CGS2           238k 77 / 133, 2.25M 508 / 595, 4M 871 / 913
+//   FP64 CSR, one reduction  238k 61 / 115, 2.25M 395 / 472, 4M 635 / 700
+//   FP32 diagonals, CGS2     1.44M 121 / 148, 2.9M 240 / 243, 3.2M 280 / 266
+//   FP32 CSR, CGS2           90k 38 / 51, 1M 111 / 119, 2.6M 271 / 229
+//   FP32 CSR, one reduction  90k 29 / 44, 2.6M 192 / 195, 4M 304 / 277
+//   BF16 diagonals, CGS2     1M 95 / 107, 1.44M 124 / 137, 1.96M 171 / 167, 4M 361 / 289
+//   long rows (hexahedra)    36k 48 / 66, 275k 173 / 185 (BF16 122 / 119), 531k 300 / 283,
+//                            1.77M 907 / 782
+// Past these sizes the phases stream: the per-phase kernels have more loads in flight than one
+// block of 16 warps per multiprocessor, and with long rows the SpMV outweighs the rest of the
+// step.  FP64 dots and updates stay ahead, being fixed point here and FP64 multiply-adds there.
+long long fused_rows(const CycleArgs& a) {
+  const bool csr = a.op.dia.nd == 0, cgs2 = a.ortho == GMRES_ORTHO_CGS2;
+  if (a.op.vec) return a.prec == P_BF16 ? 200000 : 350000;
+  if (a.prec == P_FP64) return csr ? 4500000 : LLONG_MAX;
+  if (csr) return cgs2 ? 1200000 : 2600000;
+  if (!cgs2) return LLONG_MAX;
+  return a.prec == P_BF16 ? 1700000 : 2600000;
+}
+
 // CGS2 or the one-reduction MGS, EBP deflation by aggregates or none (no projector, no dense
-// deflation space); BF16 bases with CGS2.  Against one kernel per phase (CGS2, FP64, 9-point
-// stencils): 51 to 35 us a step at 4,225 unknowns, 152 to 98 us at 262k; thread-per-row CSR, 238k
-// unknowns: 112 to 75 us; long rows (3-D hexahedra, 275k unknowns): 196 to 190 us; BF16 basis,
-// 362k unknowns: 92 to 85 us.
+// deflation space); BF16 bases with CGS2.
 bool arnoldi_fusable(const CycleArgs& a) {
+  if (a.ldv > fused_rows(a)) return false;
   if (a.proj || a.op.defl.qd != 0 || a.ldv % kArnUnit != 0 || a.m + 1 > kMaxK) return false;
   if (a.ortho != GMRES_ORTHO_CGS2 && !(a.ortho == GMRES_ORTHO_MGS_LOWSYNC && a.prec != P_BF16))
     return false;

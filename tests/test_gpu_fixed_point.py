@@ -132,3 +132,16 @@ def test_adaptive_space_from_a_fused_cycle(G, orc, n, kind, ortho, df32):
                        **({"ortho": orc.MGS} if ortho else {}), **kw)
     assert ig["iters"] == io["iters"] == 47
     assert relerr(xg.cpu().numpy(), xo) <= (1e-7 if df32 else 1e-9)
+
+
+# long rows on both sides of the size up to which their cycles are fused (328,509 and 357,911 rows)
+@pytest.mark.parametrize("n", [34, 35])
+@pytest.mark.parametrize("ortho", [0, 2])
+def test_long_rows_at_the_fused_limit(G, orc, n, ortho):
+    A, b = orc.q2_bratu_assemble(n, 3.0, np.zeros((2 * n + 1) ** 3))
+    s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_NONE, fixed_iterations=True, ortho=ortho)
+    xg, ig = s.solve(to_dev(b), m=6, tol=0.0, maxit=9)
+    xo, _ = orc.gmres(A, b, m=6, tol=0.0, maxit=9, fixed_iterations=True,
+                      **({"ortho": orc.MGS} if ortho else {}))
+    assert ig["iters"] == 9
+    assert relerr(xg.cpu().numpy(), xo) <= 1e-9
