@@ -1704,15 +1704,17 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
       if (sizeof(TV) == 8 && R0 == R1)
         for (int c = t; c < k; c += kArnThreads) sred[c] = 0.0;
       arn_block_sums<TV, MODE>(sbuf, k, k, sred);
-      for (int c = t; c < k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
+      // (columns of their own: another block may still be adding up the first dots' partials)
+      double* const part2 = ctl.part + kMaxK;
+      for (int c = t; c < k; c += kArnThreads) __stcg(&part2[(size_t)bid * ctl.ldp + c], sred[c]);
       if (!arn_grid_sync<CL>(a.gbar, gen++)) {
         arn_timeout(ctl);
         return;
       }
       if constexpr (sizeof(TV) < 8)
-        arn_reduce_cols_df<24>(ctl.part, G, k, ctl.ldp, tot);
+        arn_reduce_cols_df<24>(part2, G, k, ctl.ldp, tot);
       else
-        arn_reduce_cols(ctl.part, G, k, ctl.ldp, tot);
+        arn_reduce_cols(part2, G, k, ctl.ldp, tot);
       for (int c = t; c < k; c += kArnThreads) {
         const double h2 = ssig[c] * tot[c];
         scoef[c] = (TACC)(ssig[c] * h2);
