@@ -1616,7 +1616,8 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
   }
   // FP32 basis: the coarse solve's static data for the cycle (the aggregates' piece ranges,
   // their scales, this block's rows of T^-1 when every warp has at most one) staged once in
-  // shared memory past the rows of w's slice, when it fits
+  // shared memory, when it fits: past the rows of w's slice and past c, which the coarse solve
+  // forms at the start of that slice (r entries, more than the rows of a small system's block)
   int* sap = nullptr;       // agg_piece, r + 1
   float* sus = nullptr;     // uscale, r
   float* stinv = nullptr;   // the block's rows of T^-1 (warp w: row (b - 1) + (G - 1) w)
@@ -1625,8 +1626,9 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
     const int rows = (a.defl && bid > 0 && a.r <= nwr && bid - 1 < a.r)
                          ? min(kArnWarps, (a.r - (bid - 1) + G - 2) / (G - 1)) : 0;
     const size_t need = (size_t)(a.r + 1) * 4 + (size_t)a.r * 4 + (size_t)rows * a.r * 4;
-    if (a.defl && G > 1 && a.RS > nrows && (size_t)(a.RS - nrows) * sizeof(TACC) >= need + 16) {
-      sap = reinterpret_cast<int*>(Ws + nrows);
+    const long long at = nrows > a.r ? nrows : a.r;
+    if (a.defl && G > 1 && a.RS > at && (size_t)(a.RS - at) * sizeof(TACC) >= need + 16) {
+      sap = reinterpret_cast<int*>(Ws + at);
       sus = reinterpret_cast<float*>(sap + a.r + 1);
       stinv = rows > 0 ? sus + a.r : nullptr;
       for (int q = t; q <= a.r; q += kArnThreads) sap[q] = __ldg(a.agg_piece + q);

@@ -40,3 +40,59 @@ def test_cgs2_solves_repeat_bitwise(G, orc, n, m, prec):
     if prec == 0:
         xo, _ = orc.gmres(A, b, m=m, tol=0.0, maxit=4 * m, defl=orc.Deflation(A, p.agg, p.r), **kw)
         assert relerr(first.cpu().numpy(), xo) <= 1e-9
+
+
+def _aggregates(n, px, py):
+    j, i = np.divmod(np.arange((n + 1) ** 2), n + 1)
+    return ((j * py // (n + 1)) * px + i * px // (n + 1)).astype(np.int32)
+
+
+# the coarse solve of the FP32 one-reduction step over diagonals: more aggregates than rows in a
+# block (its vector c then reaches past the rows of w's slice, where its tables used to start),
+# as many, and fewer.  20 steps in FP32: 20 x 2^-24 x the condition of the projected problem, some
+# 1e-4 at most; a wrong coarse term changes the first digit
+@pytest.mark.parametrize("n,px,py", [(64, 16, 16), (64, 16, 8), (64, 43, 3), (40, 13, 12), (90, 8, 8)])
+def test_fp32_coarse_tables(G, orc, n, px, py):
+    p = W.convdiff(n, pe=20.0, sigma=0.5, seed=n, px=1, py=1)
+    A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+    agg, r = _aggregates(n, px, py), px * py
+    kw = dict(mu_mode=1, mu_user=4.0)
+    s = gpu_solver_from_oracle(G, A, agg, r, ortho=G.ORTHO_MGS_LOWSYNC, precision=G.FP32_INNER,
+                               fixed_iterations=True, **kw)
+    xo, _ = orc.gmres(A, b, m=20, tol=0.0, maxit=20, defl=orc.Deflation(A, agg, r), ortho=orc.MGS,
+                      fixed_iterations=True, **kw)
+    first = None
+    for _ in range(10):
+        x, info = s.solve(to_dev(b), m=20, tol=0.0, maxit=20)
+        assert info["iters"] == 20
+        first = x.clone() if first is None else first
+        assert torch.equal(x, first)
+    assert relerr(first.cpu().numpy(), xo) <= 1e-3
+
+
+# the same in clusters (banded systems only, 16 rows and more a side: one operator form): blocks
+# without any rows (4 to 14 units of rows among 16 blocks), with fewer and with more than r
+@pytest.mark.parametrize("count,px", [(1, 2), (3, 2), (3, 11), (8, 5), (40, 3)])
+def test_fp32_coarse_tables_in_clusters(G, orc, count, px):
+    kw = dict(mu_mode=1, mu_user=4.0)
+    sys, ss = [], []
+    for i in range(count):
+        n = [20, 16, 40, 33, 24][i % 5]
+        p = W.convdiff(n, pe=15.0, sigma=0.4, seed=60 + i, px=1, py=1)
+        A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+        agg = _aggregates(n, px, px)
+        sys.append((A, b, agg))
+        ss.append(gpu_solver_from_oracle(G, A, agg, px * px, ortho=G.ORTHO_MGS_LOWSYNC,
+                                         precision=G.FP32_INNER, fixed_iterations=True, **kw))
+        assert ss[-1].layout()["ndiag"] == 9
+    bs = [to_dev(b) for _, b, _ in sys]
+    first = None
+    for _ in range(5):
+        xs, infos, _ = G.batch_solve(ss, bs, m=15, tol=0.0, maxit=15)
+        assert all(i["iters"] == 15 for i in infos)
+        first = [x.clone() for x in xs] if first is None else first
+        assert all(torch.equal(x, y) for x, y in zip(xs, first))
+    for x, (A, b, agg) in zip(first, sys):
+        xo, _ = orc.gmres(A, b, m=15, tol=0.0, maxit=15, defl=orc.Deflation(A, agg, px * px),
+                          ortho=orc.MGS, fixed_iterations=True, **kw)
+        assert relerr(x.cpu().numpy(), xo) <= 1e-3
