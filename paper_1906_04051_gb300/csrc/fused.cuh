@@ -1486,10 +1486,15 @@ __device__ __forceinline__ int arn_get_max(const Ctl& ctl, int G) {
 }
 
 // The 16 warps' pairs of ncols columns (sets of k) in warp order: double-FP32 multi-dots of an
-// FP64 basis rounded to FP64 once, sums of an FP32 or BF16 basis kept as pairs
+// FP64 basis rounded to FP64 once, sums of an FP32 or BF16 basis kept as pairs.  A block without
+// rows (none: some blocks of a small system's cluster) has passed no barrier since the pairs were
+// cleared, so it does not read them.
 template <typename TV, int MODE>
-__device__ __forceinline__ void arn_block_sums(const double* sbuf, int ncols, int k, double* sred) {
-  if constexpr (sizeof(TV) == 8 && MODE == kArnLowsyncDf) {
+__device__ __forceinline__ void arn_block_sums(const double* sbuf, int ncols, int k, bool none,
+                                               double* sred) {
+  if (none) {
+    for (int q = threadIdx.x; q < ncols; q += kArnThreads) sred[q] = 0.0;
+  } else if constexpr (sizeof(TV) == 8 && MODE == kArnLowsyncDf) {
     for (int q = threadIdx.x; q < ncols; q += kArnThreads) {
       const int set = q / k, c = q % k;
       const float* dfp = reinterpret_cast<const float*>(sbuf);
@@ -1674,10 +1679,8 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
       for (int q = t; q < 2 * kMaxK * 33; q += kArnThreads) sbuf[q] = 0.0;
     arn_front<TV, TACC, ND, MODE>(a, g, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sE, semax, sred);
     waited = true;
-    if (sizeof(TV) == 8 && R0 == R1)  // a block without rows (a small system's cluster)
-      for (int c = t; c < NSET * k; c += kArnThreads) sred[c] = 0.0;
     // per-block column sums (fixed order; a fixed-point multi-dot leaves them in sred)
-    arn_block_sums<TV, MODE>(sbuf, NSET * k, k, sred);
+    arn_block_sums<TV, MODE>(sbuf, NSET * k, k, R0 == R1, sred);
     // the partials: FP64 values, or double-FP32 pairs (two floats in the slot) for an FP32 or
     // BF16 basis, whose cross-block sums then run on the FP32 pipe
     for (int c = t; c < NSET * k; c += kArnThreads) __stcg(&ctl.part[(size_t)bid * ctl.ldp + c], sred[c]);
@@ -1703,9 +1706,7 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
       } else {
         arn_pass2_rows<TV, TACC, ND>(a, g, k, Ws, scoef, sbuf);
       }
-      if (sizeof(TV) == 8 && R0 == R1)
-        for (int c = t; c < k; c += kArnThreads) sred[c] = 0.0;
-      arn_block_sums<TV, MODE>(sbuf, k, k, sred);
+      arn_block_sums<TV, MODE>(sbuf, k, k, R0 == R1, sred);
       // (columns of their own: another block may still be adding up the first dots' partials)
       double* const part2 = ctl.part + kMaxK;
       for (int c = t; c < k; c += kArnThreads) __stcg(&part2[(size_t)bid * ctl.ldp + c], sred[c]);

@@ -96,3 +96,32 @@ def test_fp32_coarse_tables_in_clusters(G, orc, count, px):
         xo, _ = orc.gmres(A, b, m=15, tol=0.0, maxit=15, defl=orc.Deflation(A, agg, px * px),
                           ortho=orc.MGS, fixed_iterations=True, **kw)
         assert relerr(x.cpu().numpy(), xo) <= 1e-3
+
+
+# blocks of a cluster without any rows (systems of 2 to 6 units of 128 rows among 8 or 16 blocks)
+# add nothing to the dots, from the first step of the first cycle on: against the FP64 oracle, with
+# the tolerance of the basis precision (2^-24 or 2^-8 a step, 8 steps, projected problems of
+# condition below 100), and bitwise over fresh handles, whose workspaces hold something else
+@pytest.mark.parametrize("ortho,prec", [(0, 1), (1, 1), (0, 2)])
+@pytest.mark.parametrize("count", [1, 5, 12])
+def test_blocks_without_rows(G, orc, count, ortho, prec):
+    sys = []
+    for i in range(count):
+        n = [16, 20, 24][i % 3]
+        p = W.convdiff(n, pe=5.0, sigma=0.4, seed=80 + i, px=1, py=1)
+        sys.append(orc.q1_assemble(p.n, p.kappa, p.beta, p.f))
+    o = G.ORTHO_MGS_LOWSYNC if ortho else G.ORTHO_CGS2
+    first = None
+    for _ in range(4):
+        ss = [gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_NONE, ortho=o, precision=prec,
+                                     fixed_iterations=True) for A, _ in sys]
+        xs, infos, _ = G.batch_solve(ss, [to_dev(b) for _, b in sys], m=8, tol=0.0, maxit=8)
+        assert all(i["iters"] == 8 for i in infos)
+        first = [x.clone() for x in xs] if first is None else first
+        assert all(torch.equal(x, y) for x, y in zip(xs, first))
+        for s in ss:
+            s.close()
+    for x, (A, b) in zip(first, sys):
+        xo, _ = orc.gmres(A, b, m=8, tol=0.0, maxit=8, fixed_iterations=True,
+                          **({"ortho": orc.MGS} if ortho else {}))
+        assert relerr(x.cpu().numpy(), xo) <= (1e-4 if prec == 1 else 0.2)
