@@ -977,23 +977,32 @@ __global__ void __launch_bounds__(kSpmvRows)
 // by repeated squaring, rho = lim ||H^m||^(1/m) (Gelfand).  With N_0 = H, e_i the exponent of
 // N_i's largest entry and N_{i+1} = (N_i 2^-e_i)^2, log2 rho = sum_i e_i 2^-i: after p squarings
 // the rest is log2 ||.|| 2^-p, below the rounding of the sum at p = 56 for any matrix of order
-// 64, real or complex dominant eigenvalue, simple or not.  A rounding error of squaring i enters
-// log rho halved i times over, so the result is as accurate as an eigenvalue from the QR
-// algorithm (backward error times the eigenvalue's condition number).
-// The Francis QR iteration in one warp this replaces is a chain of some 10^5 dependent FP64
-// operations (4.2 ms at k = 50); here a cluster of 8 blocks shares the rows of each square, every
-// block keeping the whole matrix in shared memory (0.41 ms at k = 50).
+// 64, real or complex dominant eigenvalue, simple or not.
+// A squaring's rounding error is relative to ||N_i||^2, not to rho(N_i)^2, so the estimate is only
+// as good as the powers of H are close to rho's: with 2^g_i = ||N_i|| / rho(N_i) (a Kreiss bound:
+// the spectral radius moves by at most the powers' growth times the error) its relative error is
+// some 2^(3 g - 53) k.  The finite-element operators here stay at g = 0 up to Peclet numbers of
+// 1e5; dense triangular operators with entries as large as their diagonal reach g = 8 to 25, where
+// squaring is off by 1e-10 to tens of percent.  Past kRitzGrowth (or when the squares vanish) the
+// Francis QR iteration in one warp gives the estimate, as in a batch (its backward error is
+// relative to ||H||).
+// QR is a chain of some 10^5 dependent FP64 operations (4.2 ms at k = 50); squaring shares the
+// rows of each square over a cluster of 8 blocks, every block keeping the whole matrix in shared
+// memory (0.41 ms at k = 50).
 // --------------------------------------------------------------------------------------
 constexpr int kRitzCluster = 8;
 constexpr int kRitzThreads = 512;                      // 8 rows x 64 columns
 constexpr int kRitzSquarings = 56;
-constexpr int kRitzRows = kMaxM / kRitzCluster;
+constexpr double kRitzGrowth = 3.0;                    // largest g_i the squares are trusted with
 constexpr size_t kRitzSmem = 2 * kMaxM * kMaxM * sizeof(double);
 
 __global__ void __cluster_dims__(kRitzCluster, 1, 1) __launch_bounds__(kRitzThreads)
     k_ritz(Ctl ctl) {
   extern __shared__ __align__(16) double sN[];  // two copies, alternating
   __shared__ int smax[kRitzThreads / 32];
+  __shared__ int sexp[kRitzSquarings + 1];
+  __shared__ double smod;
+  __shared__ int sfail;
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   if (ctl.flags[F_STOP]) return;  // the same in every block
@@ -1013,7 +1022,7 @@ __global__ void __cluster_dims__(kRitzCluster, 1, 1) __launch_bounds__(kRitzThre
   const bool live = t / kMaxM < rows && i < n && (j & ~31) < n;
   double s = 0.0, w = 1.0;
   int e0 = 0;
-  bool ok = true;
+  bool ok = true, finite = true;
   for (int p = 0; p <= kRitzSquarings; ++p) {
     const double* N = sN + (p & 1) * (kMaxM * kMaxM);
     // the largest exponent (the high words order like the magnitudes)
@@ -1026,9 +1035,11 @@ __global__ void __cluster_dims__(kRitzCluster, 1, 1) __launch_bounds__(kRitzThre
     m = __reduce_max_sync(0xffffffffu, m);
     if ((m >> 20) == 0 || (m >> 20) == 2047) {  // zero (nilpotent H) or not finite
       ok = false;
+      finite = (m >> 20) == 0;
       break;  // the same in every block: all hold the same matrix
     }
     const int e = (m >> 20) - 1023;
+    if (t == 0) sexp[p] = e;
     if (p == 0) e0 = e;  // kept apart: the fraction then keeps all its bits
     else s += w * e;
     w *= 0.5;
@@ -1058,8 +1069,18 @@ __global__ void __cluster_dims__(kRitzCluster, 1, 1) __launch_bounds__(kRitzThre
     cl.sync();
   }
   cl.sync();  // no block leaves while another may still write to it
-  if (rank == 0 && t == 0) {
-    const double mu = ok ? ldexp(exp2(s), e0) : 0.0;
+  if (rank != 0 || t >= 32) return;
+  // largest growth: rho(N_i 2^-e_i) = 2^-g_i, so g_i = (g_{i+1} - e_{i+1}) / 2, from g = 0 at the end
+  __syncwarp();
+  double g = 0.0, gmax = 0.0;
+  for (int p = ok ? kRitzSquarings : 0; p > 0; --p) {
+    g = 0.5 * (g - sexp[p]);
+    gmax = fmax(gmax, g);
+  }
+  const double mu = ok ? ldexp(exp2(s), e0) : 0.0;
+  if (finite && (!ok || gmax > kRitzGrowth)) {
+    ritz_warp(ctl, sN, smod, sfail);
+  } else if (t == 0) {
     if (!(mu > 0.0) || !isfinite(mu)) {
       ctl.flags[F_STATUS] = GMRES_ERR_SINGULAR_COARSE;
       ctl.flags[F_STOP] = 1;

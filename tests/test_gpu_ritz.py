@@ -42,3 +42,24 @@ def test_nilpotent_matrix_has_no_estimate(G, orc):
     with pytest.raises(G.GmresError) as e:
         s.solve(to_dev(b), m=8, tol=1e-8, maxit=100)
     assert e.value.status == -4
+
+
+# dense upper triangular operators: the powers of H_k grow by 2^1.7 to 2^20 before they settle, where
+# squaring alone is off by 1e-10 to 3e-2 (all but the first).  The tolerances are some hundred times
+# what relative perturbations of 2e-15 in H_k move the spectral radius by (4e-15, 2e-12, 3e-12, 2e-8)
+@pytest.mark.parametrize("n,m,off,tol", [(30, 12, 1.0, 1e-12), (24, 16, 1.0, 2e-10),
+                                         (200, 40, 0.2, 3e-10), (40, 33, 0.7, 2e-6)])
+def test_strongly_non_normal(G, orc, n, m, off, tol):
+    rng = np.random.default_rng(n * 100 + m)
+    T = np.triu(rng.standard_normal((n, n)), 1) * off + np.diag(rng.uniform(0.5, 1.5, n))
+    b = rng.standard_normal(n)
+    A = orc.CSR(np.concatenate([[0], np.cumsum(np.arange(n, 0, -1))]),
+                np.concatenate([np.arange(i, n) for i in range(n)]),
+                np.concatenate([T[i, i:] for i in range(n)]))
+    agg = np.zeros(n, dtype=np.int32)
+    s = gpu_solver_from_oracle(G, A, agg, 1)
+    _, ig = s.solve(to_dev(b), m=m, tol=1e-30, maxit=m)
+    _, io = orc.gmres(A, b, defl=orc.Deflation(A, agg, 1), m=m, tol=1e-30, maxit=m)
+    assert ig["mu"] == pytest.approx(io["mu"], rel=tol)
+    _, ib, _ = G.batch_solve([s], [to_dev(b)], m=m, tol=1e-30, maxit=m)
+    assert ib[0]["mu"] == pytest.approx(io["mu"], rel=tol)
