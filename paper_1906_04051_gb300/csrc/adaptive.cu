@@ -207,11 +207,12 @@ __global__ void k_adapt_z(Ctl ctl, int ninv, double* __restrict__ zout, int* __r
 }
 
 // u = V_k z (the basis columns as stored, v_c = sigma_c u_c: z is scaled by sigma here).
-// FIX: the cycle left its columns in fixed point (fixed.cuh), whose units go into z as well.
+// FIX: the cycle left its columns in fixed point (fixed.cuh), whose units go into z and whose rows'
+// shifts scale the sum.
 template <bool FIX>
 __global__ void __launch_bounds__(kThreads)
     k_adapt_vz(int N, const double* __restrict__ V, long long ldv, const double* __restrict__ z,
-               Ctl ctl, double* __restrict__ u) {
+               const short* __restrict__ shifts, Ctl ctl, double* __restrict__ u) {
   __shared__ double sz[kMaxK];
   const int k = ctl.flags[F_K];
   for (int c = threadIdx.x; c < k; c += blockDim.x) {
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(kThreads)
       const double v = V[(size_t)c * ldv + i];
       s += (FIX ? (double)__double_as_longlong(v) : v) * sz[c];
     }
-    u[i] = s;
+    u[i] = FIX ? ldexp(s, -__ldg(shifts + i)) : s;
   }
 }
 
@@ -717,10 +718,10 @@ gmres_status adapt_update(gmres_s* h, CycleArgs& a) {
   for (int v = 0; v < nvec; ++v) {
     if (a.fixv)
       k_adapt_vz<true><<<grid, kThreads, 0, st>>>(N, static_cast<const double*>(a.V), ld,
-                                                  z + (size_t)v * kMaxK, ctl, u);
+                                                  z + (size_t)v * kMaxK, fx_shifts(a), ctl, u);
     else
       k_adapt_vz<false><<<grid, kThreads, 0, st>>>(N, static_cast<const double*>(a.V), ld,
-                                                   z + (size_t)v * kMaxK, ctl, u);
+                                                   z + (size_t)v * kMaxK, nullptr, ctl, u);
     k_adapt_norm<<<grid, kThreads, 0, st>>>(N, u, ctl, nrm);
     nl += 2;
     for (int pass = 0; pass < 2 && q > 0; ++pass) {

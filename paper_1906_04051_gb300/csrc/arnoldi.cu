@@ -860,11 +860,14 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// The same from a basis in fixed point (fixed.cuh): integer sums, two rows per thread.  Bound by
+// The same from a basis in fixed point (fixed.cuh): integer sums, two rows per thread, the rows'
+// shifts from the basis' last column (a cycle of no steps leaves that column as it was: any
+// shift within the exponent's range will do for sums of nothing).  Bound by
 // the basis loads (FP64 multiply-adds: 111 us per cycle at 1M rows and 50 columns).
 template <bool DEFL>
 __global__ void __launch_bounds__(kThreads)
-    k_xupdate_fx(int N, const long long* __restrict__ V, long long ldv, double* __restrict__ x,
+    k_xupdate_fx(int N, const long long* __restrict__ V, long long ldv,
+                 const short* __restrict__ shifts, double* __restrict__ x,
                  double* __restrict__ t, Ctl ctl) {
   if (ctl.flags[F_STOP]) return;
   __shared__ int4 sK[kMaxK];
@@ -888,8 +891,10 @@ __global__ void __launch_bounds__(kThreads)
       fx_axpy(a1, fx_limbs(v.z, v.w), kc);
     }
     double* out = DEFL ? t : x;
-    out[r] = fx_axpy_add(a0, DEFL ? 0.0 : x[r], scale);
-    if (r + 1 < N) out[r + 1] = fx_axpy_add(a1, DEFL ? 0.0 : x[r + 1], scale);
+    const short2 sh = __ldg(reinterpret_cast<const short2*>(shifts + r));
+    const double c0 = scale * fx_pow2(sh.x & 1023), c1 = scale * fx_pow2(sh.y & 1023);
+    out[r] = fx_axpy_add(a0, DEFL ? 0.0 : x[r], c0);
+    if (r + 1 < N) out[r + 1] = fx_axpy_add(a1, DEFL ? 0.0 : x[r + 1], c1);
   }
 }
 
@@ -1237,8 +1242,8 @@ struct Kern {
     if constexpr (sizeof(TV) == sizeof(double)) {
       if (a.fixv) {
         k_xupdate_fx<DEFL><<<grid_for((N + 2 * kThreads - 1) / (2 * kThreads), 1, 8 * a.sms),
-                             kThreads, 0, st>>>(N, static_cast<const long long*>(a.V), a.ldv, x,
-                                                a.t, a.ctl);
+                             kThreads, 0, st>>>(N, static_cast<const long long*>(a.V), a.ldv,
+                                                fx_shifts(a), x, a.t, a.ctl);
         return;
       }
     }

@@ -656,8 +656,11 @@ __global__ void __launch_bounds__(kThreads) kb_xupdate_fx(BTab tab) {
     FxAcc a{0, 0, 0, 0};
 #pragma unroll 8
     for (int c = 0; c < k; ++c) fx_axpy(a, fx_limbs(__ldg(V + (size_t)c * S.ldv)), sK[c]);
-    if (S.ctl.flags[F_DEFL_ON]) S.t[row] = fx_axpy_add(a, 0.0, sscale);
-    else S.x[row] = fx_axpy_add(a, S.x[row], sscale);
+    const short* sh = reinterpret_cast<const short*>(static_cast<const double*>(S.V) +
+                                                     (size_t)tab.m * S.ldv);  // (as k_xupdate_fx)
+    const double scale = sscale * fx_pow2(__ldg(sh + row) & 1023);
+    if (S.ctl.flags[F_DEFL_ON]) S.t[row] = fx_axpy_add(a, 0.0, scale);
+    else S.x[row] = fx_axpy_add(a, S.x[row], scale);
   }
 }
 

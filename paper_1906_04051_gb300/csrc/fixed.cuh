@@ -7,10 +7,18 @@
 // to their fixed-point unit and the rounding of the total.
 //
 // A basis column is held as 64-bit integers M relative to its largest exponent E (of the whole
-// column): v = M 2^(E - 1083), |M| <= 2^61, rounded to nearest.  Entries within 2^8 of the
-// column's largest are exact, the rest are rounded 8 bits below the FP64 spacing of the largest.
+// column) and to a shift S of the row: v = M 2^(E - S - 1083), |M| <= 2^61, rounded to nearest.
 // M = h 2^32 + l, l signed.  Converting in every pass cost some 15 integer operations per
 // element, more than the multiplications, so a column is converted once, in place.
+//
+// The row's shift (fx_shift) is 0 where its entries come within 2^8 of their columns' largest: these
+// are exact there and rounded 8 bits below the FP64 spacing of the largest elsewhere.  A row that
+// stays far below its columns' largest (an uncoupled block of a system, say, whose right-hand side
+// is small) gets a shift that gives its first nonzero entry all 53 bits; when a later column has a
+// larger entry there, the row's shift shrinks and its earlier entries are rounded to the new unit.
+// So a row's rounding errors are relative to the largest of its own entries (each in units of its
+// column's largest), as those of an FP64 sum over the row are.  Without shifts, a block 2^66 below
+// the rest of the system lost all but 10 digits.  A dot takes the other operand times 2^-S.
 //
 // Dots (fx_operand, fx_dot, fx_warp_sum, fx_value): the other operand W = wh 2^28 + wl, |W| <=
 // 2^54, relative to the largest exponent of its piece.  An error in a projection coefficient
@@ -24,7 +32,7 @@
 // column scales only: rows that hold equal values (the Dirichlet rows of an aggregate, say) keep
 // equal values, as with FP64 multiply-adds.
 //
-// Zeros convert to zeros; an infinity or a NaN shows in the largest exponent (2047), and the
+// Zeros convert to zeros whatever the shift; an infinity or a NaN shows in the largest exponent (2047), and the
 // result is then NaN.
 #pragma once
 
@@ -43,17 +51,39 @@ __device__ __forceinline__ int fx_mag(double v) { return __double2hiint(v) & 0x7
 // v's biased exponent
 __device__ __forceinline__ long long fx_round(double v, int e) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  const unsigned sh = (unsigned)(e - 1 - (int)((hi << 1) >> 21));
-  // significand with its leading one at bit 63, shifted down to one bit more than the result
-  const unsigned a = __funnelshift_l(lo, hi, 11) | 0x80000000u, b = lo << 11;
+  const int ex = (int)((hi << 1) >> 21);
+  const unsigned sh = (unsigned)(e - 1 - max(ex, 1));
+  // significand with its leading one (a zero or subnormal value has none) at bit 63, shifted down
+  // to one bit more than the result
+  const unsigned a = __funnelshift_l(lo, hi, 11) | (ex ? 0x80000000u : 0u), b = lo << 11;
   unsigned long long x = ((unsigned long long)a << 32) | b;
   asm("shr.u64 %0, %0, %1;" : "+l"(x) : "r"(sh));  // shifts past 63 give 0
   const long long s = (long long)((int)hi >> 31);
   return (((long long)x ^ s) + 1) >> 1;
 }
 
-// a basis entry of a column with largest biased exponent E
+// a basis entry of a column with largest biased exponent E (less the row's shift)
 __device__ __forceinline__ long long fx_basis(double v, int E) { return fx_round(v, E + 3); }
+
+// The shift of a row: the distance of an entry's exponent ex from its column's largest, less a
+// guard, so that entries up to 2^8 larger still fit later on (61 bits hold 53 and the guard).
+// kFxUnset: only zeros so far.
+constexpr int kFxGuard = 8;
+constexpr int kFxUnset = 1000;
+__device__ __forceinline__ int fx_shift(int ex, int E) {
+  return min(max(E - ex - kFxGuard, 0), kFxUnset - 1);
+}
+// the biased exponent of a nonzero value as fx_round takes it, 0 for zero
+__device__ __forceinline__ int fx_exp(double v) {
+  const int m = fx_mag(v);
+  return (m | __double2loint(v)) ? max(m >> 20, 1) : 0;
+}
+// 2^-s for 0 <= s <= 1022
+__device__ __forceinline__ double fx_pow2(int s) { return __hiloint2double((1023 - s) << 20, 0); }
+// an integer of a row whose shift shrinks by d > 0
+__device__ __forceinline__ long long fx_less_shift(long long m, int d) {
+  return d > 62 ? 0 : (m + (1ll << (d - 1))) >> d;
+}
 
 __device__ __forceinline__ Fx fx_limbs(unsigned lo, unsigned hi) {
   return Fx{(int)(hi + (lo >> 31)), (int)lo};
@@ -127,7 +157,7 @@ __device__ __forceinline__ void fx_axpy(FxAcc& a, const Fx v, const int4 k) {
   a.lh += (long long)v.l * k.x;
   a.ll += (v.l >> 19) * k.z;
 }
-// w + scale (sum in units of 2^60): scale = +-2^(m - 2098); two FP64 roundings
+// w + scale (sum in units of 2^60): scale = +-2^(m - 2098), times 2^-S of the row; two FP64 roundings
 __device__ __forceinline__ double fx_axpy_add(const FxAcc& a, double w, double scale) {
   const long long low = a.hl + (a.lh >> 4) + ((long long)a.ll << 2);
   const long long hi = a.hh + (low >> 28) - (1ll << 24);

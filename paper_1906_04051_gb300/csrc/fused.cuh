@@ -436,6 +436,13 @@ __device__ __forceinline__ ArnSplit arn_split(int nch) {
   return ArnSplit{S, warp % nch, warp / nch, nch, warp / nch < S};
 }
 
+// The shifts of the rows (fixed.cuh), 16 bits each, in the last of the m + 1 columns: the cycle needs
+// u_m's norm only, so that column is never stored
+template <typename TV, typename TACC>
+__device__ __forceinline__ short* arn_shifts(const ArnArgs<TV, TACC>& a) {
+  return reinterpret_cast<short*>(const_cast<TV*>(a.V) + (size_t)a.m * a.ldv);
+}
+
 // Two rows of a basis column held as fixed-point integers, past L1 (a column is converted in
 // place within the launch, after its FP64 form was read through L1)
 __device__ __forceinline__ void arn_ldfx(const long long* p, uint4& o) {
@@ -458,7 +465,7 @@ __device__ __forceinline__ void arn_ldfx(const long long* p, uint4& o) {
 template <int NSET, int G, int D>
 __device__ __forceinline__ void arn_dots_fx(int4* slot, const double* V, long long ldv, int kf,
                                             int k, int ej, long long s0, int nch, const int4* Wf,
-                                            const int4* Uf, int lane) {
+                                            const int4* Uf, const short* Sg, int lane) {
   const ArnSplit sp = arn_split(nch);
   if (!sp.live) return;
   const int nqw = (nch - 1 - sp.q0) / kArnWarps + 1;  // chunks of this warp
@@ -534,11 +541,12 @@ __device__ __forceinline__ void arn_dots_fx(int4* slot, const double* V, long lo
   if (kf < k && sp.p == sp.S - 1) {  // the FP64 column
     FxDot a{0, 0, 0, 0};
     for (int qi = 0; qi < nqw; ++qi) {
-      const double2 v = __ldcg(reinterpret_cast<const double2*>(V + (size_t)kf * ldv + at +
-                                                                (long long)qi * (kArnWarps * 64)));
+      const long long r = at + (long long)qi * (kArnWarps * 64);
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(V + (size_t)kf * ldv + r));
+      const short2 sh = __ldcg(reinterpret_cast<const short2*>(Sg + r));
       const int4 w = Wf[(size_t)(sp.q0 + qi * kArnWarps) * 32 + lane];
-      fx_dot(a, fx_limbs(fx_basis(v.x, ej)), make_int2(w.x, w.y));
-      fx_dot(a, fx_limbs(fx_basis(v.y, ej)), make_int2(w.z, w.w));
+      fx_dot(a, fx_limbs(fx_basis(v.x, ej - sh.x)), make_int2(w.x, w.y));
+      fx_dot(a, fx_limbs(fx_basis(v.y, ej - sh.y)), make_int2(w.z, w.w));
     }
     store(0, kf, a);
     if (NSET == 2) store(1, kf, FxDot{0, 0, 0, 0});
@@ -921,6 +929,9 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
       __syncthreads();
       int mw = 0;  // high word of the largest |w| of the super-tile
       constexpr int AWR = kArnAwRows64;
+      constexpr bool FX = MODE != kArnLowsyncDf;  // w and u_j become operands of integer dots
+      short* const Sg = arn_shifts(a);
+      const int eu = sE[j];
       for (long long i0 = s0 + t; i0 < s1; i0 += (long long)AWR * kArnThreads) {
         int e0[AWR], e1[AWR];
 #pragma unroll
@@ -931,7 +942,13 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
           e1[b] = live ? __ldg(a.aurp + row + 1) : 0;
         }
         TACC av[AWR];
-        int ac[AWR];
+        int ac[AWR], sh[AWR];
+        unsigned grow = 0;  // rows whose shift is too large for u_j
+#pragma unroll
+        for (int b = 0; b < AWR; ++b) {
+          const long long row = i0 + (long long)b * kArnThreads;
+          sh[b] = j > 0 && row < s1 ? __ldcg(Sg + row) : 0;
+        }
 #pragma unroll
         for (int b = 0; b < AWR; ++b) {
           const bool has = e0[b] < e1[b];
@@ -949,9 +966,37 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
               wv = fma(sig, Ws[row - s0], aw);
               a.w[row] = wv;  // the update reads w there
             }
+            const double u = Us[row - s0];
+            const int ex = fx_exp(u);
+            if (j == 0) {
+              sh[b] = ex ? fx_shift(ex, eu) : (row < N ? kFxUnset : 0);
+              __stcg(Sg + row, (short)sh[b]);
+            } else if (ex > 0 && ex > eu - sh[b]) {
+              grow |= 1u << b;
+            }
+            if (FX && sh[b]) {
+              wv *= fx_pow2(sh[b]);
+              if (MODE == kArnLowsync) Us[row - s0] = u * fx_pow2(sh[b]);
+            }
             Ws[row - s0] = wv;
             mw = max(mw, fx_mag(wv));
           }
+        }
+#pragma unroll 1
+        for (; grow; grow &= grow - 1) {
+          const long long row = i0 + (long long)(__ffs(grow) - 1) * kArnThreads;
+          const double u = __ldcg(reinterpret_cast<const double*>(a.V) + (size_t)j * a.ldv + row);
+          const int so = __ldcg(Sg + row), sn = fx_shift(fx_exp(u), eu);
+          __stcg(Sg + row, (short)sn);
+          if (!FX) continue;
+          long long* col = reinterpret_cast<long long*>(const_cast<TV*>(a.V)) + row;
+#pragma unroll 4
+          for (int c = 0; c < (so == kFxUnset ? 0 : j); ++c, col += a.ldv)
+            __stcg(col, fx_less_shift(__ldcg(col), so - sn));
+          const double wv = a.w[row] * fx_pow2(sn);
+          Ws[row - s0] = wv;
+          if (MODE == kArnLowsync) Us[row - s0] = u * fx_pow2(sn);
+          mw = max(mw, fx_mag(wv));
         }
       }
       mw = __reduce_max_sync(0xffffffffu, mw);
@@ -1042,7 +1087,7 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
       int4* slot = reinterpret_cast<int4*>(sbuf);
       arn_dots_fx<NSET, (NSET == 2 ? kArnFxGroup : kArnFxGroup1), kArnFxDepth>(
           slot, reinterpret_cast<const double*>(a.V), a.ldv, j, k, eu, s0, nch,
-          reinterpret_cast<const int4*>(Ws), reinterpret_cast<const int4*>(Us), lane);
+          reinterpret_cast<const int4*>(Ws), reinterpret_cast<const int4*>(Us), arn_shifts(a), lane);
       __syncthreads();
       arn_slot_sums<NSET>(slot, nch, k, sE, ew, eu, tile == 0, sred);
     } else {
@@ -1063,7 +1108,7 @@ __device__ __forceinline__ int4* arn_sk(double* sbuf) {
 
 // w - V (sigma o h) of the rows [s0, s1) (an FP64 basis): a row's sum of M_c K_c (at most kMaxK
 // terms) stays in integer accumulators, and FP64 enters once per row; put(r, value of row r, of
-// row r + 1) takes the results.  FIXED: the first kf columns are fixed-point integers, a last one
+// row r + 1, their shifts) takes the results.  FIXED: the first kf columns are fixed-point integers, a last one
 // (k = kf + 1) is FP64 and is converted in place on the way (no other block reads it any more:
 // the SpMV is behind the last grid barrier); else all columns are FP64 and stay so.  Each loaded
 // value's register is reloaded U columns on (past the last column: from the warp's next chunk)
@@ -1074,7 +1119,8 @@ constexpr int kArnUpdLoads = 6;  // basis loads in flight per lane
 
 template <bool FIXED, typename F>
 __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ldv,
-                                                   const double* w, long long s0, long long s1,
+                                                   const short* Sg, const double* w,
+                                                   long long s0, long long s1,
                                                    int kf, int k, const int* sE, const int4* sK,
                                                    double nscale, longlong2* sP, F&& put) {
   constexpr int U = kArnUpdLoads;
@@ -1088,16 +1134,18 @@ __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ld
   // the FP64 column's part of the rows at r, then the finished rows
   auto finish = [&](FxAcc& a0, FxAcc& a1) {
     const double2 wv = __ldcg(reinterpret_cast<const double2*>(w + r));
+    const short2 sh = __ldcg(reinterpret_cast<const short2*>(Sg + r));
     if (FIXED && kf < k) {
       double* pj = const_cast<double*>(V) + (size_t)kf * ldv + r;
       const double2 v = __ldcg(reinterpret_cast<const double2*>(pj));
-      const long long m0 = fx_basis(v.x, sE[kf]), m1 = fx_basis(v.y, sE[kf]);
+      const long long m0 = fx_basis(v.x, sE[kf] - sh.x), m1 = fx_basis(v.y, sE[kf] - sh.y);
       *reinterpret_cast<longlong2*>(pj) = make_longlong2(m0, m1);
       fx_axpy(a0, fx_limbs(m0), sK[kf]);
       fx_axpy(a1, fx_limbs(m1), sK[kf]);
     }
     // rows past N: w and the basis are zero there
-    put(r, fx_axpy_add(a0, wv.x, nscale), fx_axpy_add(a1, wv.y, nscale));
+    put(r, fx_axpy_add(a0, wv.x, sh.x ? nscale * fx_pow2(sh.x) : nscale),
+        fx_axpy_add(a1, wv.y, sh.y ? nscale * fx_pow2(sh.y) : nscale), sh);
   };
   FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
   if (sp.live && (!one || c0 < c1)) {
@@ -1112,6 +1160,8 @@ __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ld
     }
     for (; r >= s0; r -= kArnWarps * 64) {
       if (!one) a0 = a1 = FxAcc{0, 0, 0, 0};
+      short2 sr = make_short2(0, 0);
+      if (!FIXED) sr = __ldcg(reinterpret_cast<const short2*>(Sg + r));
 #pragma unroll 1
       for (int b = c0; b < c1; b += U) {
         nb += U;
@@ -1131,8 +1181,8 @@ __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ld
             f1 = fx_limbs(v[u].z, v[u].w);
           } else {
             const int e = sE[on ? b + u : c0];
-            f0 = fx_limbs(fx_basis(__hiloint2double((int)v[u].y, (int)v[u].x), e));
-            f1 = fx_limbs(fx_basis(__hiloint2double((int)v[u].w, (int)v[u].z), e));
+            f0 = fx_limbs(fx_basis(__hiloint2double((int)v[u].y, (int)v[u].x), e - sr.x));
+            f1 = fx_limbs(fx_basis(__hiloint2double((int)v[u].w, (int)v[u].z), e - sr.y));
           }
           if (more && nb + u < c1) arn_ldfx(pn + (size_t)u * ldv, v[u]);
           if (on) {
@@ -1177,12 +1227,13 @@ __device__ __forceinline__ void arn_fx_coefs(int k, const double* scoef, const i
   __syncthreads();
 }
 
-// u_{j+1} of the block's rows into vout (and ush, indexed from R0); returns the warp's part of
+// u_{j+1} of the block's rows into vout unless null (and ush, indexed from R0); returns the warp's part of
 // ||u_{j+1}||^2, and in mx the high word of the thread's largest |u_{j+1}|.  kf: the columns
 // already in fixed point
 template <bool FIXED>
-__device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, double* vout,
-                                                const double* w, long long R0, long long R1,
+__device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, const short* Sg,
+                                                double* vout, const double* w, long long R0,
+                                                long long R1,
                                                 int kf, int k, const double* scoef,
                                                 const int* sE, double* sbuf, double* sscale,
                                                 double* ush, int& mx) {
@@ -1191,9 +1242,9 @@ __device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, 
   int m = 0;
   arn_fx_coefs(k, scoef, sE, sK, sscale);
   arn_rows_update_fx<FIXED>(
-      V, ldv, w, R0, R1, kf, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
-      [&](long long r, double u0, double u1) {
-        *reinterpret_cast<double2*>(vout + r) = make_double2(u0, u1);
+      V, ldv, Sg, w, R0, R1, kf, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
+      [&](long long r, double u0, double u1, short2) {
+        if (vout) *reinterpret_cast<double2*>(vout + r) = make_double2(u0, u1);
         if (ush) *reinterpret_cast<double2*>(ush + (r - R0)) = make_double2(u0, u1);
         nrm = fma(u0, u0, fma(u1, u1, nrm));
         m = max(m, max(fx_mag(u0), fx_mag(u1)));
@@ -1205,8 +1256,8 @@ __device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, 
 // CGS2, first update and second multi-dot of an FP64 basis: per super-tile (from the last) w -= V
 // (sigma o h) into w and shared memory (the newest column becomes fixed-point on the way), its
 // operand form, then V^T w into sred
-__device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, double* w, int RS,
-                                             long long R0, long long R1, int k,
+__device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, const short* Sg,
+                                             double* w, int RS, long long R0, long long R1, int k,
                                              const double* scoef, const int* sE, double* Ws,
                                              double* sbuf, int* semax, double* sscale,
                                              double* sred) {
@@ -1223,9 +1274,11 @@ __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, dou
     __syncthreads();
     int mw = 0;
     arn_rows_update_fx<true>(
-        V, ldv, w, s0, s1, k - 1, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
-        [&](long long r, double u0, double u1) {
+        V, ldv, Sg, w, s0, s1, k - 1, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
+        [&](long long r, double u0, double u1, short2 sh) {
           *reinterpret_cast<double2*>(w + r) = make_double2(u0, u1);
+          if (sh.x) u0 *= fx_pow2(sh.x);
+          if (sh.y) u1 *= fx_pow2(sh.y);
           *reinterpret_cast<double2*>(Ws + (r - s0)) = make_double2(u0, u1);
           mw = max(mw, max(fx_mag(u0), fx_mag(u1)));
         });
@@ -1238,7 +1291,7 @@ __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, dou
     __syncthreads();
     const int nch = (int)((s1 - s0) >> 6);
     arn_dots_fx<1, kArnFxGroup1, kArnFxDepth>(slot, V, ldv, k, k, 0, s0, nch,
-                                 reinterpret_cast<const int4*>(Ws), nullptr, lane);
+                                 reinterpret_cast<const int4*>(Ws), nullptr, Sg, lane);
     __syncthreads();
     arn_slot_sums<1>(slot, nch, k, sE, ew, 0, tile == tiles - 1, sred);
   }
@@ -1701,7 +1754,7 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
         scoef[c] = (TACC)(ssig[c] * sg[c]);
       }
       if constexpr (sizeof(TV) == 8) {
-        arn_pass2_fx(a.V, a.ldv, a.w, a.RS, R0, R1, k, scoef, sE, Ws,
+        arn_pass2_fx(a.V, a.ldv, arn_shifts(a), a.w, a.RS, R0, R1, k, scoef, sE, Ws,
                      sbuf, semax, &sscale, sred);
       } else {
         arn_pass2_rows<TV, TACC, ND>(a, g, k, Ws, scoef, sbuf);
@@ -1771,8 +1824,8 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
     int mx = 0;
     if constexpr (sizeof(TV) == 8)
       nrm = arn_update_fx<MODE != kArnLowsyncDf>(
-          a.V, a.ldv, vout, a.w, R0, R1, MODE == kArnLowsync ? k - 1 : k, k, scoef, sE, sbuf,
-          &sscale, ush, mx);
+          a.V, a.ldv, arn_shifts(a), k < a.m ? vout : nullptr, a.w, R0, R1,
+          MODE == kArnLowsync ? k - 1 : k, k, scoef, sE, sbuf, &sscale, ush, mx);
     else
       nrm = arn_update<TV, TACC, false>(a, g, k, Ws, scoef, ush, R0, R1,
                                           reinterpret_cast<float*>(sbuf));

@@ -116,6 +116,11 @@ struct CycleArgs {
 };
 
 // Phases of a solve; each launch_phase call enqueues the kernels of one phase.
+// the rows' shifts of a fixed-point basis: in its last column, which a cycle does not store
+inline const short* fx_shifts(const CycleArgs& a) {
+  return reinterpret_cast<const short*>(static_cast<const double*>(a.V) + (size_t)a.m * a.ldv);
+}
+
 enum Phase {
   PH_SETUP = 0,     // gmres_create: validation, aggregates, T, T^-1
   PH_RESIDUAL,      // r = b - A x in FP64, u_0, stopping decision

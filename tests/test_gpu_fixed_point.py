@@ -1,6 +1,8 @@
 """The fixed-point dots and column combinations of the FP64 Arnoldi steps (csrc/fixed.cuh): sizes
 at the edges of chunks and units, operand ranges that exercise the per-piece exponents, and
 exact power-of-two scaling (the integer arithmetic sees the same limbs)."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -145,3 +147,76 @@ def test_long_rows_at_the_fused_limit(G, orc, n, ortho):
                       **({"ortho": orc.MGS} if ortho else {}))
     assert ig["iters"] == 9
     assert relerr(xg.cpu().numpy(), xo) <= 1e-9
+
+
+def _two_blocks(orc, A, b, q, f):
+    """diag(A, A) with right-hand sides b and 2^-q b / f."""
+    B = orc.CSR(np.concatenate([A.rowptr, A.rowptr[1:] + A.rowptr[-1]]),
+                np.concatenate([A.col, A.col + A.n]), np.concatenate([A.val, A.val]))
+    return B, np.concatenate([b, np.ldexp(b / f, -q)])
+
+
+def _permute(orc, A, seed):
+    perm = np.random.default_rng(seed).permutation(A.n)
+    inv = np.argsort(perm)
+    rows = [sorted(zip(inv[A.col[A.rowptr[i]:A.rowptr[i + 1]]],
+                       A.val[A.rowptr[i]:A.rowptr[i + 1]])) for i in perm]
+    return orc.CSR(np.cumsum([0] + [len(q) for q in rows]), np.array([c for q in rows for c, _ in q]),
+                   np.array([v for q in rows for _, v in q])), perm
+
+
+# An uncoupled block whose right-hand side is 2^-q / f times the other's has a solution in the same
+# proportion: all that the blocks share are the projection coefficients.  A basis in fixed point has
+# to keep that as FP64 does, however far the block lies below the columns' largest entries, and
+# also where its rows start from zeros and grow as the Krylov space spreads ("point": one nonzero
+# entry of b).  The bound is what FP64 makes of it: ten times the largest deviation of the
+# oracle over three factors f that are not powers of two (3e-16; with an adaptive space 2e-14 to
+# 8e-13, since T^-1 amplifies)
+@pytest.mark.parametrize("q", [12, 66, 300])
+@pytest.mark.parametrize("rhs", ["full", "point"])
+@pytest.mark.parametrize("how", ["cgs2", "lowsync", "df32", "csr", "csr-lowsync", "noalloc", "batch",
+                                 "batch-lowsync", "adaptive"])
+def test_small_uncoupled_block_keeps_its_digits(G, orc, how, rhs, q):
+    p = W.convdiff(24, pe=20.0, sigma=0.5, seed=33, px=1, py=1)
+    A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+    n = A.n
+    if rhs == "point":
+        b = np.zeros(n)
+        b[n // 2] = 1.0
+    bound = 0.0
+    for f in (7.0, 1.7, 3.0):
+        B, bb = _two_blocks(orc, A, b, q, f)
+        xo, _ = orc.gmres(B, bb, m=20, tol=0.0, maxit=60, fixed_iterations=True,
+                          **(dict(defl_mode=orc.DEFL_ADAPTIVE, mu_mode=1, mu_user=5.0, rmax=4, ninv=2)
+                             if how == "adaptive" else {}))
+        bound = max(bound, 10.0 * relerr(f * np.ldexp(xo[n:], q), xo[:n]))
+    A, b = B, bb
+    perm = np.arange(A.n)
+    if how.startswith("csr"):
+        A, perm = _permute(orc, A, 3)
+    kw = dict(deflation_mode=G.DEFL_NONE, fixed_iterations=True)
+    if "lowsync" in how or how == "df32":
+        kw["ortho"] = G.ORTHO_MGS_LOWSYNC
+    if how == "df32":
+        kw["dot_arith"] = G.DOT_DF32
+    if how == "adaptive":  # the first cycle is a fused one, whose basis the space comes from
+        kw.update(deflation_mode=G.DEFL_ADAPTIVE, mu_mode=1, mu_user=5.0, rmax=4, ninv=2)
+    s = gpu_solver_from_oracle(G, A, **kw)
+    bd = to_dev(b[perm])
+    from paper_1906_04051_gb300 import _native as N
+    if how.startswith("batch"):
+        xs, infos, _ = G.batch_solve([s], [bd], m=20, tol=0.0, maxit=60)
+        x, info = xs[0], infos[0]
+    elif how == "noalloc":
+        x, info = torch.empty_like(bd), N.gmres_info()
+        torch.cuda.synchronize()
+        assert N.load().gmres_solve_noalloc(s.handle, bd.data_ptr(), None, 20, 0.0, 60, x.data_ptr(),
+                                            ctypes.byref(info)) >= 0
+        info = info.as_dict()
+    else:
+        x, info = s.solve(bd, m=20, tol=0.0, maxit=60)
+    assert info["iters"] == 60
+    y = np.empty(A.n)
+    y[perm] = x.cpu().numpy()
+    assert np.linalg.norm(y[:n]) > 0
+    assert relerr(3.0 * np.ldexp(y[n:], q), y[:n]) <= bound
