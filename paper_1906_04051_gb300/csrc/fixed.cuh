@@ -73,11 +73,6 @@ constexpr int kFxUnset = 1000;
 __device__ __forceinline__ int fx_shift(int ex, int E) {
   return min(max(E - ex - kFxGuard, 0), kFxUnset - 1);
 }
-// the biased exponent of a nonzero value as fx_round takes it, 0 for zero
-__device__ __forceinline__ int fx_exp(double v) {
-  const int m = fx_mag(v);
-  return (m | __double2loint(v)) ? max(m >> 20, 1) : 0;
-}
 // 2^-s for 0 <= s <= 1022
 __device__ __forceinline__ double fx_pow2(int s) { return __hiloint2double((1023 - s) << 20, 0); }
 // an integer of a row whose shift shrinks by d > 0
@@ -92,7 +87,7 @@ __device__ __forceinline__ Fx fx_limbs(long long m) {
   return fx_limbs((unsigned)m, (unsigned)((unsigned long long)m >> 32));
 }
 
-// the other operand of a dot (wh, wl) of a piece with largest biased exponent E
+// the other operand of a dot (wh, wl) of a piece with largest biased exponent E, plus the row's shift
 __device__ __forceinline__ int2 fx_operand(double v, int E) {
   const long long m = fx_round(v, E + 10);
   const int wl = (int)((unsigned)m << 4) >> 4;

@@ -892,6 +892,87 @@ __device__ __forceinline__ void arn_slot_sums(const int4* slot, int nch, int k, 
   }
 }
 
+// The shift of a row with entry u of column j (largest exponent E), kept at p: chosen at the first
+// column, reduced where u does not fit
+__device__ __forceinline__ int arn_shift_of(short* p, int j, double u, int E, bool row) {
+  const int ex = fx_mag(u) >> 20;  // (subnormal entries count as zeros)
+  int s = j > 0 ? __ldcg(p) : (row ? kFxUnset : 0);
+  if (ex > 0 && (s == kFxUnset || ex > E - s)) s = fx_shift(ex, E);
+  else if (j > 0) return s;
+  __stcg(p, (short)s);
+  return s;
+}
+
+// Rows that column j outgrew (bit b of grow: row q0 + b kArnThreads; any: of the warp's lanes): their
+// new shifts, their earlier entries in the new unit, their operands
+// again.  Rare; the warp shares a row's columns, one round of loads per 32 of them.
+template <int NSET>
+__device__ __forceinline__ void arn_grow(double* V, long long ldv, const double* w, short* Sg, int j,
+                                         int q0, unsigned any, unsigned grow, int ew, int eu, int2* Wf,
+                                         int2* Uf) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (; any; any &= any - 1) {
+    const int b = __ffs(any) - 1, q = q0 + b * kArnThreads;
+    const bool mine = grow >> b & 1u;
+    int so = 0, sn = 0;
+    if (mine) {
+      const double u = __ldcg(V + (size_t)j * ldv + q);
+      so = __ldcg(Sg + q);
+      sn = arn_shift_of(Sg + q, j, u, eu, true);
+      Wf[q] = fx_operand(__ldcg(w + q), ew + sn);
+      if (NSET == 2) Uf[q] = fx_operand(u, eu + sn);
+    }
+    unsigned lanes = __ballot_sync(0xffffffffu, mine && so != kFxUnset);
+#pragma unroll 1
+    for (; lanes; lanes &= lanes - 1) {
+      const int l = __ffs(lanes) - 1;
+      const int d = __shfl_sync(0xffffffffu, so - sn, l);
+      long long* col = reinterpret_cast<long long*>(V) + (q - lane + l) + (size_t)lane * ldv;
+      for (int c = lane; c < j; c += 32, col += 32 * ldv)
+        __stcg(col, fx_less_shift(__ldcg(col), d));
+    }
+  }
+}
+
+// w and u_j (for two dots) of n rows, at Ws and Us, as operands of the fixed-point dots in place: ew,
+// eu the largest exponents of w in the super-tile and of u_j.  V, w and Sg point at the first row;
+// the first `live` rows exist.  (A call of its own: inlined it would spill registers around the dots.)
+template <int NSET>
+__device__ __noinline__ void arn_operands(double* V, long long ldv, const double* w, short* Sg, int j,
+                                          int n, int live, int ew, int eu, double* Ws, double* Us) {
+  constexpr int B = 4;  // rows per thread whose shifts are loaded at once
+  int2* const Wf = reinterpret_cast<int2*>(Ws);
+  int2* const Uf = reinterpret_cast<int2*>(Us);
+  for (int q0 = threadIdx.x; q0 < n; q0 += B * kArnThreads) {
+    int sh[B];
+    if (j > 0) {
+#pragma unroll
+      for (int b = 0; b < B; ++b)
+        sh[b] = q0 + b * kArnThreads < n ? __ldcg(Sg + q0 + b * kArnThreads) : 0;
+    } else {
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        const int q = q0 + b * kArnThreads;
+        sh[b] = q < n ? arn_shift_of(Sg + q, 0, Us[q], eu, q < live) : 0;
+      }
+    }
+    unsigned grow = 0;  // rows whose shift is too large for u_j
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int q = q0 + b * kArnThreads;
+      if (q < n) {
+        const double u = Us[q];
+        grow |= (fx_mag(u) >> 20 > max(eu - sh[b], 0) ? 1u : 0u) << b;
+        Wf[q] = fx_operand(Ws[q], ew + sh[b]);
+        if (NSET == 2) Uf[q] = fx_operand(u, eu + sh[b]);
+      }
+    }
+    const unsigned any = __reduce_or_sync(0xffffffffu, grow);
+    if (any) arn_grow<NSET>(V, ldv, w, Sg, j, q0, any, grow, ew, eu, Wf, Uf);
+  }
+}
+
 // SpMV, coarse correction and multi-dot of step j over the block's super-tiles (a function
 // of its own, so that the cycle loop's state stays out of these loops' registers)
 template <typename TV, typename TACC, int ND, int MODE>
@@ -929,9 +1010,6 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
       __syncthreads();
       int mw = 0;  // high word of the largest |w| of the super-tile
       constexpr int AWR = kArnAwRows64;
-      constexpr bool FX = MODE != kArnLowsyncDf;  // w and u_j become operands of integer dots
-      short* const Sg = arn_shifts(a);
-      const int eu = sE[j];
       for (long long i0 = s0 + t; i0 < s1; i0 += (long long)AWR * kArnThreads) {
         int e0[AWR], e1[AWR];
 #pragma unroll
@@ -942,13 +1020,7 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
           e1[b] = live ? __ldg(a.aurp + row + 1) : 0;
         }
         TACC av[AWR];
-        int ac[AWR], sh[AWR];
-        unsigned grow = 0;  // rows whose shift is too large for u_j
-#pragma unroll
-        for (int b = 0; b < AWR; ++b) {
-          const long long row = i0 + (long long)b * kArnThreads;
-          sh[b] = j > 0 && row < s1 ? __ldcg(Sg + row) : 0;
-        }
+        int ac[AWR];
 #pragma unroll
         for (int b = 0; b < AWR; ++b) {
           const bool has = e0[b] < e1[b];
@@ -966,37 +1038,9 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
               wv = fma(sig, Ws[row - s0], aw);
               a.w[row] = wv;  // the update reads w there
             }
-            const double u = Us[row - s0];
-            const int ex = fx_exp(u);
-            if (j == 0) {
-              sh[b] = ex ? fx_shift(ex, eu) : (row < N ? kFxUnset : 0);
-              __stcg(Sg + row, (short)sh[b]);
-            } else if (ex > 0 && ex > eu - sh[b]) {
-              grow |= 1u << b;
-            }
-            if (FX && sh[b]) {
-              wv *= fx_pow2(sh[b]);
-              if (MODE == kArnLowsync) Us[row - s0] = u * fx_pow2(sh[b]);
-            }
             Ws[row - s0] = wv;
             mw = max(mw, fx_mag(wv));
           }
-        }
-#pragma unroll 1
-        for (; grow; grow &= grow - 1) {
-          const long long row = i0 + (long long)(__ffs(grow) - 1) * kArnThreads;
-          const double u = __ldcg(reinterpret_cast<const double*>(a.V) + (size_t)j * a.ldv + row);
-          const int so = __ldcg(Sg + row), sn = fx_shift(fx_exp(u), eu);
-          __stcg(Sg + row, (short)sn);
-          if (!FX) continue;
-          long long* col = reinterpret_cast<long long*>(const_cast<TV*>(a.V)) + row;
-#pragma unroll 4
-          for (int c = 0; c < (so == kFxUnset ? 0 : j); ++c, col += a.ldv)
-            __stcg(col, fx_less_shift(__ldcg(col), so - sn));
-          const double wv = a.w[row] * fx_pow2(sn);
-          Ws[row - s0] = wv;
-          if (MODE == kArnLowsync) Us[row - s0] = u * fx_pow2(sn);
-          mw = max(mw, fx_mag(wv));
         }
       }
       mw = __reduce_max_sync(0xffffffffu, mw);
@@ -1062,10 +1106,12 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
     if constexpr (sizeof(TV) == 8) {
       // w and u_j to fixed point in place (relative to the largest exponent of w in the
       // super-tile, of u_j as a whole), then the dots with every column
-      const int ew = semax[0] >> 20, eu = sE[j];
+      const int ew = semax[0] >> 20, eu = sE[j], n = (int)(s1 - s0);
+      short* const Sg = arn_shifts(a) + s0;
       if constexpr (MODE == kArnLowsyncDf) {
         // w and u_j split in place (float2 hi, lo in the 8 bytes of each double)
-        for (int q = t; q < (int)(s1 - s0); q += kArnThreads) {
+        for (int q = t; q < n; q += kArnThreads) {
+          arn_shift_of(Sg + q, j, Us[q], eu, s0 + q < N);
           float h1, l1, h2, l2;
           arn_df_split((double)Ws[q], h1, l1);
           arn_df_split((double)Us[q], h2, l2);
@@ -1079,10 +1125,8 @@ __device__ __forceinline__ void arn_front(const ArnArgs<TV, TACC>& a, const ArnR
         __syncthreads();
         continue;
       }
-      for (int q = t; q < (int)(s1 - s0); q += kArnThreads) {
-        reinterpret_cast<int2*>(Ws)[q] = fx_operand((double)Ws[q], ew);
-        if (NSET == 2) reinterpret_cast<int2*>(Us)[q] = fx_operand((double)Us[q], eu);
-      }
+      arn_operands<NSET>(reinterpret_cast<double*>(const_cast<TV*>(a.V)) + s0, a.ldv, a.w + s0, Sg, j, n,
+                         (int)min(N - s0, (long long)n), ew, eu, Ws, Us);
       __syncthreads();
       int4* slot = reinterpret_cast<int4*>(sbuf);
       arn_dots_fx<NSET, (NSET == 2 ? kArnFxGroup : kArnFxGroup1), kArnFxDepth>(
@@ -1144,8 +1188,12 @@ __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ld
       fx_axpy(a1, fx_limbs(m1), sK[kf]);
     }
     // rows past N: w and the basis are zero there
-    put(r, fx_axpy_add(a0, wv.x, sh.x ? nscale * fx_pow2(sh.x) : nscale),
-        fx_axpy_add(a1, wv.y, sh.y ? nscale * fx_pow2(sh.y) : nscale), sh);
+    double n0 = nscale, n1 = nscale;
+    if (sh.x | sh.y) {
+      n0 *= fx_pow2(sh.x);
+      n1 *= fx_pow2(sh.y);
+    }
+    put(r, fx_axpy_add(a0, wv.x, n0), fx_axpy_add(a1, wv.y, n1), sh);
   };
   FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
   if (sp.live && (!one || c0 < c1)) {
@@ -1277,8 +1325,10 @@ __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, con
         V, ldv, Sg, w, s0, s1, k - 1, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
         [&](long long r, double u0, double u1, short2 sh) {
           *reinterpret_cast<double2*>(w + r) = make_double2(u0, u1);
-          if (sh.x) u0 *= fx_pow2(sh.x);
-          if (sh.y) u1 *= fx_pow2(sh.y);
+          if (sh.x | sh.y) {  // (the operand's shift, ahead of the conversion)
+            u0 *= fx_pow2(sh.x);
+            u1 *= fx_pow2(sh.y);
+          }
           *reinterpret_cast<double2*>(Ws + (r - s0)) = make_double2(u0, u1);
           mw = max(mw, max(fx_mag(u0), fx_mag(u1)));
         });
