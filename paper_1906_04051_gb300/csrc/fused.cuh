@@ -670,9 +670,49 @@ __device__ __forceinline__ int arn_share(const ArnArgs<TV, TACC>& a, int G) {
 // about twice as fast as a warp reading one column through many consecutive chunks).  Units run
 // group by group, the warp's chunks in order, two units in flight, each value's register reloaded
 // as it is used.  S warps share a chunk's groups where the blocks have few chunks (arn_split32).
-// At a group's last chunk the lanes' partial sums of each column are added by a shuffle tree and
-// lane 0 accumulates them into wsum[set][first chunk][c].
+// At a group's last chunk the lanes' partial sums meet as double-FP32 pairs (arn_warp_pairs) and are
+// accumulated into wsum[set][first chunk][c].
 template <int ND> constexpr int arn_group() { return ND == 9 ? 6 : 5; }
+
+// Sums over the warp's lanes of up to 8 values, as double-FP32 pairs (FP32 adds would round in the
+// last bits of the largest partial sum, FP64 adds hold their pipe 64 issue slots each).  Lanes halve
+// the columns they keep in the first three exchanges: 9 pair additions for 8 columns, where a tree
+// per column takes 5 each.  The total of column arn_pairs_col(lane), in every lane.
+__device__ __forceinline__ int arn_pairs_col(int lane) {
+  return (lane >> 2 & 4) | (lane >> 2 & 2) | (lane >> 2 & 1);
+}
+template <int G>
+__device__ __forceinline__ float2 arn_warp_pairs(const float (&v)[G], int lane) {
+  static_assert(G <= 8, "eight columns at a time");
+  float s[4], c[4];
+  const bool h4 = lane & 16, h2 = lane & 8, h1 = lane & 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float lo = i < G ? v[i < G ? i : 0] : 0.f, hi = i + 4 < G ? v[i + 4 < G ? i + 4 : 0] : 0.f;
+    s[i] = h4 ? hi : lo;
+    c[i] = 0.f;
+    arn_df_add(s[i], c[i], __shfl_xor_sync(0xffffffffu, h4 ? lo : hi, 16), 0.f);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float so = __shfl_xor_sync(0xffffffffu, h2 ? s[i] : s[i + 2], 8);
+    const float co = __shfl_xor_sync(0xffffffffu, h2 ? c[i] : c[i + 2], 8);
+    s[i] = h2 ? s[i + 2] : s[i];
+    c[i] = h2 ? c[i + 2] : c[i];
+    arn_df_add(s[i], c[i], so, co);
+  }
+  const float so = __shfl_xor_sync(0xffffffffu, h1 ? s[0] : s[1], 4);
+  const float co = __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 4);
+  float rs = h1 ? s[1] : s[0], rc = h1 ? c[1] : c[0];
+  arn_df_add(rs, rc, so, co);
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1) {
+    const float s2 = __shfl_xor_sync(0xffffffffu, rs, o);
+    const float c2 = __shfl_xor_sync(0xffffffffu, rc, o);
+    arn_df_add(rs, rc, s2, c2);
+  }
+  return make_float2(rs, rc);
+}
 
 // S: warps per chunk, the same in every block of the system (so that equal rows are summed in the
 // same order everywhere): 16 / the most chunks a block holds, at least 1
@@ -742,21 +782,19 @@ __device__ __forceinline__ void arn_dots_rows(double* wsum, const TV* V, long lo
       advance();
       if (++qi == nqw) {  // the group's last chunk in this warp
 #pragma unroll
-        for (int u = 0; u < G; ++u)
-#pragma unroll
-          for (int t = 0; t < NSET; ++t) {
-            if (g0 + u < k) {
-              const TACC v = warp_sum(acc[t][u]);
-              if (lane == 0) {
-                float2* pw = reinterpret_cast<float2*>(wsum) +
-                             (size_t)(t * kArnWarps + sp.q0) * kMaxK + g0 + u;
-                float2 o = *pw;
-                arn_df_add(o.x, o.y, (float)v, 0.f);
-                *pw = o;
-              }
-            }
-            acc[t][u] = 0;
+        for (int t = 0; t < NSET; ++t) {
+          const float2 v = arn_warp_pairs<G>(acc[t], lane);
+          const int u = arn_pairs_col(lane);
+          if ((lane & 3) == 0 && u < G && g0 + u < k) {
+            float2* pw = reinterpret_cast<float2*>(wsum) +
+                         (size_t)(t * kArnWarps + sp.q0) * kMaxK + g0 + u;
+            float2 o = *pw;
+            arn_df_add(o.x, o.y, v.x, v.y);
+            *pw = o;
           }
+#pragma unroll
+          for (int q = 0; q < G; ++q) acc[t][q] = 0;
+        }
         qi = 0;
         g0 += G * sp.S;
       }
