@@ -1201,7 +1201,7 @@ constexpr int kArnUpdLoads = 6;  // basis loads in flight per lane
 
 template <bool FIXED, typename F>
 __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ldv,
-                                                   const short* Sg, const double* w,
+                                                   const short* Sg, const double* w, int N,
                                                    long long s0, long long s1,
                                                    int kf, int k, const int* sE, const int4* sK,
                                                    double nscale, longlong2* sP, F&& put) {
@@ -1225,13 +1225,13 @@ __device__ __forceinline__ void arn_rows_update_fx(const double* V, long long ld
       fx_axpy(a0, fx_limbs(m0), sK[kf]);
       fx_axpy(a1, fx_limbs(m1), sK[kf]);
     }
-    // rows past N: w and the basis are zero there
     double n0 = nscale, n1 = nscale;
     if (sh.x | sh.y) {
       n0 *= fx_pow2(sh.x);
       n1 *= fx_pow2(sh.y);
     }
-    put(r, fx_axpy_add(a0, wv.x, n0), fx_axpy_add(a1, wv.y, n1), sh);
+    // rows past N: w and the basis are zeros there, and stay so when a coefficient is not finite
+    put(r, r < N ? fx_axpy_add(a0, wv.x, n0) : 0.0, r + 1 < N ? fx_axpy_add(a1, wv.y, n1) : 0.0, sh);
   };
   FxAcc a0{0, 0, 0, 0}, a1{0, 0, 0, 0};
   if (sp.live && (!one || c0 < c1)) {
@@ -1318,8 +1318,8 @@ __device__ __forceinline__ void arn_fx_coefs(int k, const double* scoef, const i
 // already in fixed point
 template <bool FIXED>
 __device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, const short* Sg,
-                                                double* vout, const double* w, long long R0,
-                                                long long R1,
+                                                double* vout, const double* w, int N,
+                                                long long R0, long long R1,
                                                 int kf, int k, const double* scoef,
                                                 const int* sE, double* sbuf, double* sscale,
                                                 double* ush, int& mx) {
@@ -1328,7 +1328,7 @@ __device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, 
   int m = 0;
   arn_fx_coefs(k, scoef, sE, sK, sscale);
   arn_rows_update_fx<FIXED>(
-      V, ldv, Sg, w, R0, R1, kf, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
+      V, ldv, Sg, w, N, R0, R1, kf, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
       [&](long long r, double u0, double u1, short2) {
         if (vout) *reinterpret_cast<double2*>(vout + r) = make_double2(u0, u1);
         if (ush) *reinterpret_cast<double2*>(ush + (r - R0)) = make_double2(u0, u1);
@@ -1343,7 +1343,8 @@ __device__ __forceinline__ double arn_update_fx(const double* V, long long ldv, 
 // (sigma o h) into w and shared memory (the newest column becomes fixed-point on the way), its
 // operand form, then V^T w into sred
 __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, const short* Sg,
-                                             double* w, int RS, long long R0, long long R1, int k,
+                                             double* w, int N, int RS, long long R0, long long R1,
+                                             int k,
                                              const double* scoef, const int* sE, double* Ws,
                                              double* sbuf, int* semax, double* sscale,
                                              double* sred) {
@@ -1360,7 +1361,7 @@ __device__ __forceinline__ void arn_pass2_fx(const double* V, long long ldv, con
     __syncthreads();
     int mw = 0;
     arn_rows_update_fx<true>(
-        V, ldv, Sg, w, s0, s1, k - 1, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
+        V, ldv, Sg, w, N, s0, s1, k - 1, k, sE, sK, *sscale, reinterpret_cast<longlong2*>(sbuf),
         [&](long long r, double u0, double u1, short2 sh) {
           *reinterpret_cast<double2*>(w + r) = make_double2(u0, u1);
           if (sh.x | sh.y) {  // (the operand's shift, ahead of the conversion)
@@ -1417,7 +1418,7 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, const A
       for (int e = 0; e < VN; ++e) wv[e] = r + e < N ? __ldcg(a.w + r + e) : (TACC)0;
     }
 #pragma unroll
-    for (int e = 0; e < VN; ++e) un[e] = wv[e] - p[e];
+    for (int e = 0; e < VN; ++e) un[e] = r + e < N ? wv[e] - p[e] : (TACC)0;  // (as in FP64)
     if constexpr (PASS2) {  // CGS2's first update: w stays where it came from
       if (wsm) {
         acc_store<VN>(Ws + (r - R0), un);
@@ -1842,7 +1843,7 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
         scoef[c] = (TACC)(ssig[c] * sg[c]);
       }
       if constexpr (sizeof(TV) == 8) {
-        arn_pass2_fx(a.V, a.ldv, arn_shifts(a), a.w, a.RS, R0, R1, k, scoef, sE, Ws,
+        arn_pass2_fx(a.V, a.ldv, arn_shifts(a), a.w, a.N, a.RS, R0, R1, k, scoef, sE, Ws,
                      sbuf, semax, &sscale, sred);
       } else {
         arn_pass2_rows<TV, TACC, ND>(a, g, k, Ws, scoef, sbuf);
@@ -1912,7 +1913,7 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
     int mx = 0;
     if constexpr (sizeof(TV) == 8)
       nrm = arn_update_fx<MODE != kArnLowsyncDf>(
-          a.V, a.ldv, arn_shifts(a), k < a.m ? vout : nullptr, a.w, R0, R1,
+          a.V, a.ldv, arn_shifts(a), k < a.m ? vout : nullptr, a.w, a.N, R0, R1,
           MODE == kArnLowsync ? k - 1 : k, k, scoef, sE, sbuf, &sscale, ush, mx);
     else
       nrm = arn_update<TV, TACC, false>(a, g, k, Ws, scoef, ush, R0, R1,

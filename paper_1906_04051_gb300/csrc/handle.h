@@ -136,7 +136,8 @@ inline int sdefl_len(const gmres_s* h) { return (h->r > kMaxAdapt ? h->r : kMaxA
 inline gmres_status ensure_workspace(gmres_s* h, int m, int prec) {
   const int ldh = m > h->ldh ? m : h->ldh;
   // columns padded to 256 rows: the pipelined passes copy whole 256-row-aligned tiles,
-  // and the padding rows stay zero (never written after this memset)
+  // and the padding rows stay zero (the fused cycle, which takes whole units of rows, stores
+  // zeros there)
   const long long ldv = ((long long)h->n + 255) / 256 * 256;
   const int max_grid = h->sms * 8;
   if (ldh != h->ldh || prec != h->prec_ws) {
