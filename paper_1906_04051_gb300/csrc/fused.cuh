@@ -263,26 +263,27 @@ __device__ __forceinline__ void arn_reduce_cols(const double* src, int nrows, in
   __syncthreads();
 }
 
-// 16-byte vector load of VN basis elements from global memory, read-only and streamed past
-// L1 (the basis is read once per pass; L1 is mostly carved out for shared memory here)
+// 16-byte vector load of VN basis elements from global memory, streamed past L1 (the basis is read
+// once per pass; L1 is mostly carved out for shared memory here).  Not the read-only path: the
+// launch that reads a column has stored it.
 template <typename TV, typename TACC, int VN>
 __device__ __forceinline__ void arn_ldg(const TV* p, TACC (&o)[VN]) {
   if constexpr (std::is_same<TV, double>::value) {
     double x, y;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];"
+    asm volatile("ld.global.L1::no_allocate.v2.f64 {%0, %1}, [%2];"
                  : "=d"(x), "=d"(y)
                  : "l"(p));
     o[0] = (TACC)x;
     o[1] = (TACC)y;
   } else if constexpr (std::is_same<TV, float>::value) {
     float x, y, z, w;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(x), "=f"(y), "=f"(z), "=f"(w)
                  : "l"(p));
     o[0] = x; o[1] = y; o[2] = z; o[3] = w;
   } else {
     unsigned x, y;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.b32 {%0, %1}, [%2];"
+    asm volatile("ld.global.L1::no_allocate.v2.b32 {%0, %1}, [%2];"
                  : "=r"(x), "=r"(y)
                  : "l"(p));
     // a BF16 value is the upper half of its FP32 form
@@ -291,6 +292,27 @@ __device__ __forceinline__ void arn_ldg(const TV* p, TACC (&o)[VN]) {
     o[2] = __uint_as_float(y << 16);
     o[3] = __uint_as_float(y & 0xffff0000u);
   }
+}
+
+// An entry of u_j, which other blocks stored earlier in the launch (nor is this the read-only path),
+// kept in L1 for the neighbouring rows of the SpMV
+template <typename TACC>
+__device__ __forceinline__ TACC arn_ldx(const double* p) {
+  double v;
+  asm volatile("ld.global.ca.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return (TACC)v;
+}
+template <typename TACC>
+__device__ __forceinline__ TACC arn_ldx(const float* p) {
+  float v;
+  asm volatile("ld.global.ca.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return (TACC)v;
+}
+template <typename TACC>
+__device__ __forceinline__ TACC arn_ldx(const __nv_bfloat16* p) {
+  unsigned v;
+  asm volatile("ld.global.ca.u16 %0, [%1];" : "=r"(v) : "l"(p));
+  return (TACC)__uint_as_float(v << 16);
 }
 
 // An FP64 operator value read with the L2 evict-first priority: the diagonals (76 MB at
@@ -646,7 +668,7 @@ __device__ __forceinline__ void arn_dia_rows(TACC (&acc)[B], long long row0, lon
           av[b][u] = live ? arn_ld_evict_first(dval + (size_t)q * ldd + rr) : (TACC)0;
         else
           av[b][u] = live ? __ldg(dval + (size_t)q * ldd + rr) : (TACC)0;
-        xv[b][u] = live ? ld_as<TACC, TV>(x + c) : (TACC)0;
+        xv[b][u] = live ? arn_ldx<TACC>(x + c) : (TACC)0;
       }
     }
 #pragma unroll
@@ -818,7 +840,7 @@ __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj
       TACC acc = 0, x = 0;
       if (row < N) {
         const int rs = __ldg(a.rowptr + row), re = __ldg(a.rowptr + row + 1);
-        x = ld_as<TACC, TV>(xj + row);
+        x = arn_ldx<TACC>(xj + row);
         for (int q = rs; q < re; q += U) {
           int c[U];
           TACC v[U], xv[U];
@@ -828,7 +850,7 @@ __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj
             v[u] = q + u < re ? __ldg(a.val + q + u) : (TACC)0;
           }
 #pragma unroll
-          for (int u = 0; u < U; ++u) xv[u] = q + u < re ? ld_as<TACC, TV>(xj + c[u]) : (TACC)0;
+          for (int u = 0; u < U; ++u) xv[u] = q + u < re ? arn_ldx<TACC>(xj + c[u]) : (TACC)0;
 #pragma unroll
           for (int u = 0; u < U; ++u)
             if (q + u < re) acc += v[u] * xv[u];
@@ -865,7 +887,7 @@ __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj
       for (int h = 0; h < 2; ++h) {
         TACC xv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = c[h][u] >= 0 ? ld_as<TACC, TV>(xj + c[h][u]) : (TACC)0;
+        for (int u = 0; u < U; ++u) xv[u] = c[h][u] >= 0 ? arn_ldx<TACC>(xj + c[h][u]) : (TACC)0;
 #pragma unroll
         for (int u = 0; u < U; ++u)
           if (c[h][u] >= 0) acc[h] += v[h][u] * xv[u];
@@ -878,7 +900,7 @@ __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj
       for (int o = L / 2; o > 0; o >>= 1) acc[h] += __shfl_xor_sync(0xffffffffu, acc[h], o);
     if (sub < 2) {
       Ws[r0 + sub - s0] = sub ? acc[1] : acc[0];
-      Us[r0 + sub - s0] = r0 + sub < N ? ld_as<TACC, TV>(xj + r0 + sub) : (TACC)0;
+      Us[r0 + sub - s0] = r0 + sub < N ? arn_ldx<TACC>(xj + r0 + sub) : (TACC)0;
     }
   }
 }
@@ -888,7 +910,9 @@ __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj
 template <int ND, typename TV, typename TACC>
 __device__ __forceinline__ void arn_diag(const ArnArgs<TV, TACC>& a, int j, long long s0,
                                          long long s1, TACC* Ws, TACC* Us, int tid, int nthr) {
-  constexpr int B = sizeof(TACC) == 8 ? 2 : 4;  // SpMV rows per thread and batch
+  // SpMV rows per thread and batch (4 in FP32 and BF16 spill 12 to 72 bytes: 361k rows BF16 76.0 ms
+  // against 71.4, 1M rows FP32 93.9 against 93.3)
+  constexpr int B = sizeof(TACC) == 8 ? 2 : 3;
   const long long N = a.N;
   const TV* xj = a.V + (size_t)j * a.ldv;
   if constexpr (ND == kArnCsr) {
@@ -904,7 +928,7 @@ __device__ __forceinline__ void arn_diag(const ArnArgs<TV, TACC>& a, int j, long
       const long long row = i0 + (long long)b * nthr;
       if (row < s1) {
         Ws[row - s0] = row < N ? v[b] : (TACC)0;
-        Us[row - s0] = row < N ? ld_as<TACC, TV>(xj + row) : (TACC)0;
+        Us[row - s0] = row < N ? arn_ldx<TACC>(xj + row) : (TACC)0;
       }
     }
   }
