@@ -63,6 +63,8 @@ cudaError_t launch_au_planes(int n, const int* aurp, const int* aucol, const dou
 cudaError_t launch_dia_detect(int n, const int* rowptr, const int* col, int* slots, int* count,
                               cudaStream_t st);
 int dia_empty_slot();
+cudaError_t launch_col_spread(int n, const int* rowptr, const int* col, unsigned long long* out,
+                              cudaStream_t st);
 cudaError_t launch_dia_fill(int n, const int* rowptr, const int* col, const double* val,
                             const DiaOffsets& offs, long long ldd, double* dval, float* dval32,
                             cudaStream_t st);
@@ -94,6 +96,7 @@ struct OpDev {           // one operator (A or A^T) as the kernels see it
   // lanes per row of the CSR SpMV (0: a thread per row); set for long rows
   int vec;
   int au_tile_max;       // most A W entries in a tile of 256 rows
+  int scattered;         // CSR: columns far from their rows (OpHost)
 };
 
 struct CycleArgs {

@@ -946,6 +946,18 @@ __global__ void k_dia_fill(int n, const int* __restrict__ rowptr, const int* __r
   }
 }
 
+// Sums of |col - row| and of entries over kSpreadRows rows, evenly spaced
+constexpr int kSpreadRows = 4096;
+__global__ void k_col_spread(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
+                             unsigned long long* __restrict__ out) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)((long long)s * n / kSpreadRows);
+  unsigned long long dist = 0;
+  for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) dist += (unsigned)abs(col[k] - i);
+  atomicAdd(&out[0], dist);
+  atomicAdd(&out[1], (unsigned long long)(rowptr[i + 1] - rowptr[i]));
+}
+
 }  // namespace
 
 cudaError_t launch_validate(int n, long long nnz, const int* rowptr, const int* col,
@@ -1523,6 +1535,14 @@ cudaError_t launch_dia_detect(int n, const int* rowptr, const int* col, int* slo
 }
 
 int dia_empty_slot() { return kDiagEmpty; }
+
+cudaError_t launch_col_spread(int n, const int* rowptr, const int* col, unsigned long long* out,
+                              cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(*out), st);
+  if (e != cudaSuccess) return e;
+  k_col_spread<<<kSpreadRows / 256, 256, 0, st>>>(n, rowptr, col, out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_dia_fill(int n, const int* rowptr, const int* col, const double* val,
                             const DiaOffsets& offs, long long ldd, double* dval, float* dval32,

@@ -582,7 +582,8 @@ gmres_status gmres_create(gmres_t* out, const gmres_csr* A, const gmres_defl* W,
     if (s_au != GMRES_OK) return bail(s_au);
   }
   {
-    const gmres_status s_dia = build_dia(h, h->fwd);
+    gmres_status s_dia = build_dia(h, h->fwd);
+    if (s_dia == GMRES_OK) s_dia = build_spread(h, h->fwd);
     if (s_dia != GMRES_OK) return bail(s_dia);
   }
   if (opts.mu_mode == GMRES_MU_NORM_INF) {
@@ -654,7 +655,8 @@ gmres_status gmres_adjoint_solve(gmres_t h, const double* g, const double* lam0,
       const gmres_status s_au = build_au(h, h->adj);
       if (s_au != GMRES_OK) return s_au;
     }
-    const gmres_status s_dia = build_dia(h, h->adj);
+    gmres_status s_dia = build_dia(h, h->adj);
+    if (s_dia == GMRES_OK) s_dia = build_spread(h, h->adj);
     if (s_dia != GMRES_OK) return s_dia;
     h->adj.ready = true;
   }
