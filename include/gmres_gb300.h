@@ -271,7 +271,8 @@ gmres_status gmres_batch_solve(int32_t count, gmres_t const* hs, const double* c
 
 /* Per-phase device time (ms, from CUDA events on the handle stream while profiling is on;
  * the setup entry is host wall time) and kernel launch counts (always counted) summed
- * since the last reset.  ms and launches (host, GMRES_PH_COUNT entries each) may be NULL.
+ * since the last reset.  A batched solve adds, under GMRES_PH_ARNOLDI, each system's cycles that
+ * ran in a thread-block cluster.  ms and launches (host, GMRES_PH_COUNT entries each) may be NULL.
  * reset != 0 zeroes the sums after reading them.  enable: 1 on, 0 off, -1 unchanged.
  * Host-only; never blocks. */
 gmres_status gmres_profile(gmres_t h, int32_t enable, int32_t reset, double* ms,

@@ -4,8 +4,8 @@
 // per running system: the two or three barriers of a step are then cluster barriers among a few
 // blocks, systems do not wait for each other inside a cycle, and the step's launches (six to
 // eight, over all systems) are gone.  Batches it does not cover (a system of more than kClusterRows
-// rows, operators of different forms, an option without a fused step) run the steps as phase
-// kernels.  The rest of a cycle (x update, corrections, residual, restart decision) is phase
+// rows, operators of different forms, an option without a fused step, sizes that would leave most
+// of the device waiting for a few clusters) run the steps as phase kernels.  The rest of a cycle (x update, corrections, residual, restart decision) is phase
 // kernels in either case.
 //
 // A phase kernel runs over a flattened list of row tiles drawn from all systems, so each launch
@@ -21,6 +21,7 @@
 // once into the body of a conditional `while` graph node, and a last kernel sets the loop
 // condition (any system still running), so the whole solve is one graph launch.
 #include <algorithm>
+#include <functional>
 #include <map>
 #include <memory>
 
@@ -949,6 +950,52 @@ cudaError_t build_tables(BatchCtx& c, cudaStream_t st) {
   return cudaStreamSynchronize(st);
 }
 
+// Whether clusters beat the phase kernels for the systems of a batch, with clusters of G blocks, fit
+// of them at once.  A cluster's step costs rows / G times the per-row time of one multiprocessor, and
+// the clusters wait for the largest system or the last wave; a phase spreads all rows over the whole
+// device but adds its launches.  In units of the latter's time per row:
+//   clusters  f (d R + (1 - d) T / SMs)    R: most rows a block steps through, T: all rows
+//   phases    T + c
+// f: how many times the whole device's time per row one multiprocessor takes, all of them busy; d:
+// the share of it that does not shrink when few are; c: launches less barriers.  Measured (80
+// steps of GMRES(40), 6 to 160 equal systems of 4,096 to 74,088 rows, us a step, clusters / phases):
+//   FP64 CGS2, 9 diagonals      6 of 74k 119 / 184, 16 of 74k 393 / 396, 36 of 74k 473 / 810
+//   CSR, tile by tile, 9 a row  16 of 36k 236 / 223, 16 of 74k 500 / 399, 36 of 74k 570 / 817
+//   CSR at random, 9 a row      16 of 74k 686 / 414, 80 of 36k 1195 / 918, 36 of 74k 752 / 864
+//   27 a row, by tiles          16 of 36k 430 / 290, 36 of 36k 469 / 587
+//   27 a row, at random         6 of 36k 179 / 157, 16 of 74k 1269 / 567, 36 of 36k 617 / 621
+//   BF16, 27 a row, at random   16 of 74k 1330 / 962, 36 of 74k 1507 / 1743; 9 diagonals 128 / 551
+// 28 systems of 4k to 74k rows on diagonals, FP64 CGS2: 43.6 ms in clusters, 36.0 as phases.
+bool clusters_pay(const BatchCtx& c, int G, int fit) {
+  bool csr = false, vec = false, scattered = false;
+  std::vector<long long> rows, slot(fit, 0);
+  long long T = 0;
+  for (gmres_s* h : c.hs) {
+    const OpDev op = make_op(h, h->fwd);
+    csr |= op.dia.nd == 0;
+    vec |= op.vec != 0;
+    scattered |= op.scattered != 0;
+    rows.push_back(h->ldv);
+    T += h->ldv;
+  }
+  // largest first, each to the cluster that is free first
+  std::sort(rows.begin(), rows.end(), std::greater<long long>());
+  for (long long r : rows) {
+    std::pop_heap(slot.begin(), slot.end(), std::greater<long long>());
+    slot.back() += r;
+    std::push_heap(slot.begin(), slot.end(), std::greater<long long>());
+  }
+  const double R = (double)*std::max_element(slot.begin(), slot.end()) / G;
+  const int form = !csr ? 0 : 1 + (vec ? 1 : 0) + (scattered ? 2 : 0);
+  static const double kF[3][5] = {{88, 106, 132, 132, 172},   // FP64 CGS2: diagonals; CSR by tiles,
+                                  {70, 94, 130, 124, 166},    // long rows by tiles, at random,
+                                  {58, 62, 90, 90, 150}};     // long rows; FP64 one reduction; 32 bits
+  const double f = kF[c.prec != P_FP64 ? 2 : c.ortho == GMRES_ORTHO_CGS2 ? 0 : 1][form];
+  const double d = !csr ? 0.8 : vec ? 1.0 : 0.9;
+  const double launches = c.prec == P_FP64 ? 165000.0 : 500000.0;
+  return f * (d * R + (1.0 - d) * (double)T / c.hs[0]->sms) < (double)T + launches;
+}
+
 // Whether the systems of the batch can run their cycles in clusters (fused.cuh), and in which
 // sizes.  While many systems run, clusters of 2 or 4 blocks (the most systems at once, the least
 // waiting inside a system); when the running systems fit the device in clusters of 8, and of 16,
@@ -974,6 +1021,7 @@ FusedBatch plan_fused(const BatchCtx& c) {
     if (!same || h->ldv > kClusterRows || !arnoldi_fusable(a)) return none;
   }
   const int sizes[kBatchTiers] = {2, 4, 8, 16};
+  int G = 0, at_once = 0;  // the clusters that the whole batch starts with
   for (int t = 0; t < kBatchTiers; ++t) {
     int fit = 0;
     f.fit = &fit;
@@ -984,8 +1032,12 @@ FusedBatch plan_fused(const BatchCtx& c) {
     if (e != cudaSuccess || fit < 1) break;
     f.G[f.tiers] = sizes[t];
     f.upto[f.tiers++] = sizes[t] == 4 ? kClusterWaves * fit : fit;
+    if (t == 0 || c.count <= f.upto[f.tiers - 1]) {
+      G = sizes[t];
+      at_once = fit;
+    }
   }
-  return f;
+  return f.tiers && clusters_pay(c, G, at_once) ? f : none;
 }
 
 // the kernel arguments of every system's cycles, largest first, to the device
@@ -1237,6 +1289,7 @@ gmres_status batch_solve_impl(int count, gmres_t const* hs, const double* const*
     if ((e = cudaMemcpy(&hm, hs[i]->meta.p, sizeof(Meta), cudaMemcpyDeviceToHost)) != cudaSuccess)
       return cuda_fail(nullptr, e, "batch status");
     const gmres_status si = (gmres_status)hm.flags[F_STATUS];
+    if (ctx->fb.tiers) hs[i]->plaunch[PH_ARNOLDI] += hm.counts[C_CYCLES];
     if (infos) {
       infos[i].iters = hm.counts[C_STEPS];
       infos[i].cycles = hm.counts[C_CYCLES];

@@ -55,7 +55,7 @@ struct OpHost {
   int au_tile_max = 0;                 // most A W entries in a tile of 256 rows
   DiaOffsets dia{};
   long long ldd = 0;
-  bool scattered = false;  // no diagonals, and mean |col - row| above n / 16 (see build_spread)
+  bool scattered = false;  // mean |col - row| above n / 16
   bool ready = false;
 };
 
@@ -226,18 +226,25 @@ inline Ctl make_ctl(gmres_s* h) {
 
 // Diagonal storage of operator o when it has at most kMaxDiag distinct diagonals and they
 // are at least 80 % filled (the Q1 stencils: 9 diagonals, 99.6 % filled); otherwise the
-// CSR kernels are used.
+// CSR kernels are used.  Also whether the gathers scatter over the whole vector: mean |col - row| is
+// n / 3 in a random numbering, a few percent of n in a lexicographic, banded or tile-by-tile one.
 inline gmres_status build_dia(gmres_s* h, OpHost& o) {
   cudaStream_t st = h->stream;
   const int n = h->n;
   o.dia.nd = 0;
   DevMem slots;
-  CK(h, slots.ensure(sizeof(int) * 65));
+  // the diagonals' slots, their count, then the sums of k_col_spread (8-byte aligned)
+  CK(h, slots.ensure(sizeof(int) * 70));
   int* sl = slots.as<int>();
   CK(h, launch_dia_detect(n, o.rowptr.as<int>(), o.col.as<int>(), sl, sl + 64, st));
-  int hs[65];
+  CK(h, launch_col_spread(n, o.rowptr.as<int>(), o.col.as<int>(),
+                          reinterpret_cast<unsigned long long*>(sl + 66), st));
+  int hs[70];
   CK(h, cudaMemcpyAsync(hs, sl, sizeof(hs), cudaMemcpyDeviceToHost, st));
   CK(h, cudaStreamSynchronize(st));
+  unsigned long long spread[2];
+  std::memcpy(spread, hs + 66, sizeof(spread));
+  o.scattered = 16.0 * (double)spread[0] > (double)spread[1] * (double)n;
   if (hs[64] > kMaxDiag || hs[64] < 1) return GMRES_OK;
   DiaOffsets offs{};
   for (int i = 0; i < 64; ++i)
@@ -259,24 +266,6 @@ inline gmres_status build_dia(gmres_s* h, OpHost& o) {
   CK(h, cudaStreamSynchronize(st));
   o.dia = offs;
   o.ldd = ldd;
-  return GMRES_OK;
-}
-
-// Whether the gathers of a CSR operator scatter over the whole vector: mean |col - row| is n / 3 in
-// a random numbering, below 2 % of n from 190,000 rows on in a lexicographic, banded or
-// tile-by-tile one.  Asked only of systems large enough for fused_rows to depend on it.
-constexpr int kSpreadMinRows = 150000;
-inline gmres_status build_spread(gmres_s* h, OpHost& o) {
-  o.scattered = false;
-  if (o.dia.nd > 0 || h->n < kSpreadMinRows) return GMRES_OK;
-  DevMem sums;
-  CK(h, sums.ensure(2 * sizeof(unsigned long long)));
-  unsigned long long hv[2] = {0, 0};
-  CK(h, launch_col_spread(h->n, o.rowptr.as<int>(), o.col.as<int>(),
-                          sums.as<unsigned long long>(), h->stream));
-  CK(h, cudaMemcpyAsync(hv, sums.p, sizeof(hv), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
-  o.scattered = 16.0 * (double)hv[0] > (double)hv[1] * (double)h->n;
   return GMRES_OK;
 }
 

@@ -96,7 +96,7 @@ struct OpDev {           // one operator (A or A^T) as the kernels see it
   // lanes per row of the CSR SpMV (0: a thread per row); set for long rows
   int vec;
   int au_tile_max;       // most A W entries in a tile of 256 rows
-  int scattered;         // CSR: columns far from their rows (OpHost)
+  int scattered;         // columns far from their rows (OpHost)
 };
 
 struct CycleArgs {

@@ -582,8 +582,7 @@ gmres_status gmres_create(gmres_t* out, const gmres_csr* A, const gmres_defl* W,
     if (s_au != GMRES_OK) return bail(s_au);
   }
   {
-    gmres_status s_dia = build_dia(h, h->fwd);
-    if (s_dia == GMRES_OK) s_dia = build_spread(h, h->fwd);
+    const gmres_status s_dia = build_dia(h, h->fwd);
     if (s_dia != GMRES_OK) return bail(s_dia);
   }
   if (opts.mu_mode == GMRES_MU_NORM_INF) {
@@ -655,8 +654,7 @@ gmres_status gmres_adjoint_solve(gmres_t h, const double* g, const double* lam0,
       const gmres_status s_au = build_au(h, h->adj);
       if (s_au != GMRES_OK) return s_au;
     }
-    gmres_status s_dia = build_dia(h, h->adj);
-    if (s_dia == GMRES_OK) s_dia = build_spread(h, h->adj);
+    const gmres_status s_dia = build_dia(h, h->adj);
     if (s_dia != GMRES_OK) return s_dia;
     h->adj.ready = true;
   }
