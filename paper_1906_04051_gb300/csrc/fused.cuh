@@ -1691,9 +1691,9 @@ template <typename TV, typename TACC, int ND, int MODE, bool CL>
 __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int G, const int bid) {
   static_assert(MODE != kArnLowsyncDf || sizeof(TV) == 8, "the double-FP32 multi-dot takes an FP64 basis");
   static_assert(MODE == kArnCgs2 || sizeof(TV) == sizeof(TACC), "BF16 bases use CGS2");
-  // the FP32 one-reduction step of a banded operator runs its coarse solve in FP32, every
+  // the FP32 one-reduction step of a banded operator in a grid runs its coarse solve in FP32, every
   // other instantiation in FP64
-  constexpr bool C32 = sizeof(TV) == 4 && MODE == kArnLowsync && ND != kArnCsr;
+  constexpr bool C32 = sizeof(TV) == 4 && MODE == kArnLowsync && ND != kArnCsr && !CL;
   constexpr int NSET = MODE == kArnCgs2 ? 1 : 2;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double tot[2 * kMaxK + 1];
