@@ -138,16 +138,21 @@ typedef enum {
 } gmres_ortho;
 
 typedef enum {
-  GMRES_DOT_FP64 = 0,  /* the basis multi-dot to FP64 accuracy (in the fused step as exact
-                          integer sums of fixed-point operands, the basis to 61 bits of its
-                          column's largest entry, w to 54 bits of its largest in a block's
-                          rows; in FP64 FMAs elsewhere) */
+  GMRES_DOT_FP64 = 0,  /* the basis multi-dot to FP64 accuracy: in FP64 FMAs, or (fused cycles)
+                          as exact integer sums of fixed-point operands, w cut to 54 bits of
+                          its largest entry in a block's rows.  The fused FP64 cycles hold the
+                          basis in 64-bit fixed point, and basis updates and x are formed from
+                          it, a row's sum in integers and rounded once: an entry is kept to
+                          61 bits of its column's largest, or, in a row that stays more than
+                          2^8 below, to at least 53 bits of the row's largest (entries in
+                          units of their columns' largest), so that a row's errors are
+                          relative to its own entries, as in FP64 */
   GMRES_DOT_DF32 = 1   /* the multi-dot V^T [w, v_j] of the one-reduction MGS step in
                           double-FP32 on the FP32 pipe: each FP64 operand split into two
                           floats (47 significant bits), products exact by FMA (Dekker's
                           two-product), sums by Knuth's TwoSum, each block's totals rounded
                           to FP64 once; magnitudes below 2^-126 count as 0.  The rest of the
-                          step (SpMV, update, norm, H, rotations) stays FP64.  FP64 solves
+                          step (SpMV, update, norm, H, rotations) keeps FP64 accuracy.  FP64 solves
                           with GMRES_ORTHO_MGS_LOWSYNC only (GMRES_ERR_INVALID_ARG
                           otherwise); applied where the step runs fused (a diagonal-structured
                           A, aggregate or no deflation), FP64 FMAs elsewhere */

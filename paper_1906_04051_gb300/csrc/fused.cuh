@@ -32,7 +32,8 @@
 // rows, w' in shared memory in between), one more grid barrier, and coefficients h + h'.
 // Every reduction is formed in a fixed order: runs are bitwise reproducible.  The per-phase
 // register budgets (loads in flight) are set so that no loop needs local memory: with 220 KB
-// of shared memory per block, spilled registers would live in L2.
+// of shared memory per block, spilled registers would live in L2 (the FP64 one-reduction step with a
+// run-time number of diagonals keeps 4 bytes there, 16 in clusters; the others none).
 //
 // The batched form (k_arnoldi_batch) runs the same cycle for one system per thread-block
 // cluster, whose hardware barrier takes the place of the grid barriers.
@@ -58,8 +59,10 @@ constexpr int kArnWarps = 16;
 constexpr int kArnThreads = kArnWarps * 32;
 constexpr int kArnUnit = kPartUnit;              // rows per unit of the row partition
 constexpr size_t kArnSmem = 220 * 1024;          // dynamic shared memory
-// reductions: lane-wise totals [2][kMaxK][33] (FP64) or warp sums [2][16][kMaxK] (FP32)
+// reductions: per set of dots, warp and column an int4 (fixed point) or a pair of floats; the
+// updates' coefficients and shared partial sums (arn_sk)
 constexpr size_t kArnScratch = 2 * kMaxK * 33 * sizeof(double);
+static_assert(kArnScratch >= 2 * kArnWarps * kMaxK * sizeof(int4), "two sets of slots");
 constexpr long long kArnSpins = 1LL << 21;       // polls of the barrier word: about a second
 constexpr int kArnNormCol = 2 * kMaxK;           // column of ctl.part holding the norm partials
 constexpr int kArnMaxCol = kArnNormCol + 1;      // and the blocks' largest |u_{j+1}| (high words)
@@ -96,7 +99,7 @@ struct ArnArgs {
   const int* rowptr;  // CSR (no diagonal storage)
   const int* col;
   const TACC* val;
-  int vec;            // CSR: long rows, 4 lanes each
+  int vec;            // CSR: long rows, 8 lanes each (arn_csr)
   const int* aurp;
   const int* aucol;
   const TACC* auval;
@@ -1514,15 +1517,17 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, const A
       finish();
     }
   }
-  if constexpr (PASS2) return 0.0;
-  // the warp's total in double-FP32, rounded once
+  if constexpr (PASS2) {
+    return 0.0;
+  } else {  // the warp's total in double-FP32, rounded once
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float a2 = __shfl_xor_sync(0xffffffffu, ns, o);
-    const float b2 = __shfl_xor_sync(0xffffffffu, nc, o);
-    arn_df_add(ns, nc, a2, b2);
+    for (int o = 16; o > 0; o >>= 1) {
+      const float a2 = __shfl_xor_sync(0xffffffffu, ns, o);
+      const float b2 = __shfl_xor_sync(0xffffffffu, nc, o);
+      arn_df_add(ns, nc, a2, b2);
+    }
+    return (double)ns + (double)nc;
   }
-  return (double)ns + (double)nc;
 }
 
 // CGS2, first update and second multi-dot of an FP32 or BF16 basis: per super-tile (from the last)
@@ -1530,7 +1535,7 @@ __device__ __forceinline__ double arn_update(const ArnArgs<TV, TACC>& a, const A
 template <typename TV, typename TACC, int ND>
 __device__ __forceinline__ void arn_pass2_rows(const ArnArgs<TV, TACC>& a, const ArnRows& g, int k, TACC* Ws,
                                             const TACC* scoef, double* sbuf) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
   const long long R0 = g.R0, R1 = g.R1;
   const int tiles = (int)((R1 - R0 + a.RS - 1) / a.RS);
   for (int tile = tiles - 1; tile >= 0; --tile) {
@@ -1714,7 +1719,7 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
   const ArnRows g = arn_rows(a, G, bid);
   const long long R0 = g.R0, R1 = g.R1;
   // shared memory: w and u_j of a super-tile, s' (r), reduction scratch, the rows of L
-  // (stride kMaxK), the FP64 multi-dot staging
+  // (stride kMaxK)
   TACC* Ws = reinterpret_cast<TACC*>(smem);
   TACC* Us = Ws + a.RS;
   TACC* Ss = Us + a.RS;
@@ -1838,11 +1843,10 @@ __device__ __forceinline__ void arn_cycle(const ArnArgs<TV, TACC>& a, const int 
   for (int j = 0; j < a.jmax; ++j) {
     const int k = j + 1;
     const TACC sig = (TACC)ssig[j];
-    // partial sums of the multi-dot in shared memory, so that they persist across
-    // super-tiles (FP64: lane-wise per column; FP32: per warp and column; double-FP32:
-    // pairs per warp and column)
+    // the pairs per warp and column of an FP32, BF16 or double-FP32 multi-dot, which add up over
+    // the super-tiles (fixed point stores its slots anew in each)
     if constexpr (sizeof(TV) < 8 || MODE == kArnLowsyncDf)
-      for (int q = t; q < 2 * kMaxK * 33; q += kArnThreads) sbuf[q] = 0.0;
+      for (int q = t; q < (int)(kArnScratch / sizeof(double)); q += kArnThreads) sbuf[q] = 0.0;
     arn_front<TV, TACC, ND, MODE>(a, g, j, sig, waited, j > 0, Ws, Us, Ss, sbuf, sE, semax, sred);
     waited = true;
     // per-block column sums (fixed order; a fixed-point multi-dot leaves them in sred)
