@@ -108,6 +108,8 @@ gmres_status run(gmres_s* h, OpHost& o, const double* b, const double* x0, int m
   // the whole cycle in one persistent kernel where it applies (fused.cuh): not over a dense
   // deflation space, but those solves' cycles before they have one
   const bool fusable = !mgs && arnoldi_fusable(a);
+  // (the double-FP32 option is for solves with aggregates or no deflation)
+  if (ada || dw) a.dot_arith = GMRES_DOT_FP64;
   if (fusable) CK(h, cudaMemsetAsync(h->gbar.p, 0, 4 * sizeof(unsigned), st));
   const int mu_mode = h->opts.mu_mode;
   double mu = 0.0;

@@ -220,3 +220,25 @@ def test_small_uncoupled_block_keeps_its_digits(G, orc, how, rhs, q):
     y[perm] = x.cpu().numpy()
     assert np.linalg.norm(y[:n]) > 0
     assert relerr(3.0 * np.ldexp(y[n:], q), y[:n]) <= bound
+
+
+# GMRES_DOT_DF32 is for solves with aggregates or without deflation: the undeflated cycles of an
+# adaptive or a dense-W solve keep FP64 accuracy, also where floats would underflow
+@pytest.mark.parametrize("dense", [False, True])
+def test_double_float_dots_not_with_a_dense_space(G, orc, dense):
+    p = W.convdiff(40, pe=25.0, sigma=0.5, seed=140, px=1, py=1)
+    A, b = orc.q1_assemble(p.n, p.kappa, p.beta, p.f)
+    kw = dict(rmax=20, ortho=2) if not dense else dict(ortho=2)
+    xs = []
+    for q, arith in ((-140, G.DOT_DF32), (0, G.DOT_FP64)):
+        if dense:
+            w = np.linalg.qr(np.random.default_rng(2).standard_normal((A.n, 3)))[0]
+            s = G.Solver(to_dev(A.rowptr), to_dev(A.col), to_dev(A.val), w_dense=to_dev(w),
+                         fixed_iterations=True, dot_arith=arith, **kw)
+        else:
+            s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_ADAPTIVE, fixed_iterations=True,
+                                       mu_mode=1, mu_user=5.0, dot_arith=arith, **kw)
+        x, info = s.solve(to_dev(np.ldexp(b, q)), m=15, tol=0.0, maxit=40)
+        assert info["iters"] == 40
+        xs.append(np.ldexp(x.cpu().numpy(), -q))
+    assert np.array_equal(xs[0], xs[1])
