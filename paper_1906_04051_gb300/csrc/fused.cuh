@@ -485,8 +485,8 @@ __device__ __forceinline__ void arn_ldfx(const long long* p, uint4& o) {
 // reductions and lane 0 stores them in slot[set][first chunk][c] (once per super-tile).
 // Bound by the loads; per element 6 IMAD.WIDE and a few simple integer operations, where 2 FP64
 // multiply-adds hold their pipe for 64 issue slots each (q1-n1024, GMRES(50), a step of the whole
-// kernel: 228 us with FP64 multiply-adds in dots and update, 151 us in fixed point; 4.2M rows,
-// GMRES(40): 690 to 450 us).
+// kernel: 228 us with FP64 multiply-adds in dots and update, 152 us in fixed point; 4M rows without
+// deflation, 45 columns: 743 us as FP64 phases, 453 us).
 template <int NSET, int G, int D>
 __device__ __forceinline__ void arn_dots_fx(int4* slot, const double* V, long long ldv, int kf,
                                             int k, int ej, long long s0, int nch, const int4* Wf,
