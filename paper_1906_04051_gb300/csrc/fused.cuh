@@ -853,7 +853,9 @@ __device__ __forceinline__ void arn_csr(const ArnArgs<TV, TACC>& a, const TV* xj
             v[u] = q + u < re ? __ldg(a.val + q + u) : (TACC)0;
           }
 #pragma unroll
-          for (int u = 0; u < U; ++u) xv[u] = q + u < re ? arn_ldx<TACC>(xj + c[u]) : (TACC)0;
+          for (int u = 0; u < U; ++u)  // (16-bit gathers under a predicate wait for one another: a row
+                                       // of 100,000 BF16 entries 8.3 ms, 6.2 without; column 0 then)
+            xv[u] = sizeof(TV) == 2 || q + u < re ? arn_ldx<TACC>(xj + c[u]) : (TACC)0;
 #pragma unroll
           for (int u = 0; u < U; ++u)
             if (q + u < re) acc += v[u] * xv[u];
