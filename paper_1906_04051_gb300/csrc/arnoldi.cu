@@ -993,11 +993,13 @@ __global__ void __launch_bounds__(kSpmvRows)
 // relative to ||H||).
 // QR is a chain of some 10^5 dependent FP64 operations (4.2 ms at k = 50); squaring shares the
 // rows of each square over a cluster of 8 blocks, every block keeping the whole matrix in shared
-// memory (0.41 ms at k = 50).
+// memory (0.41 ms at k = 50), at some 75 us for the 56 barriers of any k: up to kRitzSmall QR is the
+// faster one (us, squaring / QR: 74 / 6 at k = 1, 94 / 82 at 6, 96 / 143 at 8).
 // --------------------------------------------------------------------------------------
 constexpr int kRitzCluster = 8;
 constexpr int kRitzThreads = 512;                      // 8 rows x 64 columns
 constexpr int kRitzSquarings = 56;
+constexpr int kRitzSmall = 6;
 constexpr double kRitzGrowth = 3.0;                    // largest g_i the squares are trusted with
 constexpr size_t kRitzSmem = 2 * kMaxM * kMaxM * sizeof(double);
 
@@ -1014,6 +1016,10 @@ __global__ void __cluster_dims__(kRitzCluster, 1, 1) __launch_bounds__(kRitzThre
   const int n = ctl.flags[F_K];
   if (n <= 0) return;
   const int t = threadIdx.x, rank = (int)cl.block_rank(), ldh = ctl.ldh;
+  if (n <= kRitzSmall) {
+    if (rank == 0 && t < 32) ritz_warp(ctl, sN, smod, sfail);
+    return;
+  }
   // the Hessenberg block as built; entries below the subdiagonal are never written, so they
   // are taken as the zeros they are (not read from memory)
   for (int q = t; q < kMaxM * kMaxM; q += kRitzThreads) {
