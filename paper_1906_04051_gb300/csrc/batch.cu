@@ -1011,7 +1011,7 @@ FusedBatch plan_fused(const BatchCtx& c) {
     CycleArgs a{};
     a.op = make_op(h, h->fwd);
     a.ldv = h->ldv;
-    a.m = c.m;
+    a.m = std::max(c.m, 2);  // (GMRES(1) as well: a cluster's barriers are cheap)
     a.prec = c.prec;
     a.ortho = c.ortho;
     a.sms = h->sms;

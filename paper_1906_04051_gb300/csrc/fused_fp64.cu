@@ -53,8 +53,12 @@ long long fused_rows(const CycleArgs& a) {
 // deflation space); BF16 bases with CGS2.
 bool arnoldi_fusable(const CycleArgs& a) {
   if (a.ldv > fused_rows(a)) return false;
+  // GMRES(1) in FP64: the exponent of u_0 costs a grid barrier and a pass over it in every cycle (10
+  // cycles, us, fused / phases: 10,000 rows CGS2 883 / 849, CSR 879 / 814; GMRES(2) 652 / 665)
+  const bool dia = a.op.dia.nd > 0, cgs2 = a.ortho == GMRES_ORTHO_CGS2;
+  if (a.m < 2 && a.prec == P_FP64 && (cgs2 || !dia)) return false;
   if (a.proj || a.op.defl.qd != 0 || a.ldv % kArnUnit != 0 || a.m + 1 > kMaxK) return false;
-  if (a.ortho != GMRES_ORTHO_CGS2 && !(a.ortho == GMRES_ORTHO_MGS_LOWSYNC && a.prec != P_BF16))
+  if (!cgs2 && !(a.ortho == GMRES_ORTHO_MGS_LOWSYNC && a.prec != P_BF16))
     return false;
   const int r = a.op.defl.r;
   // with deflation: the pieces split at this kernel's block rows (built at setup for a

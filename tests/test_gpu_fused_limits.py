@@ -58,3 +58,23 @@ def test_both_sides_of_the_lines(orc, n, order, ortho, prec, fused):
     xo, _ = orc.gmres(A, b, m=6, tol=0.0, maxit=6, fixed_iterations=True,
                       **({"ortho": orc.MGS} if ortho else {}))
     assert relerr(xg.cpu().numpy(), xo) <= (1e-9 if prec == 0 else 1e-4)
+
+
+# GMRES(1) in FP64 with CGS2 runs its cycles as phases, in a batch in clusters; GMRES(2) fused
+@pytest.mark.parametrize("m", [1, 2])
+def test_shortest_restarts(orc, m):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1906_04051_gb300 as G
+    from paper_1906_04051_gb300 import build as B
+    B.build()
+    A, b = _stencil27(orc, 12, None)
+    s = gpu_solver_from_oracle(G, A, deflation_mode=G.DEFL_NONE, fixed_iterations=True)
+    xo, _ = orc.gmres(A, b, m=m, tol=0.0, maxit=8, fixed_iterations=True)
+    xg, ig = s.solve(to_dev(b), m=m, tol=0.0, maxit=8)
+    assert ig["iters"] == 8 and (s.profile()["arnoldi"][1] > 0) == (m > 1)
+    assert relerr(xg.cpu().numpy(), xo) <= 1e-9
+    s.profile(reset=True)
+    xs, infos, _ = G.batch_solve([s], [to_dev(b)], m=m, tol=0.0, maxit=8)
+    assert infos[0]["iters"] == 8 and s.profile()["arnoldi"][1] > 0
+    assert relerr(xs[0].cpu().numpy(), xo) <= 1e-9
