@@ -950,50 +950,68 @@ cudaError_t build_tables(BatchCtx& c, cudaStream_t st) {
   return cudaStreamSynchronize(st);
 }
 
-// Whether clusters beat the phase kernels for the systems of a batch, with clusters of G blocks, fit
-// of them at once.  A cluster's step costs rows / G times the per-row time of one multiprocessor, and
-// the clusters wait for the largest system or the last wave; a phase spreads all rows over the whole
-// device but adds its launches.  In units of the latter's time per row:
-//   clusters  f (d R + (1 - d) T / SMs)    R: most rows a block steps through, T: all rows
-//   phases    T + c
-// f: how many times the whole device's time per row one multiprocessor takes, all of them busy; d:
-// the share of it that does not shrink when few are; c: launches less barriers.  Measured (80
-// steps of GMRES(40), 6 to 160 equal systems of 4,096 to 74,088 rows, us a step, clusters / phases):
-//   FP64 CGS2, 9 diagonals      6 of 74k 119 / 184, 16 of 74k 393 / 396, 36 of 74k 473 / 810
-//   CSR, tile by tile, 9 a row  16 of 36k 236 / 223, 16 of 74k 500 / 399, 36 of 74k 570 / 817
-//   CSR at random, 9 a row      16 of 74k 686 / 414, 80 of 36k 1195 / 918, 36 of 74k 752 / 864
-//   27 a row, by tiles          16 of 36k 430 / 290, 36 of 36k 469 / 587
-//   27 a row, at random         6 of 36k 179 / 157, 16 of 74k 1269 / 567, 36 of 36k 617 / 621
-//   BF16, 27 a row, at random   16 of 74k 1330 / 962, 36 of 74k 1507 / 1743; 9 diagonals 128 / 551
-// 28 systems of 4k to 74k rows on diagonals, FP64 CGS2: 43.6 ms in clusters, 36.0 as phases.
+// Whether clusters of G blocks, `fit` of them at once, beat the phase kernels for a batch: the time of
+// a step by either path, in microseconds.  Clusters wait for the largest system, or the last wave:
+// every system takes t0 for the barriers and sums of its step and its rows on G multiprocessors,
+// one system after another in each place, largest first.  A phase takes its launches (p0) and all
+// rows on the whole device.  A row's time is the SpMV's, linear in the entries per row (z) and by
+// their kind, and the basis', linear in the columns (K on average).  A cycle adds its start (cyc), and
+// as phases the launches of the steps it does not take (idle: a mixed-precision cycle is refined
+// after some `inner` steps).  Least squares over 1,440 batches (1 to 160 equal systems of 400 to
+// 74,088 rows, 9 and 27 entries a row on diagonals, tile by tile and at random, GMRES(4) and
+// GMRES(40)): 7 to 18 % off in the mean; what it picks is within 0.8 % of the better path in the
+// mean.  us a step, clusters / phases:
+//   FP64 CGS2, 9 diagonals   GMRES(40)  6 of 74k 119 / 184, 36 of 74k 473 / 810, 160 of 400 95 / 86
+//                            GMRES(4)   40 of 400 64 / 46, 80 of 74k 911 / 779
+//   9 a row at random        GMRES(40)  16 of 74k 686 / 414, 36 of 74k 752 / 864
+//   27 a row by tiles, BF16  GMRES(4)   16 of 74k 729 / 417, 160 of 16k 986 / 791
+// The rule of fixed sizes before it took 28 systems of 4k to 74k rows to clusters (FP64 CGS2,
+// diagonals: 43.6 ms, 36.0 as phases).
+struct StepCost {
+  double t0, cyc, b, c, p0, idle, bp;  // b, c, bp: per row and column (c: rows over all of the device)
+  int inner;
+};
 bool clusters_pay(const BatchCtx& c, int G, int fit) {
-  bool csr = false, vec = false, scattered = false;
-  std::vector<long long> rows, slot(fit, 0);
-  long long T = 0;
+  static const StepCost kStep[5] = {
+      {25.6, 34, 0.245e-3, 0.332e-3, 46.4, 0, 8.71e-6, 0},  // FP64 CGS2
+      {18.1, 33, 0.134e-3, 0.183e-3, 41.4, 0, 6.55e-6, 0},  // FP64 one reduction
+      {21.5, 30, 0, 0.376e-3, 45.3, 35, 23.7e-6, 12},       // FP32 CGS2
+      {16.7, 28, 0, 0.310e-3, 41.0, 33, 19.0e-6, 12},       // FP32 one reduction
+      {21.1, 63, 0, 1.93e-3, 54.3, 31, 55.0e-6, 6}};        // BF16
+  // SpMV, ns a row on one multiprocessor: diagonals, CSR with its columns near by, scattered; by precision
+  static const double kCl[3][3][2] = {{{4.5, 0.494}, {1.35, 1.25}, {5.95, 1.47}},
+                                      {{-0.5, 0.418}, {-2.0, 0.817}, {-0.25, 1.217}},
+                                      {{-6.0, 0.896}, {-9.25, 1.49}, {-8.35, 1.98}}};
+  // and ps a row on the whole device: columns near by, scattered
+  static const double kPh[3][2][2] = {
+      {{38.5, 7.67}, {51, 8.4}}, {{-26, 8.3}, {-12.5, 9.0}}, {{-108, 12.1}, {-114, 13.9}}};
+  const int pr = c.prec == P_FP64 ? 0 : c.prec == P_FP32 ? 1 : 2;
+  const StepCost& q =
+      kStep[pr == 2 ? 4 : 2 * pr + (c.ortho == GMRES_ORTHO_CGS2 ? 0 : 1)];
+  const int n = q.inner ? std::min(c.m, q.inner) : c.m;
+  const double K = 0.5 * (n + 1);
+  std::vector<std::pair<double, double>> sys;  // rows, us a row on one multiprocessor
+  double rows = 0.0, phases = q.p0 + q.idle * ((double)c.m / n - 1.0);
   for (gmres_s* h : c.hs) {
     const OpDev op = make_op(h, h->fwd);
-    csr |= op.dia.nd == 0;
-    vec |= op.vec != 0;
-    scattered |= op.scattered != 0;
-    rows.push_back(h->ldv);
-    T += h->ldv;
+    const double z = op.dia.nd > 0 ? op.dia.nd : (double)h->nnz / h->n;
+    const int far = op.dia.nd == 0 && op.scattered, kind = op.dia.nd > 0 ? 0 : 1 + far;
+    const double cl = 1e-3 * std::max(0.3, kCl[pr][kind][0] + kCl[pr][kind][1] * z);
+    const double ph = 1e-6 * std::max(5.0, kPh[pr][far][0] + kPh[pr][far][1] * z);
+    sys.emplace_back((double)h->ldv, cl);
+    rows += (double)h->ldv;
+    phases += (ph + q.bp * K) * (double)h->ldv;
   }
-  // largest first, each to the cluster that is free first
-  std::sort(rows.begin(), rows.end(), std::greater<long long>());
-  for (long long r : rows) {
-    std::pop_heap(slot.begin(), slot.end(), std::greater<long long>());
-    slot.back() += r;
-    std::push_heap(slot.begin(), slot.end(), std::greater<long long>());
+  std::sort(sys.begin(), sys.end(), std::greater<std::pair<double, double>>());
+  std::vector<double> place(fit, 0.0);  // a heap, the place that is free first on top
+  for (const auto& s : sys) {
+    std::pop_heap(place.begin(), place.end(), std::greater<double>());
+    place.back() += q.t0 + (s.second + q.b * K) * s.first / G;
+    std::push_heap(place.begin(), place.end(), std::greater<double>());
   }
-  const double R = (double)*std::max_element(slot.begin(), slot.end()) / G;
-  const int form = !csr ? 0 : 1 + (vec ? 1 : 0) + (scattered ? 2 : 0);
-  static const double kF[3][5] = {{88, 106, 132, 132, 172},   // FP64 CGS2: diagonals; CSR by tiles,
-                                  {70, 94, 130, 124, 166},    // long rows by tiles, at random,
-                                  {58, 62, 90, 90, 150}};     // long rows; FP64 one reduction; 32 bits
-  const double f = kF[c.prec != P_FP64 ? 2 : c.ortho == GMRES_ORTHO_CGS2 ? 0 : 1][form];
-  const double d = !csr ? 0.8 : vec ? 1.0 : 0.9;
-  const double launches = c.prec == P_FP64 ? 165000.0 : 500000.0;
-  return f * (d * R + (1.0 - d) * (double)T / c.hs[0]->sms) < (double)T + launches;
+  const double clusters = *std::max_element(place.begin(), place.end()) + q.cyc / n +
+                          q.c * K * rows / c.hs[0]->sms;
+  return 1.05 * clusters < phases;
 }
 
 // Whether the systems of the batch can run their cycles in clusters (fused.cuh), and in which
@@ -1011,7 +1029,7 @@ FusedBatch plan_fused(const BatchCtx& c) {
     CycleArgs a{};
     a.op = make_op(h, h->fwd);
     a.ldv = h->ldv;
-    a.m = std::max(c.m, 2);  // (GMRES(1) as well: a cluster's barriers are cheap)
+    a.m = c.m;
     a.prec = c.prec;
     a.ortho = c.ortho;
     a.sms = h->sms;

@@ -45,8 +45,9 @@ def test_sums_over_lanes(orc, ortho, prec, kind, batch):
     assert (s.layout()["ndiag"] > 0) == (kind == "dia")
     b = to_dev(np.ones(n))
     if batch:
-        xs, infos, _ = G.batch_solve([s], [b], m=1, tol=0.0, maxit=1)
+        xs, infos, _ = G.batch_solve([s], [b], m=20, tol=0.0, maxit=1)  # (in a cluster)
         x, info = xs[0], infos[0]
+        assert s.profile()["arnoldi"][1] > 0
     else:
         x, info = s.solve(b, m=1, tol=0.0, maxit=1)
     assert info["iters"] == 1
